@@ -31,6 +31,14 @@ constexpr int kWideMaxStride = 3;
 // slots no longer leave room for 16 warps per SM, and only every second slot
 // is stored.
 constexpr int kQdSlotsFull = 12;
+// Evaluation from the monomials' values (kernels_sum.cu): limits above which
+// a handle keeps to the general kernels alone: tables of more than a quarter
+// of the free device memory (looked up from 1 GiB), and the pointers of its
+// addition lists.
+constexpr size_t kSumTableAsk = size_t{1} << 30;
+constexpr int64_t kSumPointersMax = int64_t{64} << 20;
+constexpr int kSumTiles = 3;       // log2 of the points per tile: 0, 1, 2
+constexpr int kSumCoefSkew = 40;  // and bits the components of a coefficient may be apart
 
 struct DeviceBuf {
   void *p = nullptr;
@@ -119,6 +127,20 @@ struct polyeval {
   std::vector<BatchTile> btiles;
   int batch_gcap = pe::kPointsPerWarp;  // most monomial groups a partial tile may take
   int batch_chunks = 0, batch_mode = 0;  // 0: built-in choice
+  // evaluation from the monomials' values (kernels_sum.cu)
+  int sum_L = 0;  // digits per number; 0: not available, the general kernels evaluate every call
+  struct SumLaunch {  // per log2 of the points of a tile
+    bool ok = false, tab_shared = false;
+    int threads = 0, blocks = 0;  // blocks: resident on the whole device
+    size_t smem = 0;
+  };
+  SumLaunch sum_launch[3];
+  int sum_batch_lg = 0;
+  std::vector<pe::SumSys> sum_sys;
+  int64_t sum_power_total = 0, sum_items_n = 0;  // batch
+  DeviceBuf sum_fac_ptr, sum_fac, sum_coef, sum_polys, sum_act, sum_bits, sum_hit_ptr, sum_hits, sum_sysd, sum_prefix, sum_items;
+  DeviceBuf sum_table, sum_ctl;  // sum_ctl: two work counters, whether any point is flagged, the points' flags
+  int64_t sum_points = 0;        // flags
   // timing of the main kernel
   bool timing = false;
   cudaEvent_t ev[2 * kMaxTimingEvents] = {};
@@ -561,18 +583,27 @@ pe::MainParams main_params(const polyeval *h) {
   return p;
 }
 
+// The next pair of timing events (nullptr: not timed).
+void timing_events(polyeval *h, cudaEvent_t &e0, cudaEvent_t &e1) {
+  e0 = e1 = nullptr;
+  if (!h->timing) return;
+  if (h->ev_used < kMaxTimingEvents) {
+    e0 = h->ev[2 * h->ev_used];
+    e1 = h->ev[2 * h->ev_used + 1];
+    h->ev_used++;
+  } else {
+    h->ev_dropped++;
+  }
+}
+
+// The general main kernel.  A call restricted to flagged points (mp.any) is
+// part of an evaluation that zeroed the counter and times the whole of it.
 int run_main(polyeval *h, const pe::MainParams &mp, cudaStream_t s, int mode = 0) {
   if (mp.n_items <= 0) return PE_OK;
-  if (cudaMemsetAsync(h->counter.p, 0, sizeof(unsigned), s) != cudaSuccess) return PE_ECUDA;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (h->timing) {
-    if (h->ev_used < kMaxTimingEvents) {
-      e0 = h->ev[2 * h->ev_used];
-      e1 = h->ev[2 * h->ev_used + 1];
-      h->ev_used++;
-    } else {
-      h->ev_dropped++;
-    }
+  if (!mp.any) {
+    if (cudaMemsetAsync(h->counter.p, 0, sizeof(unsigned), s) != cudaSuccess) return PE_ECUDA;
+    timing_events(h, e0, e1);
   }
   if (e0 && cudaEventRecord(e0, s) != cudaSuccess) return PE_ECUDA;
   const Shape sh = shape_for(h, mp.n_items, mode);
@@ -584,6 +615,349 @@ int run_main(polyeval *h, const pe::MainParams &mp, cudaStream_t s, int mode = 0
   if (e1 && cudaEventRecord(e1, s) != cudaSuccess) return PE_ECUDA;
   return PE_OK;
 }
+
+// ---------------------------------------------------------------------------
+// evaluation from the monomials' values
+// ---------------------------------------------------------------------------
+
+// sum_ctl: work counter of the sum kernel, whether any point is flagged, the
+// general kernels' counter, one spare word, the flags.
+constexpr size_t kCtlFlags = 16;
+
+// Lists, digits and buffers for a compiled system set, after everything the
+// general kernels need.  PE_OK with h->sum_L = 0 when the set does not suit
+// the kernels or the device has no room: those then evaluate every call.
+int setup_sum(polyeval *h, const Compiled &c) {
+  int dev = 0, optin = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+    return PE_ECUDA;
+  const int L = h->qd ? 8 : h->dd ? 4 : 3;
+  const int S = h->count;
+  const int cd = elem_doubles(h);
+  if (h->paper || c.poly_sys.empty()) return PE_OK;
+  const int64_t M = static_cast<int64_t>(c.mono_ptr.size()) - 1;
+  const size_t polys = c.poly_sys.size();
+  // per polynomial: its variables, those in the most monomials first (a warp's
+  // lists are then about equally long)
+  std::vector<pe::SumPoly> sp(polys);
+  std::vector<int32_t> act, count, slot;
+  std::vector<uint32_t> bits;
+  int64_t pointers = 0;
+  h->sum_sys.assign(S, pe::SumSys{});
+  for (size_t gp = 0; gp < polys; gp++) {
+    const SysDesc &d = h->sys[c.poly_sys[gp]];
+    pe::SumSys &ss = h->sum_sys[c.poly_sys[gp]];
+    const int32_t t0 = c.poly_ptr[gp], t1 = c.poly_ptr[gp + 1];
+    sp[gp].act_off = static_cast<int32_t>(act.size());
+    sp[gp].bits_off = static_cast<int32_t>(bits.size());
+    sp[gp].hit_off = pointers;
+    bits.resize(bits.size() + static_cast<size_t>((d.n + 31) / 32), 0u);
+    count.assign(d.n, 0);
+    for (int32_t j = c.mono_ptr[t0]; j < c.mono_ptr[t1]; j++) count[c.var[j] & 0xffffu]++;
+    for (int v = 0; v < d.n; v++)
+      if (count[v]) {
+        act.push_back(v);
+        bits[sp[gp].bits_off + (v >> 5)] |= 1u << (v & 31);
+      }
+    sp[gp].act_n = static_cast<int32_t>(act.size()) - sp[gp].act_off;
+    std::stable_sort(act.begin() + sp[gp].act_off, act.end(), [&](int32_t a, int32_t b) { return count[a] > count[b]; });
+    ss.act_max = std::max(ss.act_max, std::max(sp[gp].act_n, 1));
+    pointers += static_cast<int64_t>((t1 - t0 + pe::kSumBlock - 1) / pe::kSumBlock) * (sp[gp].act_n + 1);
+    if (pointers > kSumPointersMax || act.size() > INT32_MAX / 2 || bits.size() > INT32_MAX / 2) return PE_OK;
+  }
+  // per system: magnitude range, headroom
+  int m_max = 1, act_most = 1;
+  for (int s = 0; s < S; s++) {
+    const SysDesc &d = h->sys[s];
+    pe::SumSys &ss = h->sum_sys[s];
+    ss.act_max = std::max(ss.act_max, 1);
+    act_most = std::max(act_most, ss.act_max);
+    int deg = 1, m_sys = 1;
+    double gamma = 0.0;
+    for (int32_t gp = d.poly0; gp < d.poly0 + d.N; gp++) {
+      deg = std::max(deg, c.poly_deg[gp]);
+      const int32_t t0 = c.poly_ptr[gp], t1 = c.poly_ptr[gp + 1];
+      m_sys = std::max(m_sys, t1 - t0);
+      for (int32_t t = t0; t < t1; t++) {
+        const double re = std::fabs(c.coef[static_cast<size_t>(t) * cd]);
+        const double im = std::fabs(c.coef[static_cast<size_t>(t) * cd + cd / 2]);
+        int er = 0, ei = 0;
+        std::frexp(re, &er);
+        std::frexp(im, &ei);
+        // components so far apart that one common exponent would cost the
+        // smaller one its own relative precision
+        if (re != 0.0 && im != 0.0 && std::abs(er - ei) > kSumCoefSkew) return PE_OK;
+        if (re != 0.0 || im != 0.0)
+          gamma = std::max(gamma, std::fabs(static_cast<double>(re > im ? er : ei)) + 1.0);
+      }
+    }
+    // every monomial value within 2^(+-900) of 1: no overflow, and the low
+    // parts of the results well above the smallest normal double
+    if (gamma > 800.0) return PE_OK;
+    ss.most_log2 = static_cast<float>((900.0 - gamma) / deg);
+    int bl = 1;
+    while (bl < 62 && (int64_t{1} << bl) <= static_cast<int64_t>(m_sys) * d.emax) bl++;
+    ss.head_bits = std::max(pe::sum_head_bits_min(L), bl + 1);
+    if (ss.head_bits > 40) return PE_OK;
+    m_max = std::max(m_max, m_sys);
+  }
+  // launches: points per tile, threads, table in shared memory where it fits.
+  // A tile takes a multiple of kSumBlock monomials at a time.
+  const size_t room = static_cast<size_t>(optin) - 256;  // 256: the kernel's static shared memory
+  if (pe::prepare_sum(L, room) != cudaSuccess) return PE_ECUDA;
+  bool any = false;
+  for (int lg = 0; lg < kSumTiles; lg++) {
+    polyeval::SumLaunch &sl = h->sum_launch[lg];
+    int t = std::max(64, pe::kSumBlock << lg);
+    while (t < pe::kSumThreadsMax && (t >> lg) < std::max(m_max, act_most)) t *= 2;
+    sl.threads = h->batch ? pe::kSumThreadsMax : t;
+    for (int shared = 1; shared >= 0 && !sl.ok; shared--) {
+      size_t most = 0;
+      for (int s = 0; s < S; s++)
+        most = std::max(most, pe::sum_smem_bytes(L, h->sys[s].n, h->sum_sys[s].act_max, h->sys[s].emax, lg, sl.threads,
+                                                 shared != 0));
+      if (most > room) continue;
+      int b = 0;
+      if (pe::sum_occupancy(L, shared != 0, sl.threads, most, &b) != cudaSuccess) return PE_ECUDA;
+      if (b < 1) continue;
+      sl.ok = true;
+      sl.tab_shared = shared != 0;
+      sl.smem = most;
+      sl.blocks = b * h->sms;
+    }
+    any = any || sl.ok;
+  }
+  if (!any) return PE_OK;
+  // batch: the points per tile of every system (one launch)
+  if (h->batch) {
+    int lg = kSumTiles - 1;
+    while (lg > 0 && !h->sum_launch[lg].tab_shared) lg--;
+    if (!h->sum_launch[lg].tab_shared) {
+      lg = kSumTiles - 1;
+      while (lg > 0 && !h->sum_launch[lg].ok) lg--;
+      if (!h->sum_launch[lg].ok) return PE_OK;
+    }
+    h->sum_batch_lg = lg;
+    for (int s = 0; s < S; s++) h->sum_sys[s].lg = lg;
+  }
+  // tables and flags
+  int64_t fl = 0;
+  size_t tb = 0;
+  std::vector<int64_t> prefix{0};
+  for (int s = 0; s < S; s++) {
+    SysDesc &d = h->sys[s];
+    pe::SumSys &ss = h->sum_sys[s];
+    const int64_t P = h->batch ? d.P : h->max_points;
+    ss.flag_off = d.fl_off = fl;
+    fl += P;
+    ss.tab_off = static_cast<int64_t>(tb);
+    size_t most = 0;
+    for (int lg = 0; lg < kSumTiles; lg++) {
+      if (h->batch ? lg != ss.lg : !h->sum_launch[lg].ok) continue;
+      const int64_t tiles = (P + (1 << lg) - 1) >> lg;
+      most = std::max(most, static_cast<size_t>(tiles) * pe::sum_blob_bytes(L, d.n, d.emax, lg));
+      if (h->batch) prefix.push_back(prefix.back() + static_cast<int64_t>(d.n) * (tiles << lg));
+    }
+    tb += most;
+  }
+  if (tb == 0) return PE_OK;
+  if (tb > kSumTableAsk) {
+    size_t free_bytes = 0, all = 0;
+    if (cudaMemGetInfo(&free_bytes, &all) != cudaSuccess) return PE_ECUDA;
+    if (tb > free_bytes / 4) return PE_OK;
+  }
+  // monomials by falling k, their factors, the addition lists
+  if (static_cast<int64_t>(c.var.size()) + 4 * pointers > INT32_MAX) return PE_OK;
+  std::vector<int32_t> order(M), fac_ptr(M + 1), hit_ptr;
+  std::vector<uint32_t> fac(c.var.size());
+  std::vector<uint16_t> hits;
+  hit_ptr.reserve(static_cast<size_t>(pointers));
+  hits.reserve(c.var.size() + 2 * static_cast<size_t>(pointers));
+  std::vector<int32_t> at(static_cast<size_t>(act_most));
+  int32_t nf = 0;
+  fac_ptr[0] = 0;
+  for (size_t gp = 0; gp < polys; gp++) {
+    const int n = h->sys[c.poly_sys[gp]].n, na = sp[gp].act_n;
+    const int32_t t0 = c.poly_ptr[gp], t1 = c.poly_ptr[gp + 1];
+    slot.resize(n);
+    for (int i = 0; i < na; i++) slot[act[sp[gp].act_off + i]] = i;
+    auto k_of = [&](int32_t t) { return c.mono_ptr[t + 1] - c.mono_ptr[t]; };
+    std::iota(order.begin() + t0, order.begin() + t1, t0);
+    std::stable_sort(order.begin() + t0, order.begin() + t1, [&](int32_t a, int32_t b) { return k_of(a) > k_of(b); });
+    for (int32_t b = t0; b < t1; b += pe::kSumBlock) {
+      const int32_t e = std::min(b + pe::kSumBlock, t1);
+      std::fill(at.begin(), at.begin() + na, 0);
+      for (int32_t t = b; t < e; t++) {
+        for (int32_t j = c.mono_ptr[order[t]]; j < c.mono_ptr[order[t] + 1]; j++) {
+          const uint32_t v = c.var[j] & 0xffffu, a = c.var[j] >> 16;
+          fac[nf++] = (a - 1) * static_cast<uint32_t>(n) + v;
+          at[slot[v]]++;
+        }
+        fac_ptr[t + 1] = nf;
+      }
+      size_t nh = hits.size();
+      const size_t hp = hit_ptr.size();
+      for (int i = 0; i < na; i++) {
+        hit_ptr.push_back(static_cast<int32_t>(nh / 4));
+        const int32_t n_hits = at[i];
+        at[i] = static_cast<int32_t>(nh);
+        nh += static_cast<size_t>(n_hits + 3) / 4 * 4;
+      }
+      hit_ptr.push_back(static_cast<int32_t>(nh / 4));
+      hits.resize(nh, 0);
+      for (int32_t t = b; t < e; t++)
+        for (int32_t j = c.mono_ptr[order[t]]; j < c.mono_ptr[order[t] + 1]; j++)
+          hits[at[slot[c.var[j] & 0xffffu]]++] = static_cast<uint16_t>((t - b) | (c.var[j] >> 16) << 6);
+      for (int i = 0; i < na; i++)  // filled up to a multiple of four: the last monomial, zero times
+        for (size_t x = at[i]; x < 4 * static_cast<size_t>(hit_ptr[hp + i + 1]); x++)
+          hits[x] = static_cast<uint16_t>(hits[x - 1] & (pe::kSumBlock - 1));
+    }
+  }
+  // batch: items of one tile and a run of polynomials, the costly first
+  std::vector<int32_t> words;
+  if (h->batch) {
+    struct Run {
+      int32_t gp, polys, tile, s;
+      double cost;
+    };
+    std::vector<Run> runs;
+    double total = 0.0;
+    auto cost_of = [&](size_t gp) {
+      const int32_t t0 = c.poly_ptr[gp], t1 = c.poly_ptr[gp + 1];
+      return static_cast<double>(c.mono_ptr[t1] - c.mono_ptr[t0]) + 2.0 * h->sys[c.poly_sys[gp]].n + 64.0;
+    };
+    for (size_t gp = 0; gp < c.poly_sys.size(); gp++) {
+      const SysDesc &d = h->sys[c.poly_sys[gp]];
+      total += cost_of(gp) * static_cast<double>((d.P + (1 << h->sum_batch_lg) - 1) >> h->sum_batch_lg);
+    }
+    const double share = total / (16.0 * h->sum_launch[h->sum_batch_lg].blocks);
+    for (int s = 0; s < S; s++) {
+      const SysDesc &d = h->sys[s];
+      const int lg = h->sum_sys[s].lg;
+      const int32_t tiles = (d.P + (1 << lg) - 1) >> lg;
+      for (int32_t p = 0; p < d.N;) {
+        Run r{d.poly0 + p, 0, 0, s, 0.0};
+        while (p < d.N && (r.polys == 0 || r.cost + cost_of(d.poly0 + p) <= share)) {
+          r.cost += cost_of(d.poly0 + p);
+          r.polys++;
+          p++;
+        }
+        for (int32_t t = 0; t < tiles; t++) {
+          r.tile = t;
+          runs.push_back(r);
+        }
+      }
+    }
+    std::stable_sort(runs.begin(), runs.end(), [](const Run &a, const Run &b) { return a.cost > b.cost; });
+    for (const Run &r : runs) words.insert(words.end(), {r.gp, r.polys, r.tile, r.s});
+    h->sum_items_n = static_cast<int64_t>(runs.size());
+    h->sum_power_total = prefix.back();
+    if (h->sum_items_n == 0 || h->sum_items_n > INT32_MAX) return PE_OK;
+  }
+  // a device that cannot hold the extra buffers evaluates with the general
+  // kernels
+  DeviceBuf ord, co;
+  int rc;
+  if ((rc = h->sum_fac_ptr.upload(fac_ptr)) || (rc = h->sum_fac.upload(fac)) || (rc = h->sum_polys.upload(sp)) || (rc = h->sum_act.upload(act)) || (rc = h->sum_bits.upload(bits)) ||
+      (rc = h->sum_hit_ptr.upload(hit_ptr)) || (rc = h->sum_hits.upload(hits)) || (rc = h->sum_sysd.upload(h->sum_sys)) ||
+      (rc = h->sum_prefix.upload(prefix)) || (rc = h->sum_items.upload(words)) || (rc = ord.upload(order)) ||
+      (rc = co.upload(c.coef)) ||
+      (rc = h->sum_coef.alloc(static_cast<size_t>(M) * 4 * (L == 3 ? 8 : L == 4 ? 12 : 20))) ||
+      (rc = h->sum_table.alloc(tb)) || (rc = h->sum_ctl.alloc(kCtlFlags + static_cast<size_t>(fl)))) {
+    for (DeviceBuf *b : {&h->sum_fac_ptr, &h->sum_fac, &h->sum_polys, &h->sum_act, &h->sum_bits, &h->sum_hit_ptr, &h->sum_hits, &h->sum_sysd,
+                         &h->sum_prefix, &h->sum_items, &h->sum_coef, &h->sum_table, &h->sum_ctl})
+      b->alloc(0);
+    return rc == PE_ENOMEM ? PE_OK : rc;
+  }
+  if (cudaMemcpy(h->sysd.p, h->sys.data(), h->sys.size() * sizeof(SysDesc), cudaMemcpyHostToDevice) != cudaSuccess)
+    return PE_ECUDA;  // the flags' offsets
+  if (pe::convert_coef_sum(L, static_cast<const double *>(co.p), static_cast<const int32_t *>(ord.p),
+                           static_cast<int32_t *>(h->sum_coef.p), M, nullptr) != cudaSuccess ||
+      cudaDeviceSynchronize() != cudaSuccess)
+    return PE_ECUDA;
+  h->sum_points = fl;
+  h->sum_L = L;
+  return PE_OK;
+}
+
+// Points per tile (log2) of a single-system call: 8 points, which one
+// 128-byte row of the table holds, or as few as it takes to give every SM a
+// (polynomial, tile) item.
+int sum_tile_log2(const polyeval *h, int64_t P) {
+  const int64_t N = h->sys[0].N;
+  int best = -1;
+  for (int lg = kSumTiles - 1; lg >= 0; lg--) {
+    if (!h->sum_launch[lg].ok) continue;
+    if (best >= 0 && (h->sum_launch[best].tab_shared || !h->sum_launch[lg].tab_shared) &&
+        N * ((P + (1 << best) - 1) >> best) >= h->sms)
+      break;
+    best = lg;
+  }
+  return best;
+}
+
+// Queue the evaluation (e0: recorded after the power table).  P < 0: batch.
+int run_sum(polyeval *h, const void *points, int64_t P, void *out_f, void *out_J, cudaEvent_t e0, cudaStream_t s) {
+  pe::SumParams sp{};
+  sp.poly_ptr = static_cast<const int32_t *>(h->poly_ptr.p);
+  sp.fac_ptr = static_cast<const int32_t *>(h->sum_fac_ptr.p);
+  sp.fac = static_cast<const uint32_t *>(h->sum_fac.p);
+  sp.coef = static_cast<const int32_t *>(h->sum_coef.p);
+  sp.polys = static_cast<const pe::SumPoly *>(h->sum_polys.p);
+  sp.act = static_cast<const int32_t *>(h->sum_act.p);
+  sp.act_bits = static_cast<const uint32_t *>(h->sum_bits.p);
+  sp.hit_ptr = static_cast<const int32_t *>(h->sum_hit_ptr.p);
+  sp.hits = static_cast<const uint2 *>(h->sum_hits.p);
+  sp.sys = static_cast<const SysDesc *>(h->sysd.p);
+  sp.sum_sys = static_cast<const pe::SumSys *>(h->sum_sysd.p);
+  sp.prefix = static_cast<const int64_t *>(h->sum_prefix.p);
+  sp.items = static_cast<const int4 *>(h->sum_items.p);
+  sp.points = static_cast<const double *>(points);
+  sp.out_f = static_cast<double *>(out_f);
+  sp.out_J = static_cast<double *>(out_J);
+  sp.table = static_cast<unsigned char *>(h->sum_table.p);
+  sp.count = h->count;
+  sp.n_polys_total = h->n_polys_total;
+  unsigned char *ctl = static_cast<unsigned char *>(h->sum_ctl.p);
+  sp.counter = reinterpret_cast<unsigned *>(ctl);
+  sp.any = reinterpret_cast<int32_t *>(ctl + 4);
+  sp.flags = ctl + kCtlFlags;
+  int lg = h->sum_batch_lg;
+  if (P >= 0) {
+    const SysDesc &d = h->sys[0];
+    lg = sum_tile_log2(h, P);
+    const int64_t tiles = (P + (1 << lg) - 1) >> lg;
+    const polyeval::SumLaunch &sl = h->sum_launch[lg];
+    sp.single_P = static_cast<int32_t>(P);
+    sp.single_lg = lg;
+    sp.power_total = static_cast<int64_t>(d.n) * (tiles << lg);
+    // runs of polynomials that share a copy of the table: about 8 runs per
+    // resident block, so that the last wave is short
+    const int64_t run = std::max<int64_t>(1, std::min<int64_t>(16, tiles * d.N / (8 * static_cast<int64_t>(sl.blocks))));
+    sp.group_polys = static_cast<int32_t>(run);
+    sp.groups = static_cast<int32_t>((d.N + run - 1) / run);
+    sp.n_items = tiles * sp.groups;
+    if (sp.n_items > INT32_MAX) return PE_ERANGE;
+  } else {
+    sp.single_P = -1;
+    sp.power_total = h->sum_power_total;
+    sp.n_items = h->sum_items_n;
+  }
+  const polyeval::SumLaunch &sl = h->sum_launch[lg];
+  const size_t flagged = P >= 0 ? static_cast<size_t>(P) : static_cast<size_t>(h->sum_points);
+  if (cudaMemsetAsync(h->sum_ctl.p, 0, kCtlFlags + flagged, s) != cudaSuccess) return PE_ECUDA;
+  if (pe::launch_sum_powers(h->sum_L, sp, s) != cudaSuccess) return PE_ECUDA;
+  if (e0 && cudaEventRecord(e0, s) != cudaSuccess) return PE_ECUDA;
+  const int grid = static_cast<int>(std::min<int64_t>(sp.n_items, sl.blocks));
+  if (pe::launch_sum(h->sum_L, sp, sl.tab_shared, sl.threads, sl.smem, grid, s) != cudaSuccess) return PE_ECUDA;
+  h->kernels_launched += 2;
+  return PE_OK;
+}
+
+const int32_t *sum_any(const polyeval *h) { return reinterpret_cast<const int32_t *>(static_cast<const unsigned char *>(h->sum_ctl.p) + 4); }
+unsigned *general_counter(const polyeval *h) { return reinterpret_cast<unsigned *>(static_cast<unsigned char *>(h->sum_ctl.p) + 8); }
+const unsigned char *sum_flags(const polyeval *h) { return static_cast<const unsigned char *>(h->sum_ctl.p) + kCtlFlags; }
 
 }  // namespace
 
@@ -624,6 +998,7 @@ int polyeval_create(const pe_system *sys, int precision, uint32_t flags, int64_t
     h = new polyeval();
     set_precision(h, precision);
     h->batch = false;
+    h->paper = (flags & PE_PAPER_KERNELS) != 0;
     h->count = 1;
     h->max_points = max_points;
     h->sys.resize(1);
@@ -679,6 +1054,10 @@ int polyeval_create(const pe_system *sys, int precision, uint32_t flags, int64_t
         delete h;
         return rc;
       }
+    }
+    if ((rc = setup_sum(h, c)) != PE_OK) {
+      delete h;
+      return rc;
     }
   } catch (const std::bad_alloc &) {
     delete h;
@@ -776,6 +1155,10 @@ int polyeval_create_many(const pe_system *systems, int32_t count, int precision,
         return rc;
       }
     }
+    if ((rc = setup_sum(h, c)) != PE_OK) {
+      delete h;
+      return rc;
+    }
   } catch (const std::bad_alloc &) {
     delete h;
     return PE_ENOMEM;
@@ -829,8 +1212,10 @@ int default_groups(int64_t P) {
   return G;
 }
 
+// `general`: with the general kernels alone (the autotuner, whose choices are
+// theirs).
 int eval_single(polyeval *h, const void *points, int64_t P, void *out_f, void *out_J, cudaStream_t s, int chunks,
-                int mode, int groups = 0) {
+                int mode, int groups = 0, bool general = false) {
   if (!h || h->batch || P < 0) return PE_EINVAL;
   if (P == 0) return PE_OK;
   if (P > h->max_points) return PE_ERANGE;
@@ -865,8 +1250,21 @@ int eval_single(polyeval *h, const void *points, int64_t P, void *out_f, void *o
     h->kernels_launched += 3;
     return PE_OK;
   }
+  // First from the monomials' values; the general kernels below then take
+  // the tiles of flagged points (none, as a rule: they return at once).
+  const bool by_values = h->sum_L > 0 && !general && d.N > 0;
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  if (by_values) {
+    timing_events(h, e0, e1);
+    const int r = run_sum(h, points, P, out_f, out_J, e0, s);
+    if (r != PE_OK) return r;
+  }
   if (table_levels(h, d.emax) > 0) {
     pe::PowerParams pp{};
+    if (by_values) {
+      pp.any = sum_any(h);
+      pp.flags = sum_flags(h);
+    }
     pp.sys = static_cast<const SysDesc *>(h->sysd.p);
     pp.points = static_cast<const double *>(points);
     pp.table = static_cast<double *>(h->table.p);
@@ -890,9 +1288,12 @@ int eval_single(polyeval *h, const void *points, int64_t P, void *out_f, void *o
         if (groups <= 0) groups = t.groups;
       }
   }
-  // monomial groups per warp (double-double and double kernels only)
+  // monomial groups per warp (double-double and double kernels only; after
+  // the evaluation from the monomials' values they are chosen per item)
   int G = block_format(h) ? 1 : (groups > 0 ? groups : default_groups(P));
   if (G != 1 && G != 2 && G != 4 && G != 8 && G != 16) G = 1;
+  const bool regroup = by_values && !block_format(h) && groups <= 0;
+  if (regroup) G = 1;
   mp.groups = G;
   mp.tile_points = pe::kPointsPerWarp / G;
   mp.single_T = static_cast<int32_t>((P + mp.tile_points - 1) / mp.tile_points);
@@ -920,32 +1321,52 @@ int eval_single(polyeval *h, const void *points, int64_t P, void *out_f, void *o
   mp.scratch_J = C > 1 ? mp.scratch_f + static_cast<size_t>(C - 1) * f_doubles : nullptr;
   mp.n_items = base * C;
   if (mp.n_items > INT32_MAX) return PE_ERANGE;  // the work counter is 32-bit
+  mp.finish = C == 1;
+  pe::Only only{nullptr, nullptr, static_cast<int32_t>(P)};
+  if (by_values) {
+    mp.any = only.any = sum_any(h);
+    mp.flags = only.flags = sum_flags(h);
+    mp.regroup = regroup;
+    mp.counter = general_counter(h);
+  }
   int rc = run_main(h, mp, s, mode);
   if (rc != PE_OK) return rc;
-  if (h->qd) {  // add the chunks' accumulators, round to quad-double
-    if (base > 0 && pe::launch_finalize_qd(mp.out_f, mp.out_J, mp.scratch_f, mp.scratch_J, 2 * static_cast<int64_t>(d.N) * P,
-                                           2 * static_cast<int64_t>(d.N) * d.n * P, C, s) != cudaSuccess)
+  if (C > 1 && h->qd) {  // add the chunks' accumulators, round to quad-double
+    if (pe::launch_finalize_qd(mp.out_f, mp.out_J, mp.scratch_f, mp.scratch_J, 2 * static_cast<int64_t>(d.N) * P,
+                               2 * static_cast<int64_t>(d.N) * d.n * P, C, only, s) != cudaSuccess)
       return PE_ECUDA;
-    if (base > 0) h->kernels_launched++;
-    return PE_OK;
+    h->kernels_launched++;
+  } else if (C > 1) {
+    if (pe::launch_combine(h->dd, mp.out_f, mp.out_J, mp.scratch_f, mp.scratch_J, f_doubles, J_doubles, C, only, s) !=
+        cudaSuccess)
+      return PE_ECUDA;
+    h->kernels_launched++;
   }
-  if (C == 1) return rc;
-  if (pe::launch_combine(h->dd, mp.out_f, mp.out_J, mp.scratch_f, mp.scratch_J, f_doubles, J_doubles, C, s) !=
-      cudaSuccess)
-    return PE_ECUDA;
-  h->kernels_launched += 2;  // f and J passes
+  if (e1 && cudaEventRecord(e1, s) != cudaSuccess) return PE_ECUDA;
   return PE_OK;
 }
 
 // One batch evaluation.  chunks > 0 and mode > 0 force the monomial chunk
 // count and the launch shape (the autotuner); 0 takes the handle's choice,
 // else the built-in one (one chunk; the shape from the item count).
-int eval_many(polyeval *h, const void *points, void *out_f, void *out_J, cudaStream_t s, int chunks, int mode) {
+int eval_many(polyeval *h, const void *points, void *out_f, void *out_J, cudaStream_t s, int chunks, int mode,
+              bool general = false) {
   if (!h || !h->batch) return PE_EINVAL;
   if (h->n_items_batch == 0) return PE_OK;
   if (!points || !out_f || !out_J || !arrays_aligned(points, out_f, out_J)) return PE_EINVAL;
+  const bool by_values = h->sum_L > 0 && !general;
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  if (by_values) {
+    timing_events(h, e0, e1);
+    const int r = run_sum(h, points, -1, out_f, out_J, e0, s);
+    if (r != PE_OK) return r;
+  }
   if (h->power_total_batch > 0) {
     pe::PowerParams pp{};
+    if (by_values) {
+      pp.any = sum_any(h);
+      pp.flags = sum_flags(h);
+    }
     pp.sys = static_cast<const SysDesc *>(h->sysd.p);
     pp.prefix = static_cast<const int64_t *>(h->prefix.p);
     pp.points = static_cast<const double *>(points);
@@ -961,6 +1382,7 @@ int eval_many(polyeval *h, const void *points, void *out_f, void *out_J, cudaStr
   int C = std::max(1, std::min(chunks, kMaxChunks));
   C = static_cast<int>(std::min<int64_t>(C, 1 + static_cast<int64_t>(per_chunk ? h->scratch.bytes / per_chunk : 0)));
   if (h->n_items_batch * C > INT32_MAX) C = 1;  // the work counter is 32-bit
+  if (by_values) C = 1;  // the passes that add chunks do not know the systems' flags
   const int64_t f_doubles = static_cast<int64_t>(elem_doubles(h)) * h->f_total_batch;
   const int64_t J_doubles = static_cast<int64_t>(elem_doubles(h)) * h->J_total_batch;
   pe::MainParams mp = main_params(h);
@@ -975,20 +1397,28 @@ int eval_many(polyeval *h, const void *points, void *out_f, void *out_J, cudaStr
   mp.scratch_f = static_cast<double *>(h->scratch.p);
   mp.scratch_J = C > 1 ? mp.scratch_f + static_cast<size_t>(C - 1) * f_doubles : nullptr;
   mp.n_items = h->n_items_batch * C;
-  const int rc = run_main(h, mp, s, std::max(mode, 0));
+  mp.finish = C == 1;
+  if (by_values) {
+    mp.any = sum_any(h);
+    mp.flags = sum_flags(h);
+    mp.regroup = !block_format(h);
+    mp.counter = general_counter(h);
+  }
+  const int rc = run_main(h, mp, s, by_values ? 2 : std::max(mode, 0));
   if (rc != PE_OK) return rc;
-  if (h->qd) {  // add the chunks' accumulators, round to quad-double
+  const pe::Only every{};
+  if (C > 1 && h->qd) {  // add the chunks' accumulators, round to quad-double
     if (pe::launch_finalize_qd(mp.out_f, mp.out_J, mp.scratch_f, mp.scratch_J, 2 * h->f_total_batch,
-                               2 * h->J_total_batch, C, s) != cudaSuccess)
+                               2 * h->J_total_batch, C, every, s) != cudaSuccess)
       return PE_ECUDA;
     h->kernels_launched++;
-    return PE_OK;
+  } else if (C > 1) {
+    if (pe::launch_combine(h->dd, mp.out_f, mp.out_J, mp.scratch_f, mp.scratch_J, f_doubles, J_doubles, C, every, s) !=
+        cudaSuccess)
+      return PE_ECUDA;
+    h->kernels_launched++;
   }
-  if (C == 1) return PE_OK;
-  if (pe::launch_combine(h->dd, mp.out_f, mp.out_J, mp.scratch_f, mp.scratch_J, f_doubles, J_doubles, C, s) !=
-      cudaSuccess)
-    return PE_ECUDA;
-  h->kernels_launched += 2;  // f and J passes
+  if (e1 && cudaEventRecord(e1, s) != cudaSuccess) return PE_ECUDA;
   return PE_OK;
 }
 
@@ -1039,10 +1469,10 @@ int autotune_many(polyeval *h, const void *points, void *out_f, void *out_J, cud
       if (h->n_items_batch * C > INT32_MAX) continue;
       for (int m = 1; m <= 2 && rc == PE_OK; m++) {
         if (m == 1 && h->n_items_batch * C > capacity) continue;  // one wave only when every item is resident
-        rc = eval_many(h, points, out_f, out_J, s, C, m);  // warm-up
+        rc = eval_many(h, points, out_f, out_J, s, C, m, true);  // warm-up
         if (rc != PE_OK) break;
         if (cudaEventRecord(e0, s) != cudaSuccess) rc = PE_ECUDA;
-        for (int r = 0; r < 3 && rc == PE_OK; r++) rc = eval_many(h, points, out_f, out_J, s, C, m);
+        for (int r = 0; r < 3 && rc == PE_OK; r++) rc = eval_many(h, points, out_f, out_J, s, C, m, true);
         if (rc == PE_OK && (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess))
           rc = PE_ECUDA;
         float ms = 0.0f;
@@ -1119,10 +1549,10 @@ int polyeval_autotune(polyeval_t *h, const void *points, int64_t P, void *out_f,
       if (base * C > INT32_MAX) continue;
       for (int m = 1; m <= 2 && rc == PE_OK; m++) {
         if (m == 1 && base * C > capacity) continue;  // one wave only when every item is resident
-        rc = eval_single(h, points, P, out_f, out_J, s, C, m, G);  // warm-up
+        rc = eval_single(h, points, P, out_f, out_J, s, C, m, G, true);  // warm-up
         if (rc != PE_OK) break;
         if (cudaEventRecord(e0, s) != cudaSuccess) rc = PE_ECUDA;
-        for (int r = 0; r < 3 && rc == PE_OK; r++) rc = eval_single(h, points, P, out_f, out_J, s, C, m, G);
+        for (int r = 0; r < 3 && rc == PE_OK; r++) rc = eval_single(h, points, P, out_f, out_J, s, C, m, G, true);
         if (rc == PE_OK && (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess))
           rc = PE_ECUDA;
         float ms = 0.0f;

@@ -49,6 +49,7 @@ struct SysDesc {
   int64_t f_off;   // f       [N][P]
   int64_t J_off;   // J       [N][n][P]
   int64_t tab_off; // powers  [emax-2][n][P]  (x^2 .. x^(emax-1))
+  int64_t fl_off;  // flags   [P]  (points left to the general kernels by kernels_sum.cu)
 };
 
 struct MainParams {
@@ -80,6 +81,13 @@ struct MainParams {
   double *scratch_J;
   unsigned int *counter;    // work counter (zeroed before each launch)
   int *status;              // device status word
+  // After the evaluation of kernels_sum.cu: only flagged points are
+  // evaluated, so that a point's results do not depend on its neighbours
+  // (nullptr: all points).
+  const int32_t *any;           // whether there is one
+  const unsigned char *flags;   // per point
+  int32_t regroup;          // choose the monomial groups per item from its flagged points (double-double and double)
+  int32_t finish;           // quad-double: round the sums in the outputs (calls of one chunk)
 };
 
 struct PowerParams {
@@ -92,7 +100,85 @@ struct PowerParams {
   int32_t single_P;         // >= 0: single-system handle
   int32_t single_n;
   int32_t single_emax;
+  const int32_t *any;           // as in MainParams: only flagged points
+  const unsigned char *flags;
 };
+
+// Evaluation from the monomials' values (kernels_sum.cu), in numbers of L
+// digits: L = 3 (double), 4 (double-double), 8 (quad-double).
+constexpr int kSumThreadsMax = 256;
+constexpr int kSumPointsMax = 4;   // points per tile: 1, 2 or 4
+constexpr int kSumBlock = 64;      // monomials per block of the addition lists (their entries hold 6 bits of it)
+
+// One compiled system.
+struct SumSys {
+  int64_t tab_off;    // bytes: its tables
+  int64_t flag_off;   // its points' flags
+  float most_log2;    // points with a coordinate modulus outside 2^(+-most_log2) are flagged
+  int32_t lg;         // log2 of the points per tile (batch handles)
+  int32_t act_max;    // most variables of a polynomial
+  int32_t head_bits;  // headroom of the window: log2 of a bound of sum_t a_t
+};
+
+// One polynomial: its variables ("active"), and its lists, per block of
+// kSumBlock monomials one per active variable.
+struct SumPoly {
+  int64_t hit_off;   // first list pointer: per block act_n + 1 offsets into hits
+  int32_t act_off;   // active variables, in act
+  int32_t act_n;
+  int32_t bits_off;  // the same as a bit mask of n bits
+  int32_t pad;
+};
+
+struct SumParams {
+  const int32_t *poly_ptr;  // [Ntot+1] monomials of each polynomial (by falling k within it)
+  const int32_t *fac_ptr;   // [M+1] offsets into fac
+  const uint32_t *fac;      // table entries (a - 1) n + v of each monomial
+  const int32_t *coef;      // [M][kSumCoefWords] digits
+  const SumPoly *polys;     // [Ntot]
+  const int32_t *act;
+  const uint32_t *act_bits;
+  const int32_t *hit_ptr;
+  const uint2 *hits;        // four 16-bit entries each: monomial of the block | exponent << 6 (0: no more)
+  const SysDesc *sys;
+  const SumSys *sum_sys;
+  const int64_t *prefix;    // batch: [count+1] prefix sums of n_s * padded points
+  const int4 *items;        // batch: (first polynomial, polynomials, tile, system)
+  const double *points;
+  double *out_f;
+  double *out_J;
+  unsigned char *table;
+  int64_t power_total;      // (variable, padded point) pairs
+  int64_t n_items;
+  int32_t count;
+  int32_t single_P;         // >= 0: single-system handle
+  int32_t single_lg;
+  int32_t groups, group_polys;  // single: runs of polynomials per tile, polynomials per run
+  int32_t n_polys_total;
+  unsigned *counter;        // work counter and ...
+  int32_t *any;             // ... whether any point is flagged, zeroed before each call with ...
+  unsigned char *flags;     // ... the flags of the points
+};
+
+template <int L>
+constexpr int kSumCoefWords = L == 3 ? 8 : L == 4 ? 12 : 20;
+
+// Bytes of a tile's table (entries x^1 .. x^levels of n variables) and of the
+// table with the inverses that follow it.
+__host__ __device__ constexpr size_t sum_entry_bytes(int L) { return L == 3 ? 32 : L == 4 ? 36 : 68; }
+__host__ __device__ constexpr size_t sum_tab_bytes(int L, int n, int levels, int lg) {
+  return ((static_cast<size_t>(levels) * n * sum_entry_bytes(L) << lg) + 15) & ~size_t{15};
+}
+__host__ __device__ constexpr size_t sum_blob_bytes(int L, int n, int levels, int lg) {
+  return sum_tab_bytes(L, n, levels, lg) + sum_tab_bytes(L, n, 1, lg);
+}
+size_t sum_smem_bytes(int L, int n, int act_max, int levels, int lg, int threads, bool tab_shared);
+int sum_head_bits_min(int L);
+cudaError_t prepare_sum(int L, size_t smem);
+cudaError_t sum_occupancy(int L, bool tab_shared, int threads, size_t smem, int *blocks);
+cudaError_t launch_sum_powers(int L, const SumParams &p, cudaStream_t s);
+cudaError_t launch_sum(int L, const SumParams &p, bool tab_shared, int threads, size_t smem, int grid, cudaStream_t s);
+cudaError_t convert_coef_sum(int L, const double *coef, const int32_t *order, int32_t *out, int64_t M, cudaStream_t s);
 
 // Launchers (kernels.cu).  `dd` selects complex double-double, else complex
 // double.  They return the cudaError_t of the launch.
@@ -106,8 +192,14 @@ cudaError_t fp64_peak_probe(cudaStream_t s, double *fma_per_s, double *sm_clock_
 // Adds the chunk partial results into the outputs and renormalises:
 // out[i] = out[i] + scratch_1[i] + ... + scratch_{C-1}[i] for the f and J
 // arrays of one system (elements of `doubles_per_elem` doubles).
+// `only`: only the flagged points (single-system calls).
+struct Only {
+  const int32_t *any;          // nullptr: every entry
+  const unsigned char *flags;
+  int32_t P;
+};
 cudaError_t launch_combine(bool dd, double *out_f, double *out_J, const double *scratch_f, const double *scratch_J,
-                           int64_t f_doubles, int64_t J_doubles, int chunks, cudaStream_t s);
+                           int64_t f_doubles, int64_t J_doubles, int chunks, const Only &only, cudaStream_t s);
 
 // Newton step (newton.cu): solve J dx = -f per point, x += dx.
 struct NewtonParams {
@@ -165,7 +257,8 @@ cudaError_t launch_main_qd(const MainParams &p, int warps_per_block, size_t smem
 // 1 .. chunks-1 of the same layout) and rounds them to quad-double in the
 // outputs.  Components are 32-byte halves of a complex entry.
 cudaError_t launch_finalize_qd(double *out_f, double *out_J, const double *scratch_f, const double *scratch_J,
-                               int64_t f_components, int64_t J_components, int chunks, cudaStream_t s);
+                               int64_t f_components, int64_t J_components, int chunks, const Only &only,
+                               cudaStream_t s);
 
 // Path tracker (track.cu).  Phases of a path and its status (the status
 // values are the PE_PATH_* codes of the C ABI).

@@ -26,7 +26,8 @@ struct Item {
   double *J_base;      // output (or scratch) base for J
 };
 
-// Returns false (and flags the status word) for an inconsistent item.
+// Returns false for an item to skip: one without a flagged point in a call
+// that evaluates only those, or an inconsistent one (flags the status word).
 __device__ __forceinline__ bool decode_item(const MainParams &kp, unsigned item, int lane, Item &it) {
   int chunk = 0;
   if (kp.single_P >= 0) {
@@ -54,6 +55,21 @@ __device__ __forceinline__ bool decode_item(const MainParams &kp, unsigned item,
       it.tile * (kPointsPerWarp / it.groups) >= it.P) {
     if (lane == 0) atomicOr(kp.status, 1);
     return false;
+  }
+  if (kp.flags) {
+    // flagged points only; few of them spread over the warp's monomial
+    // groups: the most groups whose sub-tile holds them all
+    const int tp = kPointsPerWarp / it.groups, q = it.tile * tp + lane;
+    const unsigned set = __ballot_sync(0xffffffffu, lane < tp && q < it.P && kp.flags[kp.sys[it.s].fl_off + q] != 0);
+    if (set == 0u) return false;
+    if (kp.regroup) {
+      int first = __ffs(static_cast<int>(set)) - 1, last = 31 - __clz(static_cast<int>(set)), sub = tp;
+      while (sub > 1 && first / (sub / 2) == last / (sub / 2)) {
+        sub /= 2;
+        it.groups *= 2;
+      }
+      it.tile = (it.tile * tp + first) / sub;
+    }
   }
   int t0 = kp.poly_ptr[it.gp], t1 = kp.poly_ptr[it.gp + 1];
   if (kp.n_chunks > 1) {

@@ -58,8 +58,8 @@ __device__ void process_item(const MainParams &kp, const Item &it, typename A::V
   const SysDesc sd = kp.sys[s];
   const int n = sd.n;
   const int q = tile * kPointsPerWarp + (lane >> 1);
-  const bool valid = q < P;
-  const int qc = valid ? q : P - 1;  // lanes past the end compute on the last point and store nothing
+  const bool valid = q < P && (!kp.flags || kp.flags[sd.fl_off + q]);
+  const int qc = min(q, P - 1);  // lanes past the end compute on the last point and store nothing
   const int c = lane & 1;
   const unsigned long long sgn = c ? 0ULL : kSign;
   const size_t Pz = static_cast<size_t>(P);
@@ -156,8 +156,8 @@ __device__ void process_item_groups(const MainParams &kp, const Item &it, typena
   const int n = sd.n;
   const int g = lane / GL;
   const int q = tile * QP + ((lane % GL) >> 1);
-  const bool valid = q < P;
-  const int qc = valid ? q : P - 1;
+  const bool valid = q < P && (!kp.flags || kp.flags[sd.fl_off + q]);
+  const int qc = min(q, P - 1);
   const int c = lane & 1;
   const unsigned long long sgn = c ? 0ULL : kSign;
   const unsigned pm = 3u << (lane & 30);
@@ -248,6 +248,7 @@ __global__ void main_kernel(const MainParams kp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   typename A::V *smem = reinterpret_cast<typename A::V *>(smem_raw) + static_cast<size_t>(warp) * kp.kslots * 32;
+  if (kp.any && *kp.any == 0) return;
   for (;;) {
     unsigned item = 0;
     if (lane == 0) item = atomicAdd(kp.counter, 1u);
@@ -266,10 +267,11 @@ __global__ void main_kernel(const MainParams kp) {
 template <class A>
 __global__ void powers_kernel(const PowerParams pp) {
   constexpr int KD = A::kDoubles;
+  if (pp.any && *pp.any == 0) return;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; idx < pp.total; idx += stride) {
     int n, emax, P;
-    int64_t local, pt_off, tab_off;
+    int64_t local, pt_off, tab_off, fl_off = 0;
     if (pp.single_P >= 0) {
       n = pp.single_n;
       emax = pp.single_emax;
@@ -290,8 +292,10 @@ __global__ void powers_kernel(const PowerParams pp) {
       local = idx - pp.prefix[lo];
       pt_off = sd.pt_off;
       tab_off = sd.tab_off;
+      fl_off = sd.fl_off;
     }
     const int64_t v = local / P, q = local - v * P;
+    if (pp.flags && !pp.flags[fl_off + q]) continue;
     const typename A::Full x = A::load_full(pp.points + (pt_off + v * P + q) * KD);
     auto entry = [&](int e) { return pp.table + (tab_off + (static_cast<int64_t>(e - 2) * n + v) * P + q) * KD; };
     // x^e = x^(e - h) * x^h with h = floor(e/2): one product per entry as in
@@ -305,12 +309,20 @@ __global__ void powers_kernel(const PowerParams pp) {
   }
 }
 
-// out[i] += sum of the chunk partials, renormalised (one component per thread).
+// out[i] += sum of the chunk partials, renormalised (one component per
+// thread): f, then J.
 template <class A>
-__global__ void combine_kernel(double *out, const double *scratch, int64_t comps, int64_t stride, int chunks) {
+__global__ void combine_kernel(double *out_f, double *out_J, const double *scratch_f, const double *scratch_J,
+                               int64_t f_doubles, int64_t J_doubles, int chunks, Only only) {
   constexpr int CD = A::kDoubles / 2;  // doubles per component
+  if (only.any && *only.any == 0) return;
   const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < comps; i += step) {
+  for (int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; k < (f_doubles + J_doubles) / CD; k += step) {
+    const bool isf = k < f_doubles / CD;
+    const int64_t i = isf ? k : k - f_doubles / CD, stride = isf ? f_doubles : J_doubles;
+    if (only.any && !only.flags[i / 2 % only.P]) continue;
+    double *out = isf ? out_f : out_J;
+    const double *scratch = isf ? scratch_f : scratch_J;
     typename A::V acc = A::load_comp(out + i * CD, 0);
     for (int c = 1; c < chunks; c++) acc = A::add(acc, A::load_comp(scratch + (c - 1) * stride + i * CD, 0));
     A::store_comp(out + i * CD, 0, A::finish(acc));
@@ -318,25 +330,17 @@ __global__ void combine_kernel(double *out, const double *scratch, int64_t comps
 }
 
 cudaError_t launch_combine(bool dd, double *out_f, double *out_J, const double *scratch_f, const double *scratch_J,
-                           int64_t f_doubles, int64_t J_doubles, int chunks, cudaStream_t s) {
-  if (chunks <= 1) return cudaSuccess;
+                           int64_t f_doubles, int64_t J_doubles, int chunks, const Only &only, cudaStream_t s) {
+  if (chunks <= 1 || f_doubles + J_doubles <= 0) return cudaSuccess;
   const int threads = 256;
-  for (int pass = 0; pass < 2; pass++) {
-    double *out = pass ? out_J : out_f;
-    const double *scr = pass ? scratch_J : scratch_f;
-    const int64_t doubles = pass ? J_doubles : f_doubles;
-    const int64_t comps = dd ? doubles / 2 : doubles;
-    if (comps <= 0) continue;
-    int64_t blocks = (comps + threads - 1) / threads;
-    if (blocks > kSms * 64) blocks = kSms * 64;
-    if (dd)
-      combine_kernel<ArithDD><<<static_cast<unsigned>(blocks), threads, 0, s>>>(out, scr, comps, doubles, chunks);
-    else
-      combine_kernel<ArithF64><<<static_cast<unsigned>(blocks), threads, 0, s>>>(out, scr, comps, doubles, chunks);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  int64_t blocks = ((f_doubles + J_doubles) / (dd ? 2 : 1) + threads - 1) / threads;
+  if (blocks > kSms * 64) blocks = kSms * 64;
+  const unsigned b = static_cast<unsigned>(blocks);
+  if (dd)
+    combine_kernel<ArithDD><<<b, threads, 0, s>>>(out_f, out_J, scratch_f, scratch_J, f_doubles, J_doubles, chunks, only);
+  else
+    combine_kernel<ArithF64><<<b, threads, 0, s>>>(out_f, out_J, scratch_f, scratch_J, f_doubles, J_doubles, chunks, only);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_powers(bool dd, const PowerParams &p, cudaStream_t s) {
@@ -351,13 +355,15 @@ cudaError_t launch_powers(bool dd, const PowerParams &p, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Batch handles: each item carries its own number of monomial groups (the
-// last, partial tile of a system spreads its few points over the warp).
+// Each item with its own number of monomial groups: batch handles (the last,
+// partial tile of a system spreads its few points over the warp) and calls
+// that evaluate flagged points only.
 template <class A>
 __global__ void main_kernel_batch(const MainParams kp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   typename A::V *smem = reinterpret_cast<typename A::V *>(smem_raw) + static_cast<size_t>(warp) * kp.kslots * 32;
+  if (kp.any && *kp.any == 0) return;
   for (;;) {
     unsigned item = 0;
     if (lane == 0) item = atomicAdd(kp.counter, 1u);
@@ -407,7 +413,7 @@ cudaError_t main_occupancy(bool dd, bool batch, int warps_per_block, size_t smem
 template <class A>
 cudaError_t launch_main_t(const MainParams &p, int warps_per_block, size_t smem_bytes, int grid, cudaStream_t s) {
   const dim3 b(warps_per_block * 32);
-  if (p.single_P < 0) {
+  if (p.single_P < 0 || p.regroup) {
     main_kernel_batch<A><<<grid, b, smem_bytes, s>>>(p);
     return cudaGetLastError();
   }

@@ -43,9 +43,10 @@ __global__ void convert_coef_qd_kernel(const double *coef_qd, uint32_t *coef_blk
 __global__ void powers_qd(const PowerParams pp) {
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   uint32_t *table = reinterpret_cast<uint32_t *>(pp.table);
+  if (pp.any && *pp.any == 0) return;
   for (int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; idx < pp.total; idx += stride) {
     int n, emax, P;
-    int64_t local, pt_off, tab_off;
+    int64_t local, pt_off, tab_off, fl_off = 0;
     if (pp.single_P >= 0) {
       n = pp.single_n;
       emax = pp.single_emax;
@@ -66,8 +67,10 @@ __global__ void powers_qd(const PowerParams pp) {
       local = idx - pp.prefix[lo];
       pt_off = sd.pt_off;
       tab_off = sd.tab_off;
+      fl_off = sd.fl_off;
     }
     const int64_t v = local / P, q = local - v * P;
+    if (pp.flags && !pp.flags[fl_off + q]) continue;
     const double *xp = pp.points + (pt_off + v * P + q) * kQdDoubles;
     auto entry = [&](int e) { return table + (tab_off + (static_cast<int64_t>(e - 1) * n + v) * P + q) * kQdWords; };
     const WF x = qd::wf_from_cqd(xp);
@@ -107,13 +110,20 @@ __device__ __forceinline__ void accumulate(double *entry, int c, bool valid, con
   if (valid) qd::store_acc(p, a);
 }
 
+__device__ __forceinline__ void store_rounded(double *p, const Acc &a) {
+  double o[4];
+  qd::acc_to_qd(a, o);
+  reinterpret_cast<double2 *>(p)[0] = make_double2(o[0], o[1]);
+  reinterpret_cast<double2 *>(p)[1] = make_double2(o[2], o[3]);
+}
+
 __device__ void process_item_qd(const MainParams &kp, const Item &it, uint32_t *slots, int lane) {
   const int gp = it.gp, tile = it.tile, s = it.s, P = it.P;
   const SysDesc sd = kp.sys[s];
   const int n = sd.n;
   const int q = tile * kPointsPerWarp + (lane >> 1);
-  const bool valid = q < P;
-  const int qc = valid ? q : P - 1;
+  const bool valid = q < P && (!kp.flags || kp.flags[sd.fl_off + q]);
+  const int qc = min(q, P - 1);
   const int c = lane & 1;
   const size_t Pz = static_cast<size_t>(P);
   const int pl = gp - sd.poly0;
@@ -171,13 +181,25 @@ __device__ void process_item_qd(const MainParams &kp, const Item &it, uint32_t *
       if (j > 0) Q = qd::mul_x(Q, qd::load_wf(tel(1, v)), c);
     }
   }
-  if (valid) qd::store_acc(it.f_base + (static_cast<size_t>(sd.f_off) + static_cast<size_t>(pl) * Pz + q) * kQdDoubles + 4 * c, f);
+  if (!valid) return;
+  double *fp = it.f_base + (static_cast<size_t>(sd.f_off) + static_cast<size_t>(pl) * Pz + q) * kQdDoubles + 4 * c;
+  if (!kp.finish) {
+    qd::store_acc(fp, f);
+    return;
+  }
+  // one chunk: the sums are complete
+  store_rounded(fp, f);
+  for (int v = 0; v < n; v++) {
+    double *p = jel(v) + 4 * c;
+    store_rounded(p, qd::load_acc(p));
+  }
 }
 
 __global__ void __launch_bounds__(kWarpsPerBlockMax * 32) main_qd(const MainParams kp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t *slots = reinterpret_cast<uint32_t *>(smem_raw) + static_cast<size_t>(warp) * kp.kslots * kQdSlotWords * 32;
+  if (kp.any && *kp.any == 0) return;
   for (;;) {
     unsigned item = 0;
     if (lane == 0) item = atomicAdd(kp.counter, 1u);
@@ -193,21 +215,20 @@ __global__ void __launch_bounds__(kWarpsPerBlockMax * 32) main_qd(const MainPara
 // accumulators, rounded to a quad-double in place.  `components` covers f
 // (the first f_components) and then J.
 __global__ void finalize_qd(double *out_f, double *out_J, const double *scratch_f, const double *scratch_J,
-                            int64_t f_components, int64_t J_components, int chunks) {
+                            int64_t f_components, int64_t J_components, int chunks, Only only) {
+  if (only.any && *only.any == 0) return;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   const int64_t total = f_components + J_components;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < total; i += stride) {
     const bool isf = i < f_components;
     const int64_t j = isf ? i : i - f_components;
+    if (only.any && !only.flags[j / 2 % only.P]) continue;
     double *p = (isf ? out_f : out_J) + j * 4;
     const double *sc = isf ? scratch_f : scratch_J;
     const int64_t cs = (isf ? f_components : J_components) * 4;  // doubles between chunk copies
     Acc a = qd::load_acc(p);
     for (int c = 1; c < chunks; c++) qd::acc_add_acc(a, qd::load_acc(sc + (c - 1) * cs + j * 4));
-    double o[4];
-    qd::acc_to_qd(a, o);
-    reinterpret_cast<double2 *>(p)[0] = make_double2(o[0], o[1]);
-    reinterpret_cast<double2 *>(p)[1] = make_double2(o[2], o[3]);
+    store_rounded(p, a);
   }
 }
 
@@ -242,13 +263,14 @@ cudaError_t launch_main_qd(const MainParams &p, int warps_per_block, size_t smem
 }
 
 cudaError_t launch_finalize_qd(double *out_f, double *out_J, const double *scratch_f, const double *scratch_J,
-                               int64_t f_components, int64_t J_components, int chunks, cudaStream_t s) {
+                               int64_t f_components, int64_t J_components, int chunks, const Only &only,
+                               cudaStream_t s) {
   const int64_t total = f_components + J_components;
   if (total <= 0) return cudaSuccess;
   int64_t blocks = (total + 255) / 256;
   if (blocks > kSms * 16) blocks = kSms * 16;
   finalize_qd<<<static_cast<unsigned>(blocks), 256, 0, s>>>(out_f, out_J, scratch_f, scratch_J, f_components,
-                                                            J_components, chunks);
+                                                            J_components, chunks, only);
   return cudaGetLastError();
 }
 

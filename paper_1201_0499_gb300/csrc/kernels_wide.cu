@@ -41,9 +41,10 @@ __global__ void convert_coef_kernel(const double *coef_dd, uint32_t *coef_wide, 
 __global__ void powers_wide(const PowerParams pp) {
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   uint32_t *table = reinterpret_cast<uint32_t *>(pp.table);
+  if (pp.any && *pp.any == 0) return;
   for (int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; idx < pp.total; idx += stride) {
     int n, emax, P;
-    int64_t local, pt_off, tab_off;
+    int64_t local, pt_off, tab_off, fl_off = 0;
     if (pp.single_P >= 0) {
       n = pp.single_n;
       emax = pp.single_emax;
@@ -64,8 +65,10 @@ __global__ void powers_wide(const PowerParams pp) {
       local = idx - pp.prefix[lo];
       pt_off = sd.pt_off;
       tab_off = sd.tab_off;
+      fl_off = sd.fl_off;
     }
     const int64_t v = local / P, q = local - v * P;
+    if (pp.flags && !pp.flags[fl_off + q]) continue;
     const double *xp = pp.points + (pt_off + v * P + q) * 4;
     auto entry = [&](int e) { return table + (tab_off + (static_cast<int64_t>(e - 1) * n + v) * P + q) * kWideWords; };
     const WF x = wide::wf_from_cdd(xp[0], xp[1], xp[2], xp[3]);
@@ -111,8 +114,8 @@ __device__ void process_item_wide(const MainParams &kp, const Item &it, uint32_t
   const SysDesc sd = kp.sys[s];
   const int n = sd.n;
   const int q = tile * kPointsPerWarp + (lane >> 1);
-  const bool valid = q < P;
-  const int qc = valid ? q : P - 1;
+  const bool valid = q < P && (!kp.flags || kp.flags[sd.fl_off + q]);
+  const int qc = min(q, P - 1);
   const int c = lane & 1;
   const size_t Pz = static_cast<size_t>(P);
   const int pl = gp - sd.poly0;
@@ -261,6 +264,7 @@ __global__ void __launch_bounds__(kWarpsPerBlockMax * 32) main_wide(const MainPa
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t *slots = reinterpret_cast<uint32_t *>(smem_raw) + static_cast<size_t>(warp) * kp.kslots * kSlotWords * 32;
+  if (kp.any && *kp.any == 0) return;
   for (;;) {
     unsigned item = 0;
     if (lane == 0) item = atomicAdd(kp.counter, 1u);
