@@ -157,19 +157,17 @@ __device__ __forceinline__ void check(Num<L> &y) {
 // conversions
 // ---------------------------------------------------------------------------
 
-// Digits of floor(m / 2^sh) for a 256-bit magnitude, 0 <= sh, the quotient
-// below 2^(B L + 1).
-template <int L>
-__device__ __forceinline__ void digits_of(const qd::Mag &m, int sh, bool neg, int32_t (&d)[L]) {
+// Digits of an N-word magnitude below 2^(B L + 1), negated when neg.
+template <int L, int N>
+__device__ __forceinline__ void digits_of(const uint32_t (&x)[N], bool neg, int32_t (&d)[L]) {
   constexpr int B = Fmt<L>::B;
   constexpr int32_t kMask = (1 << B) - 1;
-  const qd::Mag x = qd::shr(m, sh);
   int32_t t = 0;
 #pragma unroll
   for (int i = 0; i < L; i++) {
     const int w = (B * i) >> 5, b = (B * i) & 31;
-    uint32_t v = x.w[w] >> b;
-    if (b != 0 && w + 1 < qd::L) v |= x.w[w + 1] << (32 - b);
+    uint32_t v = x[w] >> b;
+    if (b != 0 && w + 1 < N) v |= x[w + 1] << (32 - b);
     int32_t u = i == L - 1 ? static_cast<int32_t>(v) : static_cast<int32_t>(v) & kMask;
     if (neg) u = -u;
     t += u;
@@ -181,6 +179,50 @@ __device__ __forceinline__ void digits_of(const qd::Mag &m, int sh, bool neg, in
     }
   }
 }
+
+// A sum of NP doubles as sign and magnitude times 2^e (its leading bit found,
+// -1: zero).  Up to two parts take 128 bits, which hold more than the digits
+// of L <= 4; more take 256.
+template <int NP>
+struct Component {
+  static constexpr int N = NP <= 2 ? 4 : 8;
+  uint32_t m[N];
+  bool neg;
+  int32_t e;
+  int lead;
+  __device__ __forceinline__ explicit Component(const double *v) {
+    if constexpr (NP <= 2) {
+      double h = v[0], l = 0.0;
+      if constexpr (NP == 2) two_sum(v[0], v[1], h, l);
+      const wide::Comp c = wide::comp_from_dd(h, l);
+      m[0] = c.m.w0, m[1] = c.m.w1, m[2] = c.m.w2, m[3] = c.m.w3;
+      neg = c.s != 0u;
+      e = c.e;
+      lead = 127 - wide::clz128(c.m);
+    } else {
+      const qd::Comp c = qd::comp_from_parts<NP>(v);
+#pragma unroll
+      for (int i = 0; i < N; i++) m[i] = c.m.w[i];
+      neg = c.s != 0u;
+      e = c.e;
+      lead = 255 - qd::clz256(c.m);
+    }
+  }
+  // m 2^-s
+  __device__ __forceinline__ void shift(int s) {
+    if constexpr (NP <= 2) {
+      const wide::Mag a{m[0], m[1], m[2], m[3]}, r = s >= 0 ? wide::shr(a, s) : wide::shl(a, -s);
+      m[0] = r.w0, m[1] = r.w1, m[2] = r.w2, m[3] = r.w3;
+    } else {
+      qd::Mag a;
+#pragma unroll
+      for (int i = 0; i < N; i++) a.w[i] = m[i];
+      a = s >= 0 ? qd::shr(a, s) : qd::shl(a, -s);
+#pragma unroll
+      for (int i = 0; i < N; i++) m[i] = a.w[i];
+    }
+  }
+};
 
 // y-kind digits to balanced ones (X kind): |d_i| <= 2^(B-1) below the top.
 template <int L>
@@ -234,21 +276,18 @@ __device__ __forceinline__ Num<L> from_parts(const double *v, int t, Seen &seen)
   if (!finite) {
     seen = Seen{true, 0.0f};
   } else {
-    const qd::Comp r = qd::comp_from_parts<NP>(v), i = qd::comp_from_parts<NP>(v + NP);
-    const int zr = qd::clz256(r.m), zi = qd::clz256(i.m);
-    if (zr < 256 || zi < 256) {
+    Component<NP> r(v), i(v + NP);
+    if (r.lead >= 0 || i.lead >= 0) {
       // exponents of the leading bits
-      const int tr = r.e + 255 - zr, ti = i.e + 255 - zi;
-      const int top = zr == 256 ? ti : zi == 256 ? tr : max(tr, ti);
-      seen.bad = zr < 256 && zi < 256 && (tr - ti > kMaxSkew || ti - tr > kMaxSkew);
+      const int tr = r.e + r.lead, ti = i.e + i.lead;
+      const int top = r.lead < 0 ? ti : i.lead < 0 ? tr : max(tr, ti);
+      seen.bad = r.lead >= 0 && i.lead >= 0 && (tr - ti > kMaxSkew || ti - tr > kMaxSkew);
       // leading bit of the larger component to bit B - 2 of the top digit
       y.e = top - (B * L - 2);
-      // (a shift of the magnitude at all: its leading bit is at 250 or below,
-      // and cancelling parts may leave it lower; then the low digits are short)
-      const int sr = zr == 256 ? 0 : y.e - r.e, si = zi == 256 ? 0 : y.e - i.e;
-      const qd::Mag rm = sr < 0 ? qd::shl(r.m, -sr) : r.m, im = si < 0 ? qd::shl(i.m, -si) : i.m;
-      digits_of<L>(rm, max(sr, 0), r.s != 0u, y.re);
-      digits_of<L>(im, max(si, 0), i.s != 0u, y.im);
+      if (r.lead >= 0) r.shift(y.e - r.e);
+      if (i.lead >= 0) i.shift(y.e - i.e);
+      digits_of<L>(r.m, r.neg, y.re);
+      digits_of<L>(i.m, i.neg, y.im);
       seen.log2m = scale_modulus<L>(y, t);
       return y;
     }
@@ -270,49 +309,78 @@ __device__ __forceinline__ Num<L> as_factor(Num<L> y) {
   return y;
 }
 
-// 1 / x for a table entry x, by Newton's iteration r <- r (2 - x r) from the
-// double-precision reciprocal; each step doubles the correct bits (51, 102,
-// 204).  y kind.
+// The product of real numbers y and X (digits as above), y's scale kept.
+template <int L>
+__device__ __forceinline__ void mul_real(const int32_t (&y)[L], const int32_t (&X)[L], int32_t (&r)[L]) {
+  long long c[L];
+#pragma unroll
+  for (int k = 0; k < L; k++) {
+    c[k] = 0;
+#pragma unroll
+    for (int i = k; i < L; i++) c[k] += static_cast<long long>(X[i]) * y[k + L - 1 - i];
+  }
+  fold<L>(c, r);
+}
+
+// 1 / x for a table entry x = (a + ib) 2^(B L - 1 + e), a^2 + b^2 within a
+// factor 2 of 1: conj(x) / (a^2 + b^2), the real reciprocal by Newton's
+// iteration r <- r (2 - n r) from single precision; each step doubles the
+// correct bits (21, 42, 84, 168, 336).  y kind.  (A complex iteration takes
+// four times the multiply-adds; a double-precision start saves one step but
+// takes some 25 instructions of the FP64 pipe, 400 cycles of an SM each time.)
 template <int L>
 __device__ __forceinline__ Num<L> reciprocal(const Num<L> &X) {
   constexpr int B = Fmt<L>::B;
-  // modulus of (a + ib) within 2^(+-1/2) of 2^(B-1)
-  const double s = 1.0 / static_cast<double>(1 << B);
-  const double a = fma(static_cast<double>(X.re[L - 2]), s, static_cast<double>(X.re[L - 1]));
-  const double b = fma(static_cast<double>(X.im[L - 2]), s, static_cast<double>(X.im[L - 1]));
-  const double q = 1.0 / fma(a, a, b * b);
-  const double v[2] = {a * q, -(b * q)};
-  Seen unused;
-  // v ~ 1 / (a + ib), X = (a + ib) 2^(B (L - 1) + e)
-  Num<L> r = from_parts<L, 1>(v, B - 3, unused);
-  r.e -= B * (L - 1) + X.e;
-  constexpr int kSteps = L == 3 ? 1 : L == 4 ? 2 : 3;
-#pragma unroll 1
-  for (int k = 0; k < kSteps; k++) {
-    Num<L> u = r;
-    mul<L>(u, X);  // 1 + d, modulus near 2^(B L - 3 + ...)
-    // 2 - u: the unit sits at bit -e
-    const int bit = -u.e;
-    const int w = (bit + 1) / B, p = (bit + 1) - w * B;
-    int32_t t = 0, m = 0;
+  constexpr int32_t kMask = (1 << B) - 1;
+  int32_t n[L], r[L];
+  {
+    long long c[L];
 #pragma unroll
-    for (int i = 0; i < L; i++) {
-      t += (i == w ? (1 << p) : 0) - u.re[i];
-      m -= u.im[i];
-      if (i < L - 1) {
-        u.re[i] = t & ((1 << B) - 1);
-        t >>= B;
-        u.im[i] = m & ((1 << B) - 1);
-        m >>= B;
-      } else {
-        u.re[i] = t;
-        u.im[i] = m;
+    for (int k = 0; k < L; k++) {
+      c[k] = 0;
+#pragma unroll
+      for (int i = k; i < L; i++) {
+        c[k] += static_cast<long long>(X.re[i]) * X.re[k + L - 1 - i];
+        c[k] += static_cast<long long>(X.im[i]) * X.im[k + L - 1 - i];
       }
     }
-    const Num<L> U = as_factor<L>(u);
-    mul<L>(r, U);
+    fold<L>(c, n);  // scale 2^(B L - 1)
   }
-  return r;
+  const float f = static_cast<float>(n[L - 1]) * (1.0f / static_cast<float>(1 << (B - 1)));
+#pragma unroll
+  for (int i = 0; i < L - 1; i++) r[i] = 0;
+  r[L - 1] = __float2int_rn(__fdividef(static_cast<float>(1 << (B - 3)), f));  // scale 2^(B L - 3)
+  balance<L>(n);
+  constexpr int kSteps = L == 3 ? 2 : L == 4 ? 3 : 4;
+#pragma unroll 1
+  for (int k = 0; k < kSteps; k++) {
+    int32_t u[L], w[L];
+    mul_real<L>(r, n, u);  // 1 + d at scale 2^(B L - 3)
+    int32_t t = 0;         // 2 - u, then shifted up to scale 2^(B L - 1)
+#pragma unroll
+    for (int i = 0; i < L; i++) {
+      t += (i == L - 1 ? 1 << (B - 2) : 0) - u[i];
+      if (i < L - 1) {
+        w[i] = t & kMask;
+        t >>= B;
+      } else {
+        w[i] = t;
+      }
+    }
+    shift_digits<L>(w, 2);
+    balance<L>(w);
+    mul_real<L>(r, w, u);
+#pragma unroll
+    for (int i = 0; i < L; i++) r[i] = u[i];
+  }
+  Num<L> y;
+  int32_t minus[L];
+#pragma unroll
+  for (int i = 0; i < L; i++) minus[i] = -X.im[i];
+  mul_real<L>(r, X.re, y.re);
+  mul_real<L>(r, minus, y.im);
+  y.e = -(B * L - 1) - (B * L - 3) - X.e;
+  return y;
 }
 
 }  // namespace fx

@@ -212,6 +212,9 @@ struct NewtonParams {
   double *Jdd, *fdd;  // quad-double handles: double-double copies of the systems when not staged in shared memory
 };
 cudaError_t launch_newton(bool dd, const NewtonParams &p, cudaStream_t s);
+constexpr int kIntLuMin = 12;  // smallest system of the integer elimination (newton_int.cu)
+bool newton_int_fits(int n);
+cudaError_t launch_newton_int(const NewtonParams &p, cudaStream_t s);
 cudaError_t launch_newton_qd(const NewtonParams &p, cudaStream_t s);
 bool newton_qd_needs_scratch(int n);
 

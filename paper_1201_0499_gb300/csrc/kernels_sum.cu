@@ -504,7 +504,7 @@ __device__ __forceinline__ void own_windows(const SumParams &sp, int gp, const u
 
 template <int L, bool kTabShared>
 __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(const SumParams sp) {
-  constexpr int B = Fmt<L>::B, W = Fmt<L>::W, KC = kComp<L>;
+  constexpr int W = Fmt<L>::W, KC = kComp<L>;
   constexpr int kw = Fmt<L>::kKeep / 32, kb = Fmt<L>::kKeep % 32;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int32_t ebuf[3][kSumPointsMax];

@@ -206,6 +206,7 @@ bool newton_qd_needs_scratch(int n) { return smem_lu_bytes<CDD>(n) > kSmemLuMax;
 
 cudaError_t launch_newton(bool dd, const NewtonParams &p, cudaStream_t s) {
   if (p.P <= 0 || p.n <= 0) return cudaSuccess;
+  if (dd && newton_int_fits(p.n)) return launch_newton_int(p, s);
   return dd ? launch_newton_t<CDD>(p, s) : launch_newton_t<C64>(p, s);
 }
 
