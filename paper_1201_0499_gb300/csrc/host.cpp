@@ -131,11 +131,11 @@ struct polyeval {
   int sum_L = 0;  // digits per number; 0: not available, the general kernels evaluate every call
   struct SumLaunch {  // per log2 of the points of a tile
     bool ok = false, tab_shared = false;
-    int threads = 0, blocks = 0;  // blocks: resident on the whole device
+    int threads = 0, values = 1, blocks = 0;  // blocks: resident on the whole device
     size_t smem = 0;
   };
   SumLaunch sum_launch[3];
-  int sum_batch_lg = 0;
+  int sum_lg = 0;  // points per tile (log2) of batches and of calls with many points
   std::vector<pe::SumSys> sum_sys;
   int64_t sum_power_total = 0, sum_items_n = 0;  // batch
   DeviceBuf sum_fac_ptr, sum_fac, sum_coef, sum_polys, sum_act, sum_bits, sum_hit_ptr, sum_hits, sum_sysd, sum_prefix, sum_items;
@@ -706,41 +706,49 @@ int setup_sum(polyeval *h, const Compiled &c) {
   // A tile takes a multiple of kSumBlock monomials at a time.
   const size_t room = static_cast<size_t>(optin) - 256;  // 256: the kernel's static shared memory
   if (pe::prepare_sum(L, room) != cudaSuccess) return PE_ECUDA;
-  bool any = false;
   for (int lg = 0; lg < kSumTiles; lg++) {
     polyeval::SumLaunch &sl = h->sum_launch[lg];
     int t = std::max(64, pe::kSumBlock << lg);
     while (t < pe::kSumThreadsMax && (t >> lg) < std::max(m_max, act_most)) t *= 2;
     sl.threads = h->batch ? pe::kSumThreadsMax : t;
     for (int shared = 1; shared >= 0 && !sl.ok; shared--) {
-      size_t most = 0;
-      for (int s = 0; s < S; s++)
-        most = std::max(most, pe::sum_smem_bytes(L, h->sys[s].n, h->sum_sys[s].act_max, h->sys[s].emax, lg, sl.threads,
-                                                 shared != 0));
-      if (most > room) continue;
-      int b = 0;
-      if (pe::sum_occupancy(L, shared != 0, sl.threads, most, &b) != cudaSuccess) return PE_ECUDA;
-      if (b < 1) continue;
-      sl.ok = true;
-      sl.tab_shared = shared != 0;
-      sl.smem = most;
-      sl.blocks = b * h->sms;
+      // two monomials per thread and chunk halve the barriers: where a tile
+      // has more than one chunk and as many blocks stay resident
+      for (int values = 1; values <= ((sl.threads >> lg) < m_max ? 2 : 1); values++) {
+        size_t most = 0;
+        for (int s = 0; s < S; s++)
+          most = std::max(most, pe::sum_smem_bytes(L, h->sys[s].n, h->sum_sys[s].act_max, h->sys[s].emax, lg, sl.threads,
+                                                   values, shared != 0));
+        if (most > room) continue;
+        int b = 0;
+        if (pe::sum_occupancy(L, shared != 0, sl.threads, most, &b) != cudaSuccess) return PE_ECUDA;
+        if (b < 1 || (sl.ok && b * h->sms < sl.blocks)) continue;
+        sl.ok = true;
+        sl.tab_shared = shared != 0;
+        sl.values = values;
+        sl.smem = most;
+        sl.blocks = b * h->sms;
+      }
     }
-    any = any || sl.ok;
   }
-  if (!any) return PE_OK;
-  // batch: the points per tile of every system (one launch)
-  if (h->batch) {
-    int lg = kSumTiles - 1;
-    while (lg > 0 && !h->sum_launch[lg].tab_shared) lg--;
-    if (!h->sum_launch[lg].tab_shared) {
-      lg = kSumTiles - 1;
-      while (lg > 0 && !h->sum_launch[lg].ok) lg--;
-      if (!h->sum_launch[lg].ok) return PE_OK;
+  // The points per tile of a call with many: the launch with the most
+  // resident warps, tables in shared memory before tables in global memory,
+  // more points before fewer.  Large tables decide it: n = 128, e = 4 in
+  // double-double (37 KiB of table per 2 points) 40.4 ms with 2 points and 3
+  // blocks per SM, 44.6 ms with 4 points and 2 blocks; n = 32, e = 5, where
+  // both take 3 blocks, 277.6 and 278.5 us (1024 points each).
+  h->sum_lg = -1;
+  for (int lg = kSumTiles - 1; lg >= 0; lg--) {
+    const polyeval::SumLaunch &sl = h->sum_launch[lg];
+    if (!sl.ok) continue;
+    if (h->sum_lg >= 0) {
+      const polyeval::SumLaunch &best = h->sum_launch[h->sum_lg];
+      if (best.tab_shared != sl.tab_shared ? best.tab_shared : best.blocks * best.threads >= sl.blocks * sl.threads) continue;
     }
-    h->sum_batch_lg = lg;
-    for (int s = 0; s < S; s++) h->sum_sys[s].lg = lg;
+    h->sum_lg = lg;
   }
+  if (h->sum_lg < 0) return PE_OK;
+  for (int s = 0; s < S; s++) h->sum_sys[s].lg = h->sum_lg;  // batches: one launch
   // tables and flags
   int64_t fl = 0;
   size_t tb = 0;
@@ -829,9 +837,9 @@ int setup_sum(polyeval *h, const Compiled &c) {
     };
     for (size_t gp = 0; gp < c.poly_sys.size(); gp++) {
       const SysDesc &d = h->sys[c.poly_sys[gp]];
-      total += cost_of(gp) * static_cast<double>((d.P + (1 << h->sum_batch_lg) - 1) >> h->sum_batch_lg);
+      total += cost_of(gp) * static_cast<double>((d.P + (1 << h->sum_lg) - 1) >> h->sum_lg);
     }
-    const double share = total / (16.0 * h->sum_launch[h->sum_batch_lg].blocks);
+    const double share = total / (16.0 * h->sum_launch[h->sum_lg].blocks);
     for (int s = 0; s < S; s++) {
       const SysDesc &d = h->sys[s];
       const int lg = h->sum_sys[s].lg;
@@ -881,19 +889,13 @@ int setup_sum(polyeval *h, const Compiled &c) {
   return PE_OK;
 }
 
-// Points per tile (log2) of a single-system call: 8 points, which one
-// 128-byte row of the table holds, or as few as it takes to give every SM a
-// (polynomial, tile) item.
+// Points per tile (log2) of a single-system call: the handle's choice, or as
+// few as it takes to give every SM a (polynomial, tile) item.
 int sum_tile_log2(const polyeval *h, int64_t P) {
   const int64_t N = h->sys[0].N;
-  int best = -1;
-  for (int lg = kSumTiles - 1; lg >= 0; lg--) {
-    if (!h->sum_launch[lg].ok) continue;
-    if (best >= 0 && (h->sum_launch[best].tab_shared || !h->sum_launch[lg].tab_shared) &&
-        N * ((P + (1 << best) - 1) >> best) >= h->sms)
-      break;
-    best = lg;
-  }
+  int best = h->sum_lg;
+  for (int lg = best - 1; lg >= 0 && N * ((P + (1 << best) - 1) >> best) < h->sms; lg--)
+    if (h->sum_launch[lg].ok && (h->sum_launch[lg].tab_shared || !h->sum_launch[best].tab_shared)) best = lg;
   return best;
 }
 
@@ -923,7 +925,7 @@ int run_sum(polyeval *h, const void *points, int64_t P, void *out_f, void *out_J
   sp.counter = reinterpret_cast<unsigned *>(ctl);
   sp.any = reinterpret_cast<int32_t *>(ctl + 4);
   sp.flags = ctl + kCtlFlags;
-  int lg = h->sum_batch_lg;
+  int lg = h->sum_lg;
   if (P >= 0) {
     const SysDesc &d = h->sys[0];
     lg = sum_tile_log2(h, P);
@@ -945,6 +947,7 @@ int run_sum(polyeval *h, const void *points, int64_t P, void *out_f, void *out_J
     sp.n_items = h->sum_items_n;
   }
   const polyeval::SumLaunch &sl = h->sum_launch[lg];
+  sp.values = sl.values;
   const size_t flagged = P >= 0 ? static_cast<size_t>(P) : static_cast<size_t>(h->sum_points);
   if (cudaMemsetAsync(h->sum_ctl.p, 0, kCtlFlags + flagged, s) != cudaSuccess) return PE_ECUDA;
   if (pe::launch_sum_powers(h->sum_L, sp, s) != cudaSuccess) return PE_ECUDA;

@@ -108,6 +108,7 @@ struct PowerParams {
 // digits: L = 3 (double), 4 (double-double), 8 (quad-double).
 constexpr int kSumThreadsMax = 256;
 constexpr int kSumPointsMax = 4;   // points per tile: 1, 2 or 4
+constexpr int kSumParts = 4;       // sums that f is split into
 constexpr int kSumBlock = 64;      // monomials per block of the addition lists (their entries hold 6 bits of it)
 
 // One compiled system.
@@ -153,6 +154,7 @@ struct SumParams {
   int32_t count;
   int32_t single_P;         // >= 0: single-system handle
   int32_t single_lg;
+  int32_t values;           // monomials per thread and chunk (1 or 2)
   int32_t groups, group_polys;  // single: runs of polynomials per tile, polynomials per run
   int32_t n_polys_total;
   unsigned *counter;        // work counter and ...
@@ -172,7 +174,7 @@ __host__ __device__ constexpr size_t sum_tab_bytes(int L, int n, int levels, int
 __host__ __device__ constexpr size_t sum_blob_bytes(int L, int n, int levels, int lg) {
   return sum_tab_bytes(L, n, levels, lg) + sum_tab_bytes(L, n, 1, lg);
 }
-size_t sum_smem_bytes(int L, int n, int act_max, int levels, int lg, int threads, bool tab_shared);
+size_t sum_smem_bytes(int L, int n, int act_max, int levels, int lg, int threads, int values, bool tab_shared);
 int sum_head_bits_min(int L);
 cudaError_t prepare_sum(int L, size_t smem);
 cudaError_t sum_occupancy(int L, bool tab_shared, int threads, size_t smem, int *blocks);

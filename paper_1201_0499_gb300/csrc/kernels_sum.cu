@@ -19,8 +19,7 @@
 // a run of polynomials.  The tile's power table (digits.cuh) is copied to
 // shared memory once.  For each polynomial, chunks of monomials:
 //   A  one thread per (monomial, point) multiplies its k factors in
-//      registers; eight lanes of neighbouring points read 128 contiguous
-//      bytes of shared memory;
+//      registers (two monomials where shared memory has room for the values);
 //   -  the block agrees on the largest exponent per point, and every value is
 //      stored as a W-word two's complement integer below it (the window);
 //      (a word per sum keeps the or of its terms' bits from kKeep up: none set
@@ -417,16 +416,16 @@ __device__ __forceinline__ int value_top(const Num<L> &y) {
   return max(e, fx::kZeroExp);
 }
 
-// Component c of a value as a window integer below 2^E: bit 0 at exponent
-// E - (32 W - 1 - hb).
+// A component's digits (exponent e) as a window integer below 2^E: bit 0 at
+// exponent E - (32 W - 1 - hb).
 template <int L>
-__device__ __forceinline__ void to_window(const Num<L> &y, int c, int E, int hb, uint32_t (&z)[Fmt<L>::W]) {
+__device__ __forceinline__ void to_window(const int32_t (&d)[L], int32_t e, int E, int hb, uint32_t (&z)[Fmt<L>::W]) {
   constexpr int W = Fmt<L>::W, NW = kPackWords<L>;
   uint32_t p[NW];
-  pack_digits<L, NW>(c ? y.im : y.re, p);
+  pack_digits<L, NW>(d, p);
 #pragma unroll
   for (int i = 0; i < W; i++) z[i] = i < W - NW ? 0u : p[i - (W - NW)];
-  sar_words<W>(z, max(E - y.e - 32 * NW + 1 + hb, 0));
+  sar_words<W>(z, max(E - e - 32 * NW + 1 + hb, 0));
 }
 
 // One entry of J: the sums of its components (window integers, exponent of
@@ -490,9 +489,9 @@ __device__ __forceinline__ void own_windows(const SumParams &sp, int gp, const u
           E = e;
         }
         uint32_t z[W];
-        to_window<L>(y, 0, E, hb, z);
+        to_window<L>(y.re, y.e, E, hb, z);
         for (unsigned a = h / kSumBlock; a > 0; a--) add_words<W>(zr, z);
-        to_window<L>(y, 1, E, hb, z);
+        to_window<L>(y.im, y.e, E, hb, z);
         for (unsigned a = h / kSumBlock; a > 0; a--) add_words<W>(zi, z);
       }
     }
@@ -536,10 +535,10 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
     const size_t tab_bytes = sum_tab_bytes(L, n, levels, lg);
     const size_t exp_off = static_cast<size_t>(levels) * n * kParts<L> * 16 << lg;
     // shared memory: values first (their place does not depend on the system)
-    const int vrows = 2 * NT;
+    const int vrows = 2 * NT * sp.values;
     int4 *vq = reinterpret_cast<int4 *>(smem);
     int32_t *vr = reinterpret_cast<int32_t *>(vq + Win<L>::Q * vrows);
-    const int arows = 2 * ss.act_max << lg;
+    const int arows = 2 * (ss.act_max + kSumParts) << lg;
     int4 *aq = reinterpret_cast<int4 *>(smem + static_cast<size_t>(vrows) * W * 4);
     int32_t *ar = reinterpret_cast<int32_t *>(aq + Win<L>::Q * arows);
     uint32_t *am = reinterpret_cast<uint32_t *>(ar + Win<L>::R * arows);
@@ -561,7 +560,7 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
       const int t0 = sp.poly_ptr[gp], t1 = sp.poly_ptr[gp + 1];
       const int pl = gp - sd.poly0;
       const SumPoly sy = sp.polys[gp];
-      const int tasks = 2 * sy.act_n;
+      const int tasks = 2 * sy.act_n, all = tasks + 2 * kSumParts;
       double *Jp = sp.out_J + (static_cast<size_t>(sd.J_off) + static_cast<size_t>(pl) * n * P + qg) * 2 * KC;
       // entries of variables that do not occur in the polynomial
       if (sy.act_n < n && valid) {
@@ -573,7 +572,7 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
         }
       }
       // sums to zero; no exponent yet
-      for (int u = sub; u < tasks; u += subs) {
+      for (int u = sub; u < all; u += subs) {
         uint32_t z[W];
 #pragma unroll
         for (int i = 0; i < W; i++) z[i] = 0u;
@@ -581,48 +580,54 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
         store_window<L>(aq, ar, arows, row, z);
         am[row] = 0u;
       }
-      uint32_t fa[2][W];  // this thread's part of f
-#pragma unroll
-      for (int i = 0; i < W; i++) fa[0][i] = fa[1][i] = 0u;
       if (tid < 3 * TP) ebuf[tid >> lg][q] = fx::kZeroExp;
       __syncthreads();
       int eb = 0;  // ebuf of this chunk
-      for (int tb = t0; tb < t1; tb += subs) {
-        // A: the value of monomial tb + sub at point q
-        const int t = tb + sub;
-        const bool has = t < t1;
-        Num<L> y;
-        int et = fx::kZeroExp;
-        if (has) {
-          y = monomial_value<L>(sp, t, tab, exps, lg, q);
-          et = value_top<L>(y);
+      const int chunk = subs * sp.values;
+      for (int tb = t0; tb < t1; tb += chunk) {
+        // A: the values of monomials tb + sub, tb + sub + subs at point q, their
+        // digits to the places of their window integers
+        int em = fx::kZeroExp;
+        for (int x = 0; x < sp.values; x++) {
+          const int tl = x * subs + sub;
+          if (tb + tl >= t1) break;
+          const Num<L> y = monomial_value<L>(sp, tb + tl, tab, exps, lg, q);
+          em = max(em, value_top<L>(y));
+          uint32_t z[W];
+#pragma unroll
+          for (int i = 0; i < W; i++) z[i] = i < L ? static_cast<uint32_t>(y.re[i]) : static_cast<uint32_t>(y.e);
+          store_window<L>(vq, vr, vrows, ((2 * tl) << lg) + q, z);
+#pragma unroll
+          for (int i = 0; i < L; i++) z[i] = static_cast<uint32_t>(y.im[i]);
+          store_window<L>(vq, vr, vrows, ((2 * tl + 1) << lg) + q, z);
         }
-        int em = et;
         for (int d = TP; d < 32; d <<= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, d));
         if (lane < TP) atomicMax(&ebuf[eb][q], em);
         __syncthreads();
         const int E = ebuf[eb][q];
         const int prev = eb == 0 ? 2 : eb - 1, nxt = eb == 2 ? 0 : eb + 1;
         const int grown = tb == t0 ? 0 : E - ebuf[prev][q];
-        if (grown > 0) {
-          sar_words<W>(fa[0], grown);
-          sar_words<W>(fa[1], grown);
-        }
-        if (has) {
+        for (int x = 0; x < sp.values; x++) {
+          const int tl = x * subs + sub;
+          if (tb + tl >= t1) break;
 #pragma unroll
           for (int c = 0; c < 2; c++) {
             uint32_t z[W];
-            to_window<L>(y, c, E, hb, z);
-            store_window<L>(vq, vr, vrows, ((2 * sub + c) << lg) + q, z);
-            add_words<W>(fa[c], z);
+            int32_t d[L];
+            load_window<L>(vq, vr, vrows, ((2 * tl + c) << lg) + q, z);
+#pragma unroll
+            for (int i = 0; i < L; i++) d[i] = static_cast<int32_t>(z[i]);
+            to_window<L>(d, static_cast<int32_t>(z[L]), E, hb, z);
+            store_window<L>(vq, vr, vrows, ((2 * tl + c) << lg) + q, z);
           }
         }
         if (tid < TP) ebuf[nxt][q] = E;
         __syncthreads();
-        // B: the sums of active variable u >> 1, component u & 1 at point q
+        // B: the sums of active variable u >> 1, component u & 1 at point q, and
+        // after the variables the parts of f
         const int b0 = (tb - t0) / kSumBlock;
-        const int b1 = min((tb - t0 + subs) / kSumBlock, (t1 - t0 + kSumBlock - 1) / kSumBlock);
-        for (int u = sub; u < tasks; u += subs) {
+        const int b1 = min((tb - t0 + chunk) / kSumBlock, (t1 - t0 + kSumBlock - 1) / kSumBlock);
+        for (int u = sub; u < all; u += subs) {
           const int row = (u << lg) + q, c = u & 1;
           uint32_t a[W], odd[W - 1];
           uint32_t m = am[row];
@@ -632,6 +637,21 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
           if (grown > 0) {
             sar_words<W>(a, grown);
             m >>= min(grown, 31);
+          }
+          if (u >= tasks) {
+            constexpr int len = kSumBlock / kSumParts;
+            for (int b = b0; b < b1; b++) {
+              const int tl = (b - b0) * kSumBlock + ((u - tasks) >> 1) * len;
+              const int count = min(len, t1 - tb - tl);
+#pragma unroll 4
+              for (int k = 0; k < count; k++) {
+                uint32_t z[W];
+                load_window<L>(vq, vr, vrows, ((2 * (tl + k) + c) << lg) + q, z);
+                add_words<W>(a, z);
+              }
+            }
+            store_window<L>(aq, ar, arows, row, a);
+            continue;
           }
           for (int b = b0; b < b1; b++) {
             const int32_t *hq = sp.hit_ptr + sy.hit_off + static_cast<int64_t>(b) * (sy.act_n + 1) + (u >> 1);
@@ -670,21 +690,6 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
         eb = nxt;
         __syncthreads();
       }
-      // f: over the threads of a point, by warps, then over the warps
-      for (int d = TP; d < 32; d <<= 1) {
-#pragma unroll
-        for (int c = 0; c < 2; c++) {
-          uint32_t z[W];
-#pragma unroll
-          for (int i = 0; i < W; i++) z[i] = __shfl_xor_sync(0xffffffffu, fa[c][i], d);
-          add_words<W>(fa[c], z);
-        }
-      }
-      if (lane < TP) {
-        store_window<L>(vq, vr, vrows, ((2 * (tid >> 5)) << lg) + q, fa[0]);
-        store_window<L>(vq, vr, vrows, ((2 * (tid >> 5) + 1) << lg) + q, fa[1]);
-      }
-      __syncthreads();
       // outputs
       const int32_t ep = ebuf[eb][q] - (32 * W - 1 - hb);
       const unsigned char *ib = blob + tab_bytes;
@@ -710,9 +715,9 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
         const int c = subs - 1 - sub;
         if (c < 2) {
           uint32_t z[W], a[W];
-          load_window<L>(vq, vr, vrows, (c << lg) + q, z);
-          for (int k = 1; k < NT / 32; k++) {
-            load_window<L>(vq, vr, vrows, ((2 * k + c) << lg) + q, a);
+          load_window<L>(aq, ar, arows, ((tasks + c) << lg) + q, z);
+          for (int k = 1; k < kSumParts; k++) {
+            load_window<L>(aq, ar, arows, ((tasks + 2 * k + c) << lg) + q, a);
             add_words<W>(z, a);
           }
           store_sum<L>(sp.out_f + (static_cast<size_t>(sd.f_off) + static_cast<size_t>(pl) * P + qg) * 2 * KC + c * KC, z, ep);
@@ -752,10 +757,10 @@ cudaError_t occupancy_t(bool tab_shared, int threads, size_t smem, int *blocks) 
 
 }  // namespace
 
-size_t sum_smem_bytes(int L, int n, int act_max, int levels, int lg, int threads, bool tab_shared) {
+size_t sum_smem_bytes(int L, int n, int act_max, int levels, int lg, int threads, int values, bool tab_shared) {
   const size_t W = L == 3 ? Fmt<3>::W : L == 4 ? Fmt<4>::W : Fmt<8>::W;
-  const size_t acc = (static_cast<size_t>(2) * act_max << lg) * (W * 4 + 4);
-  return static_cast<size_t>(2) * threads * W * 4 + ((acc + 15) & ~size_t{15}) +
+  const size_t acc = (static_cast<size_t>(2) * (act_max + kSumParts) << lg) * (W * 4 + 4);
+  return static_cast<size_t>(2) * threads * values * W * 4 + ((acc + 15) & ~size_t{15}) +
          (tab_shared ? sum_tab_bytes(L, n, levels, lg) : 0);
 }
 
