@@ -61,6 +61,11 @@ struct CDD {
     return CDD{dd{__shfl_xor_sync(mask, re.h, d), __shfl_xor_sync(mask, re.l, d)},
                dd{__shfl_xor_sync(mask, im.h, d), __shfl_xor_sync(mask, im.l, d)}};
   }
+  // the value of lane `from` of each segment of `width` lanes
+  __device__ CDD shfl(unsigned mask, int from, int width) const {
+    return CDD{dd{__shfl_sync(mask, re.h, from, width), __shfl_sync(mask, re.l, from, width)},
+               dd{__shfl_sync(mask, im.h, from, width), __shfl_sync(mask, im.l, from, width)}};
+  }
 };
 
 // complex double
@@ -94,6 +99,9 @@ struct C64 {
   }
   __device__ C64 shfl_xor(unsigned mask, int d) const {
     return C64{__shfl_xor_sync(mask, re, d), __shfl_xor_sync(mask, im, d)};
+  }
+  __device__ C64 shfl(unsigned mask, int from, int width) const {
+    return C64{__shfl_sync(mask, re, from, width), __shfl_sync(mask, im, from, width)};
   }
 };
 

@@ -90,30 +90,42 @@ struct Lanes {
 // Lanes per point for an n x n system.
 __host__ __device__ constexpr int lanes_for(int n) { return n <= 4 ? 4 : n <= 8 ? 8 : n <= 16 ? 16 : 32; }
 
+// A squared modulus as an integer of the same order: the bits of the double
+// (not negative), zero for NaN, which never is the pivot.  Comparisons of
+// doubles would take the FP64 pipe.
+__device__ __forceinline__ unsigned long long modulus_key(double m) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(m));
+  return b > 0x7ff0000000000000ULL ? 0ULL : b;
+}
+
 // Returns true (uniform over the segment) when a pivot column is exactly
 // zero; b is then left partly eliminated.
 template <class C, class V, int S>
 __device__ bool lu_solve(const V &v, const Lanes<S> g) {
   const int n = v.n, lane = g.lane;
+  // the reciprocal of pivot k stays with lane k for the back substitution
+  // (about 20 instructions of the FP64 pipe against 4 or 8 shuffles)
+  const bool keep = n <= S;
+  C kept = C::zero();
   for (int k = 0; k < n; k++) {
-    double best = -1.0;
+    unsigned long long best = 0;
     int piv = n;
     for (int i = k + lane; i < n; i += S) {
-      const double m = C::load(v.Jel(i, k)).norm2_hi();  // the modulus squared: same order, no square root
+      const unsigned long long m = modulus_key(C::load(v.Jel(i, k)).norm2_hi());  // squared: same order, no square root
       if (m > best) {
         best = m;
         piv = i;
       }
     }
     for (int d = S / 2; d > 0; d >>= 1) {
-      const double ob = __shfl_xor_sync(g.mask, best, d);
+      const unsigned long long ob = __shfl_xor_sync(g.mask, best, d);
       const int op = __shfl_xor_sync(g.mask, piv, d);
       if (ob > best || (ob == best && op < piv)) {
         best = ob;
         piv = op;
       }
     }
-    if (!(best > 0.0)) return true;  // uniform over the segment
+    if (best == 0) return true;  // uniform over the segment
     if (piv != k) {
       for (int j = k + lane; j < n; j += S) {
         const C a = C::load(v.Jel(k, j)), c = C::load(v.Jel(piv, j));
@@ -129,6 +141,7 @@ __device__ bool lu_solve(const V &v, const Lanes<S> g) {
     }
     // multipliers l_i = J[i][k] / J[k][k] and the right-hand side
     const C inv = C::recip(C::load(v.Jel(k, k)));
+    if (keep && lane == k) kept = inv;
     const C bk = C::load(v.bel(k));
     for (int i = k + 1 + lane; i < n; i += S) {
       const C l = C::mul(C::load(v.Jel(i, k)), inv);
@@ -159,7 +172,7 @@ __device__ bool lu_solve(const V &v, const Lanes<S> g) {
   // lane, which costs the FP64 pipe no more than one), then the lanes over
   // the rows r < i take x_i out of y_r
   for (int i = n - 1; i >= 0; i--) {
-    const C xi = C::mul(C::load(v.bel(i)), C::recip(C::load(v.Jel(i, i))));
+    const C xi = C::mul(C::load(v.bel(i)), keep ? kept.shfl(g.mask, i, S) : C::recip(C::load(v.Jel(i, i))));
     g.sync();
     if (lane == 0) xi.store(v.bel(i));
     for (int r = lane; r < i; r += S) C::sub_mul(C::load(v.bel(r)), C::load(v.Jel(r, i)), xi).store(v.bel(r));
