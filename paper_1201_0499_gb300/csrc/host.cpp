@@ -130,15 +130,16 @@ struct polyeval {
   // evaluation from the monomials' values (kernels_sum.cu)
   int sum_L = 0;  // digits per number; 0: not available, the general kernels evaluate every call
   struct SumLaunch {  // per log2 of the points of a tile
-    bool ok = false, tab_shared = false;
+    bool ok = false, tab_shared = false, one = false;
     int threads = 0, values = 1, blocks = 0;  // blocks: resident on the whole device
     size_t smem = 0;
   };
   SumLaunch sum_launch[3];
+  double sum_products = 0.0;  // products per point of the system (single)
   int sum_lg = 0;  // points per tile (log2) of batches and of calls with many points
   std::vector<pe::SumSys> sum_sys;
   int64_t sum_power_total = 0, sum_items_n = 0;  // batch
-  DeviceBuf sum_fac_ptr, sum_fac, sum_coef, sum_polys, sum_act, sum_bits, sum_hit_ptr, sum_hits, sum_sysd, sum_prefix, sum_items;
+  DeviceBuf sum_fac, sum_coef, sum_polys, sum_act, sum_bits, sum_hit_ptr, sum_hits, sum_sysd, sum_prefix, sum_items;
   DeviceBuf sum_table, sum_ctl;  // sum_ctl: two work counters, whether any point is flagged, the points' flags
   int64_t sum_points = 0;        // flags
   // timing of the main kernel
@@ -705,7 +706,7 @@ int setup_sum(polyeval *h, const Compiled &c) {
   // launches: points per tile, threads, table in shared memory where it fits.
   // A tile takes a multiple of kSumBlock monomials at a time.
   const size_t room = static_cast<size_t>(optin) - 256;  // 256: the kernel's static shared memory
-  if (pe::prepare_sum(L, room) != cudaSuccess) return PE_ECUDA;
+  if (pe::prepare_sum(L, h->batch, room) != cudaSuccess) return PE_ECUDA;
   for (int lg = 0; lg < kSumTiles; lg++) {
     polyeval::SumLaunch &sl = h->sum_launch[lg];
     int t = std::max(64, pe::kSumBlock << lg);
@@ -716,16 +717,18 @@ int setup_sum(polyeval *h, const Compiled &c) {
       // has more than one chunk and as many blocks stay resident
       for (int values = 1; values <= ((sl.threads >> lg) < m_max ? 2 : 1); values++) {
         size_t most = 0;
+        const bool one = (sl.threads >> lg) * values >= m_max;  // one chunk: no sums in shared memory
         for (int s = 0; s < S; s++)
           most = std::max(most, pe::sum_smem_bytes(L, h->sys[s].n, h->sum_sys[s].act_max, h->sys[s].emax, lg, sl.threads,
-                                                   values, shared != 0));
+                                                   values, one, shared != 0));
         if (most > room) continue;
         int b = 0;
-        if (pe::sum_occupancy(L, shared != 0, sl.threads, most, &b) != cudaSuccess) return PE_ECUDA;
+        if (pe::sum_occupancy(L, h->batch, one, shared != 0, sl.threads, most, &b) != cudaSuccess) return PE_ECUDA;
         if (b < 1 || (sl.ok && b * h->sms < sl.blocks)) continue;
         sl.ok = true;
         sl.tab_shared = shared != 0;
         sl.values = values;
+        sl.one = one;
         sl.smem = most;
         sl.blocks = b * h->sms;
       }
@@ -748,7 +751,6 @@ int setup_sum(polyeval *h, const Compiled &c) {
     h->sum_lg = lg;
   }
   if (h->sum_lg < 0) return PE_OK;
-  for (int s = 0; s < S; s++) h->sum_sys[s].lg = h->sum_lg;  // batches: one launch
   // tables and flags
   int64_t fl = 0;
   size_t tb = 0;
@@ -762,7 +764,7 @@ int setup_sum(polyeval *h, const Compiled &c) {
     ss.tab_off = static_cast<int64_t>(tb);
     size_t most = 0;
     for (int lg = 0; lg < kSumTiles; lg++) {
-      if (h->batch ? lg != ss.lg : !h->sum_launch[lg].ok) continue;
+      if (h->batch ? lg != h->sum_lg : !h->sum_launch[lg].ok) continue;
       const int64_t tiles = (P + (1 << lg) - 1) >> lg;
       most = std::max(most, static_cast<size_t>(tiles) * pe::sum_blob_bytes(L, d.n, d.emax, lg));
       if (h->batch) prefix.push_back(prefix.back() + static_cast<int64_t>(d.n) * (tiles << lg));
@@ -839,10 +841,10 @@ int setup_sum(polyeval *h, const Compiled &c) {
       const SysDesc &d = h->sys[c.poly_sys[gp]];
       total += cost_of(gp) * static_cast<double>((d.P + (1 << h->sum_lg) - 1) >> h->sum_lg);
     }
-    const double share = total / (16.0 * h->sum_launch[h->sum_lg].blocks);
+    const double share = total / (32.0 * h->sum_launch[h->sum_lg].blocks);
     for (int s = 0; s < S; s++) {
       const SysDesc &d = h->sys[s];
-      const int lg = h->sum_sys[s].lg;
+      const int lg = h->sum_lg;
       const int32_t tiles = (d.P + (1 << lg) - 1) >> lg;
       for (int32_t p = 0; p < d.N;) {
         Run r{d.poly0 + p, 0, 0, s, 0.0};
@@ -865,15 +867,15 @@ int setup_sum(polyeval *h, const Compiled &c) {
   }
   // a device that cannot hold the extra buffers evaluates with the general
   // kernels
-  DeviceBuf ord, co;
+  DeviceBuf ord, co, fp;
   int rc;
-  if ((rc = h->sum_fac_ptr.upload(fac_ptr)) || (rc = h->sum_fac.upload(fac)) || (rc = h->sum_polys.upload(sp)) || (rc = h->sum_act.upload(act)) || (rc = h->sum_bits.upload(bits)) ||
+  if ((rc = fp.upload(fac_ptr)) || (rc = h->sum_fac.upload(fac)) || (rc = h->sum_polys.upload(sp)) || (rc = h->sum_act.upload(act)) || (rc = h->sum_bits.upload(bits)) ||
       (rc = h->sum_hit_ptr.upload(hit_ptr)) || (rc = h->sum_hits.upload(hits)) || (rc = h->sum_sysd.upload(h->sum_sys)) ||
       (rc = h->sum_prefix.upload(prefix)) || (rc = h->sum_items.upload(words)) || (rc = ord.upload(order)) ||
       (rc = co.upload(c.coef)) ||
-      (rc = h->sum_coef.alloc(static_cast<size_t>(M) * 4 * (L == 3 ? 8 : L == 4 ? 12 : 20))) ||
+      (rc = h->sum_coef.alloc(static_cast<size_t>(M) * 4 * (L == 8 ? 20 : 12))) ||
       (rc = h->sum_table.alloc(tb)) || (rc = h->sum_ctl.alloc(kCtlFlags + static_cast<size_t>(fl)))) {
-    for (DeviceBuf *b : {&h->sum_fac_ptr, &h->sum_fac, &h->sum_polys, &h->sum_act, &h->sum_bits, &h->sum_hit_ptr, &h->sum_hits, &h->sum_sysd,
+    for (DeviceBuf *b : {&h->sum_fac, &h->sum_polys, &h->sum_act, &h->sum_bits, &h->sum_hit_ptr, &h->sum_hits, &h->sum_sysd,
                          &h->sum_prefix, &h->sum_items, &h->sum_coef, &h->sum_table, &h->sum_ctl})
       b->alloc(0);
     return rc == PE_ENOMEM ? PE_OK : rc;
@@ -881,10 +883,12 @@ int setup_sum(polyeval *h, const Compiled &c) {
   if (cudaMemcpy(h->sysd.p, h->sys.data(), h->sys.size() * sizeof(SysDesc), cudaMemcpyHostToDevice) != cudaSuccess)
     return PE_ECUDA;  // the flags' offsets
   if (pe::convert_coef_sum(L, static_cast<const double *>(co.p), static_cast<const int32_t *>(ord.p),
+                           static_cast<const int32_t *>(fp.p), static_cast<const uint32_t *>(h->sum_fac.p),
                            static_cast<int32_t *>(h->sum_coef.p), M, nullptr) != cudaSuccess ||
       cudaDeviceSynchronize() != cudaSuccess)
     return PE_ECUDA;
   h->sum_points = fl;
+  h->sum_products = static_cast<double>(c.var.size());
   h->sum_L = L;
   return PE_OK;
 }
@@ -903,7 +907,6 @@ int sum_tile_log2(const polyeval *h, int64_t P) {
 int run_sum(polyeval *h, const void *points, int64_t P, void *out_f, void *out_J, cudaEvent_t e0, cudaStream_t s) {
   pe::SumParams sp{};
   sp.poly_ptr = static_cast<const int32_t *>(h->poly_ptr.p);
-  sp.fac_ptr = static_cast<const int32_t *>(h->sum_fac_ptr.p);
   sp.fac = static_cast<const uint32_t *>(h->sum_fac.p);
   sp.coef = static_cast<const int32_t *>(h->sum_coef.p);
   sp.polys = static_cast<const pe::SumPoly *>(h->sum_polys.p);
@@ -919,6 +922,8 @@ int run_sum(polyeval *h, const void *points, int64_t P, void *out_f, void *out_J
   sp.out_f = static_cast<double *>(out_f);
   sp.out_J = static_cast<double *>(out_J);
   sp.table = static_cast<unsigned char *>(h->sum_table.p);
+  sp.sys0 = h->sys[0];
+  sp.sum_sys0 = h->sum_sys[0];
   sp.count = h->count;
   sp.n_polys_total = h->n_polys_total;
   unsigned char *ctl = static_cast<unsigned char *>(h->sum_ctl.p);
@@ -932,11 +937,16 @@ int run_sum(polyeval *h, const void *points, int64_t P, void *out_f, void *out_J
     const int64_t tiles = (P + (1 << lg) - 1) >> lg;
     const polyeval::SumLaunch &sl = h->sum_launch[lg];
     sp.single_P = static_cast<int32_t>(P);
-    sp.single_lg = lg;
     sp.power_total = static_cast<int64_t>(d.n) * (tiles << lg);
-    // runs of polynomials that share a copy of the table: about 8 runs per
-    // resident block, so that the last wave is short
-    const int64_t run = std::max<int64_t>(1, std::min<int64_t>(16, tiles * d.N / (8 * static_cast<int64_t>(sl.blocks))));
+    // Runs of polynomials that share a copy of the table: until an item's start
+    // (the copy, its latencies and barriers) is less than a thirtieth of it, at
+    // most an eighth of a block's share.  (Cycles: a product of a point takes
+    // about 10 with three blocks on an SM.  n = 64 in double, 4096 points: runs
+    // of one polynomial 9.2 ms, of 16 8.7 ms.)
+    const double start = 5000.0 + static_cast<double>(pe::sum_tab_bytes(h->sum_L, d.n, d.emax, lg)) / 16.0;
+    const double poly = 8000.0 + 10.0 * h->sum_products / static_cast<double>(std::max(d.N, 1)) * (1 << lg);
+    const int64_t most = std::max<int64_t>(1, tiles * d.N / (8 * static_cast<int64_t>(sl.blocks)));
+    const int64_t run = std::min<int64_t>(most, std::max<int64_t>(1, static_cast<int64_t>(std::ceil(32.0 * start / poly))));
     sp.group_polys = static_cast<int32_t>(run);
     sp.groups = static_cast<int32_t>((d.N + run - 1) / run);
     sp.n_items = tiles * sp.groups;
@@ -948,12 +958,13 @@ int run_sum(polyeval *h, const void *points, int64_t P, void *out_f, void *out_J
   }
   const polyeval::SumLaunch &sl = h->sum_launch[lg];
   sp.values = sl.values;
+  sp.lg = lg;
   const size_t flagged = P >= 0 ? static_cast<size_t>(P) : static_cast<size_t>(h->sum_points);
   if (cudaMemsetAsync(h->sum_ctl.p, 0, kCtlFlags + flagged, s) != cudaSuccess) return PE_ECUDA;
   if (pe::launch_sum_powers(h->sum_L, sp, s) != cudaSuccess) return PE_ECUDA;
   if (e0 && cudaEventRecord(e0, s) != cudaSuccess) return PE_ECUDA;
   const int grid = static_cast<int>(std::min<int64_t>(sp.n_items, sl.blocks));
-  if (pe::launch_sum(h->sum_L, sp, sl.tab_shared, sl.threads, sl.smem, grid, s) != cudaSuccess) return PE_ECUDA;
+  if (pe::launch_sum(h->sum_L, sp, sl.one, sl.tab_shared, sl.threads, sl.smem, grid, s) != cudaSuccess) return PE_ECUDA;
   h->kernels_launched += 2;
   return PE_OK;
 }

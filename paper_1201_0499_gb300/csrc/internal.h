@@ -116,7 +116,6 @@ struct SumSys {
   int64_t tab_off;    // bytes: its tables
   int64_t flag_off;   // its points' flags
   float most_log2;    // points with a coordinate modulus outside 2^(+-most_log2) are flagged
-  int32_t lg;         // log2 of the points per tile (batch handles)
   int32_t act_max;    // most variables of a polynomial
   int32_t head_bits;  // headroom of the window: log2 of a bound of sum_t a_t
 };
@@ -133,9 +132,8 @@ struct SumPoly {
 
 struct SumParams {
   const int32_t *poly_ptr;  // [Ntot+1] monomials of each polynomial (by falling k within it)
-  const int32_t *fac_ptr;   // [M+1] offsets into fac
   const uint32_t *fac;      // table entries (a - 1) n + v of each monomial
-  const int32_t *coef;      // [M][kSumCoefWords] digits
+  const int32_t *coef;      // [M][kSumCoefWords] records: digits, exponent, first of fac, count, first factor
   const SumPoly *polys;     // [Ntot]
   const int32_t *act;
   const uint32_t *act_bits;
@@ -153,8 +151,10 @@ struct SumParams {
   int64_t n_items;
   int32_t count;
   int32_t single_P;         // >= 0: single-system handle
-  int32_t single_lg;
+  int32_t lg;               // log2 of the points per tile
   int32_t values;           // monomials per thread and chunk (1 or 2)
+  SysDesc sys0;             // single: sys[0], sum_sys[0]
+  SumSys sum_sys0;
   int32_t groups, group_polys;  // single: runs of polynomials per tile, polynomials per run
   int32_t n_polys_total;
   unsigned *counter;        // work counter and ...
@@ -163,7 +163,11 @@ struct SumParams {
 };
 
 template <int L>
-constexpr int kSumCoefWords = L == 3 ? 8 : L == 4 ? 12 : 20;
+constexpr int kSumCoefWords = L == 8 ? 20 : 12;
+
+// Rows of a tile's sums and marks: (active variable, component) tasks, rounded
+// up to eight, and the parts of f.
+__host__ __device__ constexpr int sum_rows(int act_max) { return ((2 * act_max + 7) & ~7) + 2 * kSumParts; }
 
 // Bytes of a tile's table (entries x^1 .. x^levels of n variables) and of the
 // table with the inverses that follow it.
@@ -174,13 +178,16 @@ __host__ __device__ constexpr size_t sum_tab_bytes(int L, int n, int levels, int
 __host__ __device__ constexpr size_t sum_blob_bytes(int L, int n, int levels, int lg) {
   return sum_tab_bytes(L, n, levels, lg) + sum_tab_bytes(L, n, 1, lg);
 }
-size_t sum_smem_bytes(int L, int n, int act_max, int levels, int lg, int threads, int values, bool tab_shared);
+size_t sum_smem_bytes(int L, int n, int act_max, int levels, int lg, int threads, int values, bool one,
+                      bool tab_shared);
 int sum_head_bits_min(int L);
-cudaError_t prepare_sum(int L, size_t smem);
-cudaError_t sum_occupancy(int L, bool tab_shared, int threads, size_t smem, int *blocks);
+cudaError_t prepare_sum(int L, bool batch, size_t smem);
+cudaError_t sum_occupancy(int L, bool batch, bool one, bool tab_shared, int threads, size_t smem, int *blocks);
 cudaError_t launch_sum_powers(int L, const SumParams &p, cudaStream_t s);
-cudaError_t launch_sum(int L, const SumParams &p, bool tab_shared, int threads, size_t smem, int grid, cudaStream_t s);
-cudaError_t convert_coef_sum(int L, const double *coef, const int32_t *order, int32_t *out, int64_t M, cudaStream_t s);
+cudaError_t launch_sum(int L, const SumParams &p, bool one, bool tab_shared, int threads, size_t smem, int grid,
+                       cudaStream_t s);
+cudaError_t convert_coef_sum(int L, const double *coef, const int32_t *order, const int32_t *fac_ptr, const uint32_t *fac,
+                             int32_t *out, int64_t M, cudaStream_t s);
 
 // Launchers (kernels.cu).  `dd` selects complex double-double, else complex
 // double.  They return the cudaError_t of the launch.

@@ -260,7 +260,8 @@ __device__ __forceinline__ Num<L> read_number(const double *p, int t, fx::Seen &
 }
 
 template <int L>
-__global__ void sum_coef_kernel(const double *coef, const int32_t *order, int32_t *out, int64_t M) {
+__global__ void sum_coef_kernel(const double *coef, const int32_t *order, const int32_t *fac_ptr, const uint32_t *fac,
+                                int32_t *out, int64_t M) {
   constexpr int CW = kSumCoefWords<L>;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < M; t += stride) {
@@ -277,6 +278,9 @@ __global__ void sum_coef_kernel(const double *coef, const int32_t *order, int32_
 #pragma unroll
     for (int i = 0; i < L; i++) o[i] = y.re[i], o[L + i] = y.im[i];
     o[2 * L] = y.e;
+    o[2 * L + 1] = fac_ptr[t];
+    o[2 * L + 2] = fac_ptr[t + 1] - fac_ptr[t];
+    o[2 * L + 3] = fac_ptr[t + 1] > fac_ptr[t] ? static_cast<int32_t>(fac[fac_ptr[t]]) : 0;
   }
 }
 
@@ -301,7 +305,7 @@ __global__ void __launch_bounds__(128) sum_powers(const SumParams sp) {
     const SumSys ss = sp.sum_sys[s];
     const SysDesc sd = sp.sys[s];
     const int P = sp.single_P >= 0 ? sp.single_P : sd.P;
-    const int lg = sp.single_P >= 0 ? sp.single_lg : ss.lg;
+    const int lg = sp.lg;
     const int n = sd.n;
     const int tile_entries = n << lg;
     const int tile = static_cast<int>(local / tile_entries);
@@ -386,25 +390,32 @@ __device__ __forceinline__ void store_window(int4 *quads, int32_t *rest, int row
     reinterpret_cast<int2 *>(rest)[row] = make_int2(z[4 * Q], z[4 * Q + 1]);
 }
 
-// The value of monomial t at point q of the tile.
+// The value of monomial t at point q of the tile.  Its record holds the
+// coefficient's digits and exponent, the place and number of its factors and
+// the first of them, so that one load leads to the first product.
 template <int L>
 __device__ __forceinline__ Num<L> monomial_value(const SumParams &sp, int t, const int4 *tab, const int32_t *exps, int lg,
                                                  int q) {
-  Num<L> y;
-  const int32_t *co = sp.coef + static_cast<size_t>(t) * kSumCoefWords<L>;
+  constexpr int CW = kSumCoefWords<L>;
+  int32_t r[CW];
+  const int4 *co = reinterpret_cast<const int4 *>(sp.coef + static_cast<size_t>(t) * CW);
 #pragma unroll
-  for (int i = 0; i < L; i++) y.re[i] = __ldg(co + i), y.im[i] = __ldg(co + L + i);
-  y.e = __ldg(co + 2 * L);
-  const int fb = __ldg(sp.fac_ptr + t), fe = __ldg(sp.fac_ptr + t + 1);
-  if (fb < fe) {
-    unsigned idx = __ldg(sp.fac + fb);
+  for (int i = 0; i < CW / 4; i++) {
+    const int4 x = __ldg(co + i);
+    r[4 * i] = x.x, r[4 * i + 1] = x.y, r[4 * i + 2] = x.z, r[4 * i + 3] = x.w;
+  }
+  Num<L> y;
+#pragma unroll
+  for (int i = 0; i < L; i++) y.re[i] = r[i], y.im[i] = r[L + i];
+  y.e = r[2 * L];
+  const int fb = r[2 * L + 1], fe = fb + r[2 * L + 2];
+  unsigned idx = static_cast<unsigned>(r[2 * L + 3]);
 #pragma unroll 1
-    for (int j = fb; j < fe; j++) {
-      const Num<L> x = load_factor<L>(tab, exps, idx, lg, q);
-      if (j + 1 < fe) idx = __ldg(sp.fac + j + 1);
-      fx::mul<L>(y, x);
-      if (((j - fb) & (fx::kCheckEvery - 1)) == fx::kCheckEvery - 1) fx::check<L>(y);
-    }
+  for (int j = fb; j < fe; j++) {
+    const Num<L> x = load_factor<L>(tab, exps, idx, lg, q);
+    if (j + 1 < fe) idx = __ldg(sp.fac + j + 1);
+    fx::mul<L>(y, x);
+    if (((j - fb) & (fx::kCheckEvery - 1)) == fx::kCheckEvery - 1) fx::check<L>(y);
   }
   return y;
 }
@@ -428,31 +439,38 @@ __device__ __forceinline__ void to_window(const int32_t (&d)[L], int32_t e, int 
   sar_words<W>(z, max(E - e - 32 * NW + 1 + hb, 0));
 }
 
+// The top B L - 1 bits of a window integer (exponent of bit 0: e0), counted
+// from two above bit `lead`, as y-kind digits, and their exponent.
+template <int L>
+__device__ __forceinline__ void top_digits(uint32_t (&z)[Fmt<L>::W], int lead, int32_t e0, int32_t (&d)[L], int32_t &e) {
+  constexpr int B = Fmt<L>::B, W = Fmt<L>::W, o0 = 32 * W + 1 - B * L;
+  const int sh = min(32 * W - 3 - lead, 32 * W - 1);
+  shl_words<W>(z, sh);
+#pragma unroll
+  for (int i = 0; i < L; i++) {
+    const int w = (o0 + B * i) >> 5, b = (o0 + B * i) & 31;
+    d[i] = i == L - 1 ? static_cast<int32_t>(z[W - 1]) >> (33 - B)
+                      : static_cast<int32_t>(__funnelshift_r(z[w], z[w + 1], b)) & ((1 << B) - 1);
+  }
+  e = e0 - sh + o0;
+}
+
+// The lanes that hold the parts of f: eight tasks of 2^lg points, aligned.
+__device__ __forceinline__ unsigned lanes_of_parts(int lane, int lg) {
+  const int count = 2 * kSumParts << lg;  // 8, 16 or 32
+  return count == 32 ? 0xffffffffu : ((1u << count) - 1u) << (lane & ~(count - 1));
+}
+
 // One entry of J: the sums of its components (window integers, exponent of
 // bit 0) times 1 / x_v.
 template <int L>
 __device__ __forceinline__ void finish_entry(uint32_t (&zr)[Fmt<L>::W], uint32_t (&zi)[Fmt<L>::W], int32_t e0,
                                              const Num<L> &inv, double *o) {
-  constexpr int B = Fmt<L>::B, W = Fmt<L>::W;
+  constexpr int W = Fmt<L>::W;
   const int lead = max(lead_words<W>(zr), lead_words<W>(zi));
-  const int sh = min(32 * W - 3 - lead, 32 * W - 1);
-  shl_words<W>(zr, sh);
-  shl_words<W>(zi, sh);
-  // digits of the top B L - 1 bits
-  constexpr int o0 = 32 * W + 1 - B * L;
   Num<L> y;
-#pragma unroll
-  for (int i = 0; i < L; i++) {
-    const int w = (o0 + B * i) >> 5, b = (o0 + B * i) & 31;
-    if (i == L - 1) {
-      y.re[i] = static_cast<int32_t>(zr[W - 1]) >> (33 - B);
-      y.im[i] = static_cast<int32_t>(zi[W - 1]) >> (33 - B);
-    } else {
-      y.re[i] = static_cast<int32_t>(__funnelshift_r(zr[w], zr[w + 1], b)) & ((1 << B) - 1);
-      y.im[i] = static_cast<int32_t>(__funnelshift_r(zi[w], zi[w + 1], b)) & ((1 << B) - 1);
-    }
-  }
-  y.e = e0 - sh + o0;
+  top_digits<L>(zr, lead, e0, y.re, y.e);
+  top_digits<L>(zi, lead, e0, y.im, y.e);
   fx::mul<L>(y, inv);
   store_product<L>(o, y.re, y.e);
   store_product<L>(o + kComp<L>, y.im, y.e);
@@ -501,52 +519,57 @@ __device__ __forceinline__ void own_windows(const SumParams &sp, int gp, const u
   }
 }
 
-template <int L, bool kTabShared>
+// kBatch: a batch handle (systems and items from tables in global memory);
+// else one system, whose description comes with the parameters.
+// kOne: every polynomial's monomials fit in one chunk; the sums then stay in
+// registers from the first term to the output.
+template <int L, bool kTabShared, bool kBatch, bool kOne>
 __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(const SumParams sp) {
-  constexpr int W = Fmt<L>::W, KC = kComp<L>;
+  constexpr int B = Fmt<L>::B, W = Fmt<L>::W, KC = kComp<L>;
   constexpr int kw = Fmt<L>::kKeep / 32, kb = Fmt<L>::kKeep % 32;
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int32_t ebuf[3][kSumPointsMax];
+  __shared__ int32_t ebuf[2][kSumPointsMax];
   __shared__ unsigned next_item;
   const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31;
   int64_t held = -1;  // the tile whose table is in shared memory
-  for (unsigned item = blockIdx.x;;) {
-    if (item >= static_cast<unsigned>(sp.n_items)) break;
-    int gp0, gp1, tile, s;
-    if (sp.single_P >= 0) {
-      s = 0;
-      tile = item / sp.groups;
-      const int g = item - tile * sp.groups;
-      gp0 = g * sp.group_polys;
-      gp1 = min(gp0 + sp.group_polys, sp.n_polys_total);
-    } else {
+  int eb = 0;         // ebuf of the current chunk: the largest exponent per point
+  if (tid < kSumPointsMax) ebuf[0][tid] = fx::kZeroExp;
+  for (unsigned item = blockIdx.x; item < static_cast<unsigned>(sp.n_items);) {
+    int gp0, gp1, tile, s = 0;
+    if constexpr (kBatch) {
       const int4 it = sp.items[item];
       gp0 = it.x, gp1 = it.x + it.y, tile = it.z, s = it.w;
+    } else {
+      tile = item / sp.groups;
+      gp0 = (item - tile * sp.groups) * sp.group_polys;
+      gp1 = min(gp0 + sp.group_polys, sp.n_polys_total);
     }
-    const SysDesc sd = sp.sys[s];
-    const SumSys ss = sp.sum_sys[s];
-    const int P = sp.single_P >= 0 ? sp.single_P : sd.P;
-    const int lg = sp.single_P >= 0 ? sp.single_lg : ss.lg;
+    const SysDesc &sd = kBatch ? sp.sys[s] : sp.sys0;
+    const SumSys &ss = kBatch ? sp.sum_sys[s] : sp.sum_sys0;
+    const int P = kBatch ? sd.P : sp.single_P;
+    const int lg = sp.lg;
     const int TP = 1 << lg, q = tid & (TP - 1), sub = tid >> lg, subs = NT >> lg;
     const int n = sd.n, levels = sd.emax;
     const int qg = (tile << lg) + q;
     const bool valid = qg < P;
+    const bool left = sp.flags[ss.flag_off + min(qg, P - 1)] != 0;  // to the general kernels
     const unsigned char *blob = sp.table + ss.tab_off + static_cast<size_t>(tile) * sum_blob_bytes(L, n, levels, lg);
     const size_t tab_bytes = sum_tab_bytes(L, n, levels, lg);
     const size_t exp_off = static_cast<size_t>(levels) * n * kParts<L> * 16 << lg;
-    // shared memory: values first (their place does not depend on the system)
+    // shared memory: values first (their place does not depend on the system),
+    // sums, marks, table
     const int vrows = 2 * NT * sp.values;
     int4 *vq = reinterpret_cast<int4 *>(smem);
     int32_t *vr = reinterpret_cast<int32_t *>(vq + Win<L>::Q * vrows);
-    const int arows = 2 * (ss.act_max + kSumParts) << lg;
-    int4 *aq = reinterpret_cast<int4 *>(smem + static_cast<size_t>(vrows) * W * 4);
+    const int arows = sum_rows(ss.act_max) << lg;
+    unsigned char *at = smem + static_cast<size_t>(vrows) * W * 4;
+    int4 *aq = reinterpret_cast<int4 *>(at);
     int32_t *ar = reinterpret_cast<int32_t *>(aq + Win<L>::Q * arows);
-    uint32_t *am = reinterpret_cast<uint32_t *>(ar + Win<L>::R * arows);
-    unsigned char *stab = smem + static_cast<size_t>(vrows) * W * 4 + ((static_cast<size_t>(arows) * (W * 4 + 4) + 15) & ~size_t{15});
-    // a tile whose every point is flagged already is left to the general kernels
-    if (__syncthreads_and(sp.flags[ss.flag_off + min(qg, P - 1)] != 0)) gp0 = gp1;
+    if (!kOne) at += static_cast<size_t>(arows) * W * 4;
+    uint32_t *am = reinterpret_cast<uint32_t *>(at);
+    unsigned char *stab = at + static_cast<size_t>(arows) * 4;
     const int64_t tile_id = (static_cast<int64_t>(s) << 32) | tile;
-    if (gp0 < gp1 && kTabShared && held != tile_id) {
+    if (kTabShared && held != tile_id) {
       const int4 *src = reinterpret_cast<const int4 *>(blob);
       int4 *dst = reinterpret_cast<int4 *>(stab);
       const int words = static_cast<int>(tab_bytes / 16);
@@ -555,13 +578,21 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
     }
     const int4 *tab = reinterpret_cast<const int4 *>(kTabShared ? stab : blob);
     const int32_t *exps = reinterpret_cast<const int32_t *>((kTabShared ? stab : blob) + exp_off);
+    const unsigned char *ib = blob + tab_bytes;
+    const int4 *inv4 = reinterpret_cast<const int4 *>(ib);
+    const int32_t *inve = reinterpret_cast<const int32_t *>(ib + (static_cast<size_t>(n) * kParts<L> * 16 << lg));
     const int hb = ss.head_bits;
+    // a tile whose every point is left to the general kernels is not evaluated
+    if (__syncthreads_and(left)) gp0 = gp1;
     for (int gp = gp0; gp < gp1; gp++) {
-      const int t0 = sp.poly_ptr[gp], t1 = sp.poly_ptr[gp + 1];
+      const int t0 = __ldg(sp.poly_ptr + gp), t1 = __ldg(sp.poly_ptr + gp + 1);
       const int pl = gp - sd.poly0;
       const SumPoly sy = sp.polys[gp];
-      const int tasks = 2 * sy.act_n, all = tasks + 2 * kSumParts;
+      // tasks of phase B: (active variable, component), then from a multiple
+      // of eight the parts of f
+      const int tasks = 2 * sy.act_n, fb = (tasks + 7) & ~7, all = fb + 2 * kSumParts;
       double *Jp = sp.out_J + (static_cast<size_t>(sd.J_off) + static_cast<size_t>(pl) * n * P + qg) * 2 * KC;
+      double *fp = sp.out_f + (static_cast<size_t>(sd.f_off) + static_cast<size_t>(pl) * P + qg) * 2 * KC;
       // entries of variables that do not occur in the polynomial
       if (sy.act_n < n && valid) {
         for (int v = sub; v < n; v += subs) {
@@ -571,20 +602,70 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
           store_zero<L>(o + KC);
         }
       }
-      // sums to zero; no exponent yet
-      for (int u = sub; u < all; u += subs) {
-        uint32_t z[W];
-#pragma unroll
-        for (int i = 0; i < W; i++) z[i] = 0u;
-        const int row = (u << lg) + q;
-        store_window<L>(aq, ar, arows, row, z);
-        am[row] = 0u;
+      if (t0 == t1) {  // no monomials
+        if (valid && sub < 2) store_zero<L>(fp + sub * KC);
+        continue;
       }
-      if (tid < 3 * TP) ebuf[tid >> lg][q] = fx::kZeroExp;
-      __syncthreads();
-      int eb = 0;  // ebuf of this chunk
       const int chunk = subs * sp.values;
-      for (int tb = t0; tb < t1; tb += chunk) {
+      bool again = false;
+      int32_t e0 = 0;  // exponent of the window's bit 0
+      // The sum into f (its parts are 2 TP lanes apart, in one warp).
+      auto finish_f = [&](int u, uint32_t (&a)[W]) {
+        const unsigned mask = lanes_of_parts(lane, lg);
+#pragma unroll
+        for (int d = 2; d < 2 * kSumParts; d <<= 1) {
+          uint32_t z[W];
+#pragma unroll
+          for (int i = 0; i < W; i++) z[i] = __shfl_xor_sync(mask, a[i], d << lg);
+          add_words<W>(a, z);
+        }
+        if (valid && u - fb < 2) store_sum<L>(fp + (u & 1) * KC, a, e0);
+      };
+      // An entry of J: the sum times 1 / x_v.  The other component's sum is in
+      // lane ^ TP; each lane forms its own component of the product.
+      auto finish_J = [&](int u, uint32_t (&a)[W], uint32_t m) {
+        const int c = u & 1;
+        const unsigned pair = (1u << lane) | (1u << (lane ^ TP));
+        const int v = __ldg(sp.act + sy.act_off + (u >> 1));
+        const Num<L> inv = load_factor<L>(inv4, inve, v, lg, q);
+        m |= __shfl_xor_sync(pair, m, TP);
+        am[(u << lg) + q] = m;
+        again = again || (m == 0u && valid);
+        int lead = lead_words<W>(a);
+        lead = max(lead, __shfl_xor_sync(pair, lead, TP));
+        int32_t own[L], other[L], r[L];
+        int32_t ey;
+        top_digits<L>(a, lead, e0, own, ey);
+#pragma unroll
+        for (int i = 0; i < L; i++) other[i] = __shfl_xor_sync(pair, own[i], TP);
+        const int32_t flip = c ? 0 : -1;  // real lanes subtract the product of the imaginary parts
+        long long col[L];
+#pragma unroll
+        for (int k = 0; k < L; k++) {
+          col[k] = 0;
+#pragma unroll
+          for (int i = k; i < L; i++) {
+            col[k] += static_cast<long long>(inv.re[i]) * own[k + L - 1 - i];
+            col[k] += static_cast<long long>((inv.im[i] ^ flip) - flip) * other[k + L - 1 - i];
+          }
+        }
+        fx::fold<L>(col, r);
+        if (valid && m != 0u)
+          store_product<L>(Jp + static_cast<size_t>(v) * P * 2 * KC + c * KC, r, ey + inv.e + B * L - 1);
+      };
+      int Eprev = 0;
+      if constexpr (!kOne) {  // sums to zero
+        for (int u = sub; u < all; u += subs) {
+          uint32_t z[W];
+#pragma unroll
+          for (int i = 0; i < W; i++) z[i] = 0u;
+          const int row = (u << lg) + q;
+          store_window<L>(aq, ar, arows, row, z);
+          am[row] = 0u;
+        }
+      }
+      for (int tb = t0; kOne ? tb == t0 : tb < t1; tb += chunk) {
+        const bool last = kOne || tb + chunk >= t1;
         // A: the values of monomials tb + sub, tb + sub + subs at point q, their
         // digits to the places of their window integers
         int em = fx::kZeroExp;
@@ -605,8 +686,7 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
         if (lane < TP) atomicMax(&ebuf[eb][q], em);
         __syncthreads();
         const int E = ebuf[eb][q];
-        const int prev = eb == 0 ? 2 : eb - 1, nxt = eb == 2 ? 0 : eb + 1;
-        const int grown = tb == t0 ? 0 : E - ebuf[prev][q];
+        const int grown = kOne || tb == t0 ? 0 : E - Eprev;
         for (int x = 0; x < sp.values; x++) {
           const int tl = x * subs + sub;
           if (tb + tl >= t1) break;
@@ -621,27 +701,33 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
             store_window<L>(vq, vr, vrows, ((2 * tl + c) << lg) + q, z);
           }
         }
-        if (tid < TP) ebuf[nxt][q] = E;
+        if (tid < TP) ebuf[eb ^ 1][q] = last ? fx::kZeroExp : E;  // of the next chunk
         __syncthreads();
         // B: the sums of active variable u >> 1, component u & 1 at point q, and
-        // after the variables the parts of f
-        const int b0 = (tb - t0) / kSumBlock;
+        // the parts of f
+        const int b0 = kOne ? 0 : (tb - t0) / kSumBlock;
         const int b1 = min((tb - t0 + chunk) / kSumBlock, (t1 - t0 + kSumBlock - 1) / kSumBlock);
+        e0 = E - (32 * W - 1 - hb);
         for (int u = sub; u < all; u += subs) {
+          if (u >= tasks && u < fb) continue;
           const int row = (u << lg) + q, c = u & 1;
-          uint32_t a[W], odd[W - 1];
-          uint32_t m = am[row];
-          load_window<L>(aq, ar, arows, row, a);
+          uint32_t a[W];
+          uint32_t m = 0u;
+          if constexpr (kOne) {
 #pragma unroll
-          for (int i = 0; i < W - 1; i++) odd[i] = 0u;
-          if (grown > 0) {
-            sar_words<W>(a, grown);
-            m >>= min(grown, 31);
+            for (int i = 0; i < W; i++) a[i] = 0u;
+          } else {
+            load_window<L>(aq, ar, arows, row, a);
+            m = am[row];
+            if (grown > 0) {
+              sar_words<W>(a, grown);
+              m >>= min(grown, 31);
+            }
           }
-          if (u >= tasks) {
+          if (u >= fb) {
             constexpr int len = kSumBlock / kSumParts;
             for (int b = b0; b < b1; b++) {
-              const int tl = (b - b0) * kSumBlock + ((u - tasks) >> 1) * len;
+              const int tl = (b - b0) * kSumBlock + ((u - fb) >> 1) * len;
               const int count = min(len, t1 - tb - tl);
 #pragma unroll 4
               for (int k = 0; k < count; k++) {
@@ -650,9 +736,15 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
                 add_words<W>(a, z);
               }
             }
-            store_window<L>(aq, ar, arows, row, a);
+            if constexpr (kOne)
+              finish_f(u, a);
+            else
+              store_window<L>(aq, ar, arows, row, a);
             continue;
           }
+          uint32_t odd[W - 1];
+#pragma unroll
+          for (int i = 0; i < W - 1; i++) odd[i] = 0u;
           for (int b = b0; b < b1; b++) {
             const int32_t *hq = sp.hit_ptr + sy.hit_off + static_cast<int64_t>(b) * (sy.act_n + 1) + (u >> 1);
             const int h0 = __ldg(hq), h1 = __ldg(hq + 1);
@@ -684,97 +776,79 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
 #pragma unroll
           for (int i = 0; i < W - 1; i++) up[i + 1] = odd[i];
           add_words<W>(a, up);
-          store_window<L>(aq, ar, arows, row, a);
-          am[row] = m;
+          if constexpr (kOne) {
+            finish_J(u, a, m);
+          } else {
+            store_window<L>(aq, ar, arows, row, a);
+            am[row] = m;
+          }
         }
-        eb = nxt;
+        eb ^= 1;
+        Eprev = E;
+        if (!last) __syncthreads();
+      }
+      if constexpr (!kOne) {  // every thread finishes the sums that it stored
+        for (int u = sub; u < all; u += subs) {
+          if (u >= tasks && u < fb) continue;
+          const int row = (u << lg) + q;
+          uint32_t a[W];
+          load_window<L>(aq, ar, arows, row, a);
+          if (u >= fb)
+            finish_f(u, a);
+          else
+            finish_J(u, a, am[row]);
+        }
+      }
+      if (__syncthreads_or(again)) {
+        if (valid) own_windows<L>(sp, gp, am, tab, exps, inv4, inve, lg, q, hb, sub, subs, Jp, P);
         __syncthreads();
       }
-      // outputs
-      const int32_t ep = ebuf[eb][q] - (32 * W - 1 - hb);
-      const unsigned char *ib = blob + tab_bytes;
-      const int4 *it4 = reinterpret_cast<const int4 *>(ib);
-      const int32_t *ite = reinterpret_cast<const int32_t *>(ib + (static_cast<size_t>(n) * kParts<L> * 16 << lg));
-      bool again = false;
-      if (valid) {
-        for (int i0 = sub; i0 < sy.act_n; i0 += subs) {
-          const int v = __ldg(sp.act + sy.act_off + i0);
-          double *o = Jp + static_cast<size_t>(v) * P * 2 * KC;
-          const int row = ((2 * i0) << lg) + q;
-          const Num<L> inv = load_factor<L>(it4, ite, v, lg, q);
-          if (!(am[row] | am[row + TP])) {
-            again = true;
-            continue;
-          }
-          uint32_t zr[W], zi[W];
-          load_window<L>(aq, ar, arows, row, zr);
-          load_window<L>(aq, ar, arows, row + TP, zi);
-          finish_entry<L>(zr, zi, ep, inv, o);
-        }
-        // the last threads, which have the fewest entries of J
-        const int c = subs - 1 - sub;
-        if (c < 2) {
-          uint32_t z[W], a[W];
-          load_window<L>(aq, ar, arows, ((tasks + c) << lg) + q, z);
-          for (int k = 1; k < kSumParts; k++) {
-            load_window<L>(aq, ar, arows, ((tasks + 2 * k + c) << lg) + q, a);
-            add_words<W>(z, a);
-          }
-          store_sum<L>(sp.out_f + (static_cast<size_t>(sd.f_off) + static_cast<size_t>(pl) * P + qg) * 2 * KC + c * KC, z, ep);
-        }
-        if (again) own_windows<L>(sp, gp, am, tab, exps, it4, ite, lg, q, hb, sub, subs, Jp, P);
-      }
-      __syncthreads();
     }
     if (tid == 0) next_item = atomicAdd(sp.counter, 1u) + gridDim.x;
     __syncthreads();
     item = next_item;
-    __syncthreads();
   }
 }
 
-template <int L>
-cudaError_t prepare_t(int smem) {
-  cudaError_t e = cudaFuncSetAttribute(sum_kernel<L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(sum_kernel<L, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-}
+// The kernel of a launch.
+using SumKernel = void (*)(const SumParams);
 
 template <int L>
-cudaError_t launch_t(const SumParams &p, bool tab_shared, int threads, size_t smem, int grid, cudaStream_t s) {
-  if (tab_shared)
-    sum_kernel<L, true><<<grid, threads, smem, s>>>(p);
-  else
-    sum_kernel<L, false><<<grid, threads, smem, s>>>(p);
-  return cudaGetLastError();
+SumKernel kernel_of(bool tab_shared, bool batch, bool one) {
+  if (one)
+    return tab_shared ? (batch ? sum_kernel<L, true, true, true> : sum_kernel<L, true, false, true>)
+                      : (batch ? sum_kernel<L, false, true, true> : sum_kernel<L, false, false, true>);
+  return tab_shared ? (batch ? sum_kernel<L, true, true, false> : sum_kernel<L, true, false, false>)
+                    : (batch ? sum_kernel<L, false, true, false> : sum_kernel<L, false, false, false>);
 }
 
-template <int L>
-cudaError_t occupancy_t(bool tab_shared, int threads, size_t smem, int *blocks) {
-  return tab_shared ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, sum_kernel<L, true>, threads, smem)
-                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, sum_kernel<L, false>, threads, smem);
+SumKernel kernel_of(int L, bool tab_shared, bool batch, bool one) {
+  return L == 3 ? kernel_of<3>(tab_shared, batch, one) : L == 4 ? kernel_of<4>(tab_shared, batch, one)
+                                                                : kernel_of<8>(tab_shared, batch, one);
 }
 
 }  // namespace
 
-size_t sum_smem_bytes(int L, int n, int act_max, int levels, int lg, int threads, int values, bool tab_shared) {
+size_t sum_smem_bytes(int L, int n, int act_max, int levels, int lg, int threads, int values, bool one, bool tab_shared) {
   const size_t W = L == 3 ? Fmt<3>::W : L == 4 ? Fmt<4>::W : Fmt<8>::W;
-  const size_t acc = (static_cast<size_t>(2) * (act_max + kSumParts) << lg) * (W * 4 + 4);
-  return static_cast<size_t>(2) * threads * values * W * 4 + ((acc + 15) & ~size_t{15}) +
+  return static_cast<size_t>(2) * threads * values * W * 4 +
+         (static_cast<size_t>(sum_rows(act_max)) << lg) * (one ? 4 : W * 4 + 4) +
          (tab_shared ? sum_tab_bytes(L, n, levels, lg) : 0);
 }
 
 int sum_head_bits_min(int L) { return L == 3 ? Fmt<3>::kHeadMin : L == 4 ? Fmt<4>::kHeadMin : Fmt<8>::kHeadMin; }
 
-cudaError_t prepare_sum(int L, size_t smem) {
-  const int v = static_cast<int>(smem);
-  return L == 3 ? prepare_t<3>(v) : L == 4 ? prepare_t<4>(v) : prepare_t<8>(v);
+cudaError_t prepare_sum(int L, bool batch, size_t smem) {
+  for (int k = 0; k < 4; k++) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel_of(L, k & 1, batch, k >> 1),
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
-cudaError_t sum_occupancy(int L, bool tab_shared, int threads, size_t smem, int *blocks) {
-  return L == 3   ? occupancy_t<3>(tab_shared, threads, smem, blocks)
-         : L == 4 ? occupancy_t<4>(tab_shared, threads, smem, blocks)
-                  : occupancy_t<8>(tab_shared, threads, smem, blocks);
+cudaError_t sum_occupancy(int L, bool batch, bool one, bool tab_shared, int threads, size_t smem, int *blocks) {
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kernel_of(L, tab_shared, batch, one), threads, smem);
 }
 
 cudaError_t launch_sum_powers(int L, const SumParams &p, cudaStream_t s) {
@@ -792,23 +866,24 @@ cudaError_t launch_sum_powers(int L, const SumParams &p, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_sum(int L, const SumParams &p, bool tab_shared, int threads, size_t smem, int grid, cudaStream_t s) {
-  return L == 3   ? launch_t<3>(p, tab_shared, threads, smem, grid, s)
-         : L == 4 ? launch_t<4>(p, tab_shared, threads, smem, grid, s)
-                  : launch_t<8>(p, tab_shared, threads, smem, grid, s);
+cudaError_t launch_sum(int L, const SumParams &p, bool one, bool tab_shared, int threads, size_t smem, int grid,
+                       cudaStream_t s) {
+  kernel_of(L, tab_shared, p.single_P < 0, one)<<<grid, threads, smem, s>>>(p);
+  return cudaGetLastError();
 }
 
-cudaError_t convert_coef_sum(int L, const double *coef, const int32_t *order, int32_t *out, int64_t M, cudaStream_t s) {
+cudaError_t convert_coef_sum(int L, const double *coef, const int32_t *order, const int32_t *fac_ptr, const uint32_t *fac,
+                             int32_t *out, int64_t M, cudaStream_t s) {
   if (M <= 0) return cudaSuccess;
   int64_t blocks = (M + 127) / 128;
   if (blocks > kSms * 64) blocks = kSms * 64;
   const unsigned b = static_cast<unsigned>(blocks);
   if (L == 3)
-    sum_coef_kernel<3><<<b, 128, 0, s>>>(coef, order, out, M);
+    sum_coef_kernel<3><<<b, 128, 0, s>>>(coef, order, fac_ptr, fac, out, M);
   else if (L == 4)
-    sum_coef_kernel<4><<<b, 128, 0, s>>>(coef, order, out, M);
+    sum_coef_kernel<4><<<b, 128, 0, s>>>(coef, order, fac_ptr, fac, out, M);
   else
-    sum_coef_kernel<8><<<b, 128, 0, s>>>(coef, order, out, M);
+    sum_coef_kernel<8><<<b, 128, 0, s>>>(coef, order, fac_ptr, fac, out, M);
   return cudaGetLastError();
 }
 
