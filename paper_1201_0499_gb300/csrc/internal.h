@@ -36,6 +36,34 @@ constexpr int kChainRenorm = 4;
 // Launches whose balance depends on it query the device instead.
 constexpr int kSms = 152;
 
+// Kernels of one call that follow each other on a stream: launch_next queues a
+// kernel that may be set up on the device while the one before it still runs
+// (programmatic dependent launch), and the kernel itself waits with
+// wait_for_previous() before it reads or writes anything another kernel
+// touches.  A kernel that calls let_next_start() lets its follower be set up
+// from then on, without it at its end.  Every kernel launched this way waits,
+// so completion is transitive along the chain.  What it saves is the idle time
+// between short kernels: five launches of a call at one point.
+#ifdef __CUDACC__
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+
+template <class... K, class... A>
+cudaError_t launch_next(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, K(args)...);
+}
+#endif
+
 // One compiled system inside a handle.  Offsets are in complex elements of
 // the handle's precision.
 struct SysDesc {

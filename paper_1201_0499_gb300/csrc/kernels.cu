@@ -248,6 +248,8 @@ __global__ void main_kernel(const MainParams kp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   typename A::V *smem = reinterpret_cast<typename A::V *>(smem_raw) + static_cast<size_t>(warp) * kp.kslots * 32;
+  let_next_start();
+  wait_for_previous();
   if (kp.any && *kp.any == 0) return;
   for (;;) {
     unsigned item = 0;
@@ -267,6 +269,8 @@ __global__ void main_kernel(const MainParams kp) {
 template <class A>
 __global__ void powers_kernel(const PowerParams pp) {
   constexpr int KD = A::kDoubles;
+  let_next_start();
+  wait_for_previous();
   if (pp.any && *pp.any == 0) return;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; idx < pp.total; idx += stride) {
@@ -315,6 +319,7 @@ template <class A>
 __global__ void combine_kernel(double *out_f, double *out_J, const double *scratch_f, const double *scratch_J,
                                int64_t f_doubles, int64_t J_doubles, int chunks, Only only) {
   constexpr int CD = A::kDoubles / 2;  // doubles per component
+  wait_for_previous();
   if (only.any && *only.any == 0) return;
   const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; k < (f_doubles + J_doubles) / CD; k += step) {
@@ -336,6 +341,11 @@ cudaError_t launch_combine(bool dd, double *out_f, double *out_J, const double *
   int64_t blocks = ((f_doubles + J_doubles) / (dd ? 2 : 1) + threads - 1) / threads;
   if (blocks > kSms * 64) blocks = kSms * 64;
   const unsigned b = static_cast<unsigned>(blocks);
+  if (only.any)
+    return dd ? launch_next(combine_kernel<ArithDD>, dim3(b), dim3(threads), 0, s, out_f, out_J, scratch_f, scratch_J,
+                            f_doubles, J_doubles, chunks, only)
+              : launch_next(combine_kernel<ArithF64>, dim3(b), dim3(threads), 0, s, out_f, out_J, scratch_f, scratch_J,
+                            f_doubles, J_doubles, chunks, only);
   if (dd)
     combine_kernel<ArithDD><<<b, threads, 0, s>>>(out_f, out_J, scratch_f, scratch_J, f_doubles, J_doubles, chunks, only);
   else
@@ -348,6 +358,9 @@ cudaError_t launch_powers(bool dd, const PowerParams &p, cudaStream_t s) {
   const int threads = 256;
   int64_t blocks = (p.total + threads - 1) / threads;
   if (blocks > kSms * 64) blocks = kSms * 64;
+  if (p.any)
+    return dd ? launch_next(powers_kernel<ArithDD>, dim3(static_cast<unsigned>(blocks)), dim3(threads), 0, s, p)
+              : launch_next(powers_kernel<ArithF64>, dim3(static_cast<unsigned>(blocks)), dim3(threads), 0, s, p);
   if (dd)
     powers_kernel<ArithDD><<<static_cast<unsigned>(blocks), threads, 0, s>>>(p);
   else
@@ -363,6 +376,8 @@ __global__ void main_kernel_batch(const MainParams kp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   typename A::V *smem = reinterpret_cast<typename A::V *>(smem_raw) + static_cast<size_t>(warp) * kp.kslots * 32;
+  let_next_start();
+  wait_for_previous();
   if (kp.any && *kp.any == 0) return;
   for (;;) {
     unsigned item = 0;
@@ -413,7 +428,8 @@ cudaError_t main_occupancy(bool dd, bool batch, int warps_per_block, size_t smem
 template <class A>
 cudaError_t launch_main_t(const MainParams &p, int warps_per_block, size_t smem_bytes, int grid, cudaStream_t s) {
   const dim3 b(warps_per_block * 32);
-  if (p.single_P < 0 || p.regroup) {
+  if (p.any && (p.single_P < 0 || p.regroup)) return launch_next(main_kernel_batch<A>, dim3(grid), b, smem_bytes, s, p);
+  if (p.single_P < 0) {
     main_kernel_batch<A><<<grid, b, smem_bytes, s>>>(p);
     return cudaGetLastError();
   }

@@ -43,6 +43,8 @@ __global__ void convert_coef_qd_kernel(const double *coef_qd, uint32_t *coef_blk
 __global__ void powers_qd(const PowerParams pp) {
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   uint32_t *table = reinterpret_cast<uint32_t *>(pp.table);
+  let_next_start();
+  wait_for_previous();
   if (pp.any && *pp.any == 0) return;
   for (int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; idx < pp.total; idx += stride) {
     int n, emax, P;
@@ -199,6 +201,8 @@ __global__ void __launch_bounds__(kWarpsPerBlockMax * 32) main_qd(const MainPara
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t *slots = reinterpret_cast<uint32_t *>(smem_raw) + static_cast<size_t>(warp) * kp.kslots * kQdSlotWords * 32;
+  let_next_start();
+  wait_for_previous();
   if (kp.any && *kp.any == 0) return;
   for (;;) {
     unsigned item = 0;
@@ -216,6 +220,7 @@ __global__ void __launch_bounds__(kWarpsPerBlockMax * 32) main_qd(const MainPara
 // (the first f_components) and then J.
 __global__ void finalize_qd(double *out_f, double *out_J, const double *scratch_f, const double *scratch_J,
                             int64_t f_components, int64_t J_components, int chunks, Only only) {
+  wait_for_previous();
   if (only.any && *only.any == 0) return;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   const int64_t total = f_components + J_components;
@@ -244,6 +249,7 @@ cudaError_t launch_powers_qd(const PowerParams &p, cudaStream_t s) {
   if (p.total <= 0) return cudaSuccess;
   int64_t blocks = (p.total + 127) / 128;
   if (blocks > kSms * 32) blocks = kSms * 32;
+  if (p.any) return launch_next(powers_qd, dim3(static_cast<unsigned>(blocks)), dim3(128), 0, s, p);
   powers_qd<<<static_cast<unsigned>(blocks), 128, 0, s>>>(p);
   return cudaGetLastError();
 }
@@ -258,6 +264,7 @@ cudaError_t main_qd_occupancy(int warps_per_block, size_t smem_bytes, int *block
 
 cudaError_t launch_main_qd(const MainParams &p, int warps_per_block, size_t smem_bytes, int grid, cudaStream_t s) {
   if (p.n_items <= 0) return cudaSuccess;
+  if (p.any) return launch_next(main_qd, dim3(grid), dim3(warps_per_block * 32), smem_bytes, s, p);
   main_qd<<<grid, warps_per_block * 32, smem_bytes, s>>>(p);
   return cudaGetLastError();
 }
@@ -269,6 +276,9 @@ cudaError_t launch_finalize_qd(double *out_f, double *out_J, const double *scrat
   if (total <= 0) return cudaSuccess;
   int64_t blocks = (total + 255) / 256;
   if (blocks > kSms * 16) blocks = kSms * 16;
+  if (only.any)
+    return launch_next(finalize_qd, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, s, out_f, out_J, scratch_f, scratch_J,
+                       f_components, J_components, chunks, only);
   finalize_qd<<<static_cast<unsigned>(blocks), 256, 0, s>>>(out_f, out_J, scratch_f, scratch_J, f_components,
                                                             J_components, chunks, only);
   return cudaGetLastError();

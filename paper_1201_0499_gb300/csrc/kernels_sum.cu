@@ -288,6 +288,7 @@ __global__ void sum_coef_kernel(const double *coef, const int32_t *order, const 
 // x^emax, role 1 writes 1 / x.  Points past the last repeat it.
 template <int L>
 __global__ void __launch_bounds__(128) sum_powers(const SumParams sp) {
+  let_next_start();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < 2 * sp.power_total; i += stride) {
     const bool inverse = i >= sp.power_total;
@@ -534,6 +535,8 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
   int64_t held = -1;  // the tile whose table is in shared memory
   int eb = 0;         // ebuf of the current chunk: the largest exponent per point
   if (tid < kSumPointsMax) ebuf[0][tid] = fx::kZeroExp;
+  let_next_start();
+  wait_for_previous();
   for (unsigned item = blockIdx.x; item < static_cast<unsigned>(sp.n_items);) {
     int gp0, gp1, tile, s = 0;
     if constexpr (kBatch) {
@@ -868,8 +871,7 @@ cudaError_t launch_sum_powers(int L, const SumParams &p, cudaStream_t s) {
 
 cudaError_t launch_sum(int L, const SumParams &p, bool one, bool tab_shared, int threads, size_t smem, int grid,
                        cudaStream_t s) {
-  kernel_of(L, tab_shared, p.single_P < 0, one)<<<grid, threads, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_next(kernel_of(L, tab_shared, p.single_P < 0, one), dim3(grid), dim3(threads), smem, s, p);
 }
 
 cudaError_t convert_coef_sum(int L, const double *coef, const int32_t *order, const int32_t *fac_ptr, const uint32_t *fac,

@@ -41,6 +41,8 @@ __global__ void convert_coef_kernel(const double *coef_dd, uint32_t *coef_wide, 
 __global__ void powers_wide(const PowerParams pp) {
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   uint32_t *table = reinterpret_cast<uint32_t *>(pp.table);
+  let_next_start();
+  wait_for_previous();
   if (pp.any && *pp.any == 0) return;
   for (int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; idx < pp.total; idx += stride) {
     int n, emax, P;
@@ -264,6 +266,8 @@ __global__ void __launch_bounds__(kWarpsPerBlockMax * 32) main_wide(const MainPa
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t *slots = reinterpret_cast<uint32_t *>(smem_raw) + static_cast<size_t>(warp) * kp.kslots * kSlotWords * 32;
+  let_next_start();
+  wait_for_previous();
   if (kp.any && *kp.any == 0) return;
   for (;;) {
     unsigned item = 0;
@@ -288,6 +292,7 @@ cudaError_t launch_powers_wide(const PowerParams &p, cudaStream_t s) {
   if (p.total <= 0) return cudaSuccess;
   int64_t blocks = (p.total + 127) / 128;
   if (blocks > kSms * 64) blocks = kSms * 64;
+  if (p.any) return launch_next(powers_wide, dim3(static_cast<unsigned>(blocks)), dim3(128), 0, s, p);
   powers_wide<<<static_cast<unsigned>(blocks), 128, 0, s>>>(p);
   return cudaGetLastError();
 }
@@ -308,6 +313,8 @@ cudaError_t main_wide_occupancy(bool prefetch, int warps_per_block, size_t smem_
 
 cudaError_t launch_main_wide(const MainParams &p, int warps_per_block, size_t smem_bytes, int grid, cudaStream_t s) {
   if (p.n_items <= 0) return cudaSuccess;
+  if (p.any)
+    return launch_next(p.prefetch ? main_wide<true> : main_wide<false>, dim3(grid), dim3(warps_per_block * 32), smem_bytes, s, p);
   if (p.prefetch)
     main_wide<true><<<grid, warps_per_block * 32, smem_bytes, s>>>(p);
   else
