@@ -524,8 +524,13 @@ __device__ __forceinline__ void own_windows(const SumParams &sp, int gp, const u
 // else one system, whose description comes with the parameters.
 // kOne: every polynomial's monomials fit in one chunk; the sums then stay in
 // registers from the first term to the output.
+//
+// Three blocks (24 warps) per SM, 80 registers: with two blocks double-double
+// at n = 32 took 15 % longer.  Quad-double with several chunks spills at 80
+// registers and keeps two blocks (n = 64: 3.65 ms, with three 3.83); with one
+// chunk (n = 32: 533 -> 490 us) and in batches three are faster all the same.
 template <int L, bool kTabShared, bool kBatch, bool kOne>
-__global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(const SumParams sp) {
+__global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2 : 3) sum_kernel(const SumParams sp) {
   constexpr int B = Fmt<L>::B, W = Fmt<L>::W, KC = kComp<L>;
   constexpr int kw = Fmt<L>::kKeep / 32, kb = Fmt<L>::kKeep % 32;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -807,6 +812,9 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 ? 2 : 3) sum_kernel(con
         __syncthreads();
       }
     }
+    // (Items come from a counter: equal shares of them in order, without one,
+    // took 8 % longer at n = 128, since the SMs are not equally fast; taking the
+    // next item while this one runs took 3 % longer there.)
     if (tid == 0) next_item = atomicAdd(sp.counter, 1u) + gridDim.x;
     __syncthreads();
     item = next_item;
