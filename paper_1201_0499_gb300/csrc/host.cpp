@@ -625,6 +625,43 @@ int run_main(polyeval *h, const pe::MainParams &mp, cudaStream_t s, int mode = 0
 // general kernels' counter, one spare word, the flags.
 constexpr size_t kCtlFlags = 16;
 
+// Whether the evaluation from values is the faster one for these systems:
+// nanoseconds per polynomial and point of both, fitted to measurements from 1
+// to 4096 points (GB300).  A tile's barriers cost polynomials of few products
+// more than the general kernels take for all of them, above all in double,
+// whose products are cheap there: n = 50, 8 monomials of 2 variables, 4096
+// points, general / from values: double 117 / 412 us, integer double-double
+// 290 / 468, quad-double 567 / 1142, double-double 601 / 468; n = 10, 24
+// monomials of 3: 109 / 102, (dd) 510 / 113, (qd) 319 / 263.
+bool sum_pays(const polyeval *h, const Compiled &c, const std::vector<pe::SumPoly> &sp) {
+  double general = 0.0, values = 0.0;
+  for (size_t gp = 0; gp < sp.size(); gp++) {
+    const SysDesc &d = h->sys[c.poly_sys[gp]];
+    const int32_t t0 = c.poly_ptr[gp], t1 = c.poly_ptr[gp + 1];
+    const double weight = h->batch ? d.P : 1.0, act = sp[gp].act_n, n = d.n;
+    const double factors = c.mono_ptr[t1] - c.mono_ptr[t0];
+    double products = 0.0;
+    for (int32_t t = t0; t < t1; t++) {
+      const int k = c.mono_ptr[t + 1] - c.mono_ptr[t];
+      int n2 = 0;
+      for (int32_t j = c.mono_ptr[t]; j < c.mono_ptr[t + 1]; j++) n2 += (c.var[j] >> 16) >= 2;
+      products += n2 + std::max(3 * k - 3, k);
+    }
+    const double chunks = 1.0 + 0.5 * ((t1 - t0) / 128);
+    if (h->qd) {
+      general += weight * (0.9 + 0.035 * products + 0.012 * n);
+      values += weight * (3.6 * chunks + 0.035 * factors + 0.1 * act + 0.005 * n);
+    } else if (h->dd) {
+      general += weight * (h->wide ? 0.0135 * products + 1.72e-3 * c.poly_ops[gp] : 1.98e-3 * c.poly_ops[gp]);
+      values += weight * (1.7 * chunks + 0.014 * factors + 0.035 * act + 0.005 * n);
+    } else {
+      general += weight * (2.07e-3 * c.poly_ops[gp] + 0.003 * n);
+      values += weight * (1.7 * chunks + 0.010 * factors + 0.02 * act + 0.005 * n);
+    }
+  }
+  return 1.1 * values < general;
+}
+
 // Lists, digits and buffers for a compiled system set, after everything the
 // general kernels need.  PE_OK with h->sum_L = 0 when the set does not suit
 // the kernels or the device has no room: those then evaluate every call.
@@ -667,6 +704,7 @@ int setup_sum(polyeval *h, const Compiled &c) {
     pointers += static_cast<int64_t>((t1 - t0 + pe::kSumBlock - 1) / pe::kSumBlock) * (sp[gp].act_n + 1);
     if (pointers > kSumPointersMax || act.size() > INT32_MAX / 2 || bits.size() > INT32_MAX / 2) return PE_OK;
   }
+  if (!sum_pays(h, c, sp)) return PE_OK;
   // per system: magnitude range, headroom
   int m_max = 1, act_most = 1;
   for (int s = 0; s < S; s++) {
@@ -893,6 +931,16 @@ int setup_sum(polyeval *h, const Compiled &c) {
   return PE_OK;
 }
 
+// Without host memory for the lists the handle does without them.
+int try_setup_sum(polyeval *h, const Compiled &c) {
+  try {
+    return setup_sum(h, c);
+  } catch (const std::bad_alloc &) {
+    h->sum_L = 0;
+    return PE_OK;
+  }
+}
+
 // Points per tile (log2) of a single-system call: the handle's choice, or as
 // few as it takes to give every SM a (polynomial, tile) item.
 int sum_tile_log2(const polyeval *h, int64_t P) {
@@ -1069,7 +1117,7 @@ int polyeval_create(const pe_system *sys, int precision, uint32_t flags, int64_t
         return rc;
       }
     }
-    if ((rc = setup_sum(h, c)) != PE_OK) {
+    if ((rc = try_setup_sum(h, c)) != PE_OK) {
       delete h;
       return rc;
     }
@@ -1169,7 +1217,7 @@ int polyeval_create_many(const pe_system *systems, int32_t count, int precision,
         return rc;
       }
     }
-    if ((rc = setup_sum(h, c)) != PE_OK) {
+    if ((rc = try_setup_sum(h, c)) != PE_OK) {
       delete h;
       return rc;
     }
@@ -1335,7 +1383,7 @@ int eval_single(polyeval *h, const void *points, int64_t P, void *out_f, void *o
   mp.scratch_J = C > 1 ? mp.scratch_f + static_cast<size_t>(C - 1) * f_doubles : nullptr;
   mp.n_items = base * C;
   if (mp.n_items > INT32_MAX) return PE_ERANGE;  // the work counter is 32-bit
-  mp.finish = C == 1;
+  mp.finish = by_values && C == 1;
   pe::Only only{nullptr, nullptr, static_cast<int32_t>(P)};
   if (by_values) {
     mp.any = only.any = sum_any(h);
@@ -1345,7 +1393,7 @@ int eval_single(polyeval *h, const void *points, int64_t P, void *out_f, void *o
   }
   int rc = run_main(h, mp, s, mode);
   if (rc != PE_OK) return rc;
-  if (C > 1 && h->qd) {  // add the chunks' accumulators, round to quad-double
+  if (h->qd && !mp.finish) {  // add the chunks' accumulators, round to quad-double
     if (pe::launch_finalize_qd(mp.out_f, mp.out_J, mp.scratch_f, mp.scratch_J, 2 * static_cast<int64_t>(d.N) * P,
                                2 * static_cast<int64_t>(d.N) * d.n * P, C, only, s) != cudaSuccess)
       return PE_ECUDA;
@@ -1411,7 +1459,7 @@ int eval_many(polyeval *h, const void *points, void *out_f, void *out_J, cudaStr
   mp.scratch_f = static_cast<double *>(h->scratch.p);
   mp.scratch_J = C > 1 ? mp.scratch_f + static_cast<size_t>(C - 1) * f_doubles : nullptr;
   mp.n_items = h->n_items_batch * C;
-  mp.finish = C == 1;
+  mp.finish = by_values && C == 1;
   if (by_values) {
     mp.any = sum_any(h);
     mp.flags = sum_flags(h);
@@ -1421,7 +1469,7 @@ int eval_many(polyeval *h, const void *points, void *out_f, void *out_J, cudaStr
   const int rc = run_main(h, mp, s, by_values ? 2 : std::max(mode, 0));
   if (rc != PE_OK) return rc;
   const pe::Only every{};
-  if (C > 1 && h->qd) {  // add the chunks' accumulators, round to quad-double
+  if (h->qd && !mp.finish) {  // add the chunks' accumulators, round to quad-double
     if (pe::launch_finalize_qd(mp.out_f, mp.out_J, mp.scratch_f, mp.scratch_J, 2 * h->f_total_batch,
                                2 * h->J_total_batch, C, every, s) != cudaSuccess)
       return PE_ECUDA;

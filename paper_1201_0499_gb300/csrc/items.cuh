@@ -26,8 +26,11 @@ struct Item {
   double *J_base;      // output (or scratch) base for J
 };
 
-// Returns false for an item to skip: one without a flagged point in a call
-// that evaluates only those, or an inconsistent one (flags the status word).
+// kSome: a launch that evaluates only flagged points (kernels of its own: the
+// code for it would take registers from the others).
+// Returns false for an item to skip: one without a flagged point in such a
+// launch, or an inconsistent one (flags the status word).
+template <bool kSome>
 __device__ __forceinline__ bool decode_item(const MainParams &kp, unsigned item, int lane, Item &it) {
   int chunk = 0;
   if (kp.single_P >= 0) {
@@ -56,7 +59,7 @@ __device__ __forceinline__ bool decode_item(const MainParams &kp, unsigned item,
     if (lane == 0) atomicOr(kp.status, 1);
     return false;
   }
-  if (kp.flags) {
+  if constexpr (kSome) {
     // flagged points only; few of them spread over the warp's monomial
     // groups: the most groups whose sub-tile holds them all
     const int tp = kPointsPerWarp / it.groups, q = it.tile * tp + lane;

@@ -49,7 +49,7 @@ __device__ __forceinline__ void accumulate(double *p, int c, bool valid, typenam
 
 // One work item: polynomial gp (global index) of system s at the points of
 // `tile`.  smem: this warp's prefix-product slots, [slot][lane].
-template <class A>
+template <class A, bool kSome>
 __device__ void process_item(const MainParams &kp, const Item &it, typename A::V *smem, int lane) {
   const int gp = it.gp, tile = it.tile, s = it.s, P = it.P;
   using V = typename A::V;
@@ -58,7 +58,7 @@ __device__ void process_item(const MainParams &kp, const Item &it, typename A::V
   const SysDesc sd = kp.sys[s];
   const int n = sd.n;
   const int q = tile * kPointsPerWarp + (lane >> 1);
-  const bool valid = q < P && (!kp.flags || kp.flags[sd.fl_off + q]);
+  const bool valid = q < P && (!kSome || kp.flags[sd.fl_off + q]);
   const int qc = min(q, P - 1);  // lanes past the end compute on the last point and store nothing
   const int c = lane & 1;
   const unsigned long long sgn = c ? 0ULL : kSign;
@@ -144,7 +144,7 @@ __device__ void process_item(const MainParams &kp, const Item &it, typename A::V
 // Each group keeps its derivative terms in its slots and the groups add them
 // into the row J[p, :] one after another (two monomials of a round may share
 // a variable); f is summed per group and across the groups at the end.
-template <class A, int G>
+template <class A, int G, bool kSome>
 __device__ void process_item_groups(const MainParams &kp, const Item &it, typename A::V *smem, int lane) {
   constexpr int GL = 32 / G;                     // lanes per group
   constexpr int QP = kPointsPerWarp / G;         // points per tile
@@ -156,7 +156,7 @@ __device__ void process_item_groups(const MainParams &kp, const Item &it, typena
   const int n = sd.n;
   const int g = lane / GL;
   const int q = tile * QP + ((lane % GL) >> 1);
-  const bool valid = q < P && (!kp.flags || kp.flags[sd.fl_off + q]);
+  const bool valid = q < P && (!kSome || kp.flags[sd.fl_off + q]);
   const int qc = min(q, P - 1);
   const int c = lane & 1;
   const unsigned long long sgn = c ? 0ULL : kSign;
@@ -248,20 +248,17 @@ __global__ void main_kernel(const MainParams kp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   typename A::V *smem = reinterpret_cast<typename A::V *>(smem_raw) + static_cast<size_t>(warp) * kp.kslots * 32;
-  let_next_start();
-  wait_for_previous();
-  if (kp.any && *kp.any == 0) return;
   for (;;) {
     unsigned item = 0;
     if (lane == 0) item = atomicAdd(kp.counter, 1u);
     item = __shfl_sync(kFull, item, 0);
     if (static_cast<int64_t>(item) >= kp.n_items) break;
     Item it;
-    if (!decode_item(kp, item, lane, it)) continue;
+    if (!decode_item<false>(kp, item, lane, it)) continue;
     if constexpr (G == 1)
-      process_item<A>(kp, it, smem, lane);
+      process_item<A, false>(kp, it, smem, lane);
     else
-      process_item_groups<A, G>(kp, it, smem, lane);
+      process_item_groups<A, G, false>(kp, it, smem, lane);
   }
 }
 
@@ -371,27 +368,29 @@ cudaError_t launch_powers(bool dd, const PowerParams &p, cudaStream_t s) {
 // Each item with its own number of monomial groups: batch handles (the last,
 // partial tile of a system spreads its few points over the warp) and calls
 // that evaluate flagged points only.
-template <class A>
+template <class A, bool kSome>
 __global__ void main_kernel_batch(const MainParams kp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   typename A::V *smem = reinterpret_cast<typename A::V *>(smem_raw) + static_cast<size_t>(warp) * kp.kslots * 32;
-  let_next_start();
-  wait_for_previous();
-  if (kp.any && *kp.any == 0) return;
+  if constexpr (kSome) {
+    let_next_start();
+    wait_for_previous();
+    if (*kp.any == 0) return;
+  }
   for (;;) {
     unsigned item = 0;
     if (lane == 0) item = atomicAdd(kp.counter, 1u);
     item = __shfl_sync(kFull, item, 0);
     if (static_cast<int64_t>(item) >= kp.n_items) break;
     Item it;
-    if (!decode_item(kp, item, lane, it)) continue;
+    if (!decode_item<kSome>(kp, item, lane, it)) continue;
     switch (it.groups) {
-      case 2: process_item_groups<A, 2>(kp, it, smem, lane); break;
-      case 4: process_item_groups<A, 4>(kp, it, smem, lane); break;
-      case 8: process_item_groups<A, 8>(kp, it, smem, lane); break;
-      case 16: process_item_groups<A, 16>(kp, it, smem, lane); break;
-      default: process_item<A>(kp, it, smem, lane); break;
+      case 2: process_item_groups<A, 2, kSome>(kp, it, smem, lane); break;
+      case 4: process_item_groups<A, 4, kSome>(kp, it, smem, lane); break;
+      case 8: process_item_groups<A, 8, kSome>(kp, it, smem, lane); break;
+      case 16: process_item_groups<A, 16, kSome>(kp, it, smem, lane); break;
+      default: process_item<A, kSome>(kp, it, smem, lane); break;
     }
   }
 }
@@ -404,7 +403,8 @@ cudaError_t prepare_main_t(int v) {
       (e = cudaFuncSetAttribute(main_kernel<A, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, v)) ||
       (e = cudaFuncSetAttribute(main_kernel<A, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, v)) ||
       (e = cudaFuncSetAttribute(main_kernel<A, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, v)) ||
-      (e = cudaFuncSetAttribute(main_kernel_batch<A>, cudaFuncAttributeMaxDynamicSharedMemorySize, v)))
+      (e = cudaFuncSetAttribute(main_kernel_batch<A, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, v)) ||
+      (e = cudaFuncSetAttribute(main_kernel_batch<A, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, v)))
     return e;
   return cudaSuccess;
 }
@@ -419,8 +419,8 @@ cudaError_t prepare_main(bool dd, size_t smem_bytes) {
 cudaError_t main_occupancy(bool dd, bool batch, int warps_per_block, size_t smem_bytes, int *blocks_per_sm) {
   const int t = warps_per_block * 32;
   if (batch)
-    return dd ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, main_kernel_batch<ArithDD>, t, smem_bytes)
-              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, main_kernel_batch<ArithF64>, t, smem_bytes);
+    return dd ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, main_kernel_batch<ArithDD, false>, t, smem_bytes)
+              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, main_kernel_batch<ArithF64, false>, t, smem_bytes);
   return dd ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, main_kernel<ArithDD, 1>, t, smem_bytes)
             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, main_kernel<ArithF64, 1>, t, smem_bytes);
 }
@@ -428,9 +428,9 @@ cudaError_t main_occupancy(bool dd, bool batch, int warps_per_block, size_t smem
 template <class A>
 cudaError_t launch_main_t(const MainParams &p, int warps_per_block, size_t smem_bytes, int grid, cudaStream_t s) {
   const dim3 b(warps_per_block * 32);
-  if (p.any && (p.single_P < 0 || p.regroup)) return launch_next(main_kernel_batch<A>, dim3(grid), b, smem_bytes, s, p);
+  if (p.any) return launch_next(main_kernel_batch<A, true>, dim3(grid), b, smem_bytes, s, p);
   if (p.single_P < 0) {
-    main_kernel_batch<A><<<grid, b, smem_bytes, s>>>(p);
+    main_kernel_batch<A, false><<<grid, b, smem_bytes, s>>>(p);
     return cudaGetLastError();
   }
   switch (p.groups) {

@@ -119,12 +119,13 @@ __device__ __forceinline__ void store_rounded(double *p, const Acc &a) {
   reinterpret_cast<double2 *>(p)[1] = make_double2(o[2], o[3]);
 }
 
+template <bool kSome>
 __device__ void process_item_qd(const MainParams &kp, const Item &it, uint32_t *slots, int lane) {
   const int gp = it.gp, tile = it.tile, s = it.s, P = it.P;
   const SysDesc sd = kp.sys[s];
   const int n = sd.n;
   const int q = tile * kPointsPerWarp + (lane >> 1);
-  const bool valid = q < P && (!kp.flags || kp.flags[sd.fl_off + q]);
+  const bool valid = q < P && (!kSome || kp.flags[sd.fl_off + q]);
   const int qc = min(q, P - 1);
   const int c = lane & 1;
   const size_t Pz = static_cast<size_t>(P);
@@ -185,7 +186,7 @@ __device__ void process_item_qd(const MainParams &kp, const Item &it, uint32_t *
   }
   if (!valid) return;
   double *fp = it.f_base + (static_cast<size_t>(sd.f_off) + static_cast<size_t>(pl) * Pz + q) * kQdDoubles + 4 * c;
-  if (!kp.finish) {
+  if (!kSome || !kp.finish) {
     qd::store_acc(fp, f);
     return;
   }
@@ -197,21 +198,25 @@ __device__ void process_item_qd(const MainParams &kp, const Item &it, uint32_t *
   }
 }
 
-__global__ void __launch_bounds__(kWarpsPerBlockMax * 32) main_qd(const MainParams kp) {
+// 72 registers (28 warps per SM): at 80 small polynomials take 5 % longer.
+template <bool kSome>
+__global__ void __launch_bounds__(kWarpsPerBlockMax * 32, kSome ? 1 : 7) main_qd(const MainParams kp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t *slots = reinterpret_cast<uint32_t *>(smem_raw) + static_cast<size_t>(warp) * kp.kslots * kQdSlotWords * 32;
-  let_next_start();
-  wait_for_previous();
-  if (kp.any && *kp.any == 0) return;
+  if constexpr (kSome) {
+    let_next_start();
+    wait_for_previous();
+    if (*kp.any == 0) return;
+  }
   for (;;) {
     unsigned item = 0;
     if (lane == 0) item = atomicAdd(kp.counter, 1u);
     item = __shfl_sync(0xffffffffu, item, 0);
     if (static_cast<int64_t>(item) >= kp.n_items) break;
     Item it;
-    if (!decode_item(kp, item, lane, it)) continue;
-    process_item_qd(kp, it, slots, lane);
+    if (!decode_item<kSome>(kp, item, lane, it)) continue;
+    process_item_qd<kSome>(kp, it, slots, lane);
   }
 }
 
@@ -255,17 +260,19 @@ cudaError_t launch_powers_qd(const PowerParams &p, cudaStream_t s) {
 }
 
 cudaError_t prepare_main_qd(size_t smem_bytes) {
-  return cudaFuncSetAttribute(main_qd, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes));
+  const int v = static_cast<int>(smem_bytes);
+  const cudaError_t e = cudaFuncSetAttribute(main_qd<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(main_qd<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
 }
 
 cudaError_t main_qd_occupancy(int warps_per_block, size_t smem_bytes, int *blocks_per_sm) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, main_qd, warps_per_block * 32, smem_bytes);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, main_qd<false>, warps_per_block * 32, smem_bytes);
 }
 
 cudaError_t launch_main_qd(const MainParams &p, int warps_per_block, size_t smem_bytes, int grid, cudaStream_t s) {
   if (p.n_items <= 0) return cudaSuccess;
-  if (p.any) return launch_next(main_qd, dim3(grid), dim3(warps_per_block * 32), smem_bytes, s, p);
-  main_qd<<<grid, warps_per_block * 32, smem_bytes, s>>>(p);
+  if (p.any) return launch_next(main_qd<true>, dim3(grid), dim3(warps_per_block * 32), smem_bytes, s, p);
+  main_qd<false><<<grid, warps_per_block * 32, smem_bytes, s>>>(p);
   return cudaGetLastError();
 }
 

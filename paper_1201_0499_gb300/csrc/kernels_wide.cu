@@ -110,13 +110,13 @@ __device__ __forceinline__ void accumulate_dd(double *p, int c, bool valid, dd x
 // DRAM) latency overlaps the current product's carry chains; this holds about
 // 30 more registers per thread, which pays where shared memory already limits
 // the resident warps (large k) and costs occupancy where it does not.
-template <bool Pf>
+template <bool Pf, bool kSome>
 __device__ void process_item_wide(const MainParams &kp, const Item &it, uint32_t *slots, int lane) {
   const int gp = it.gp, tile = it.tile, s = it.s, P = it.P;
   const SysDesc sd = kp.sys[s];
   const int n = sd.n;
   const int q = tile * kPointsPerWarp + (lane >> 1);
-  const bool valid = q < P && (!kp.flags || kp.flags[sd.fl_off + q]);
+  const bool valid = q < P && (!kSome || kp.flags[sd.fl_off + q]);
   const int qc = min(q, P - 1);
   const int c = lane & 1;
   const size_t Pz = static_cast<size_t>(P);
@@ -261,22 +261,24 @@ __device__ void process_item_wide(const MainParams &kp, const Item &it, uint32_t
   }
 }
 
-template <bool Pf>
+template <bool Pf, bool kSome>
 __global__ void __launch_bounds__(kWarpsPerBlockMax * 32) main_wide(const MainParams kp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t *slots = reinterpret_cast<uint32_t *>(smem_raw) + static_cast<size_t>(warp) * kp.kslots * kSlotWords * 32;
-  let_next_start();
-  wait_for_previous();
-  if (kp.any && *kp.any == 0) return;
+  if constexpr (kSome) {
+    let_next_start();
+    wait_for_previous();
+    if (*kp.any == 0) return;
+  }
   for (;;) {
     unsigned item = 0;
     if (lane == 0) item = atomicAdd(kp.counter, 1u);
     item = __shfl_sync(0xffffffffu, item, 0);
     if (static_cast<int64_t>(item) >= kp.n_items) break;
     Item it;
-    if (!decode_item(kp, item, lane, it)) continue;
-    process_item_wide<Pf>(kp, it, slots, lane);
+    if (!decode_item<kSome>(kp, item, lane, it)) continue;
+    process_item_wide<Pf, kSome>(kp, it, slots, lane);
   }
 }
 
@@ -298,27 +300,31 @@ cudaError_t launch_powers_wide(const PowerParams &p, cudaStream_t s) {
 }
 
 cudaError_t prepare_main_wide(size_t smem_bytes) {
-  const cudaError_t e =
-      cudaFuncSetAttribute(main_wide<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(main_wide<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes));
+  const int v = static_cast<int>(smem_bytes);
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(main_wide<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, v)) ||
+      (e = cudaFuncSetAttribute(main_wide<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, v)) ||
+      (e = cudaFuncSetAttribute(main_wide<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, v)) ||
+      (e = cudaFuncSetAttribute(main_wide<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, v)))
+    return e;
+  return cudaSuccess;
 }
 
 cudaError_t main_wide_occupancy(bool prefetch, int warps_per_block, size_t smem_bytes, int *blocks_per_sm) {
-  return prefetch ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, main_wide<true>, warps_per_block * 32,
+  return prefetch ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, main_wide<true, false>, warps_per_block * 32,
                                                                   smem_bytes)
-                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, main_wide<false>, warps_per_block * 32,
+                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, main_wide<false, false>, warps_per_block * 32,
                                                                   smem_bytes);
 }
 
 cudaError_t launch_main_wide(const MainParams &p, int warps_per_block, size_t smem_bytes, int grid, cudaStream_t s) {
   if (p.n_items <= 0) return cudaSuccess;
   if (p.any)
-    return launch_next(p.prefetch ? main_wide<true> : main_wide<false>, dim3(grid), dim3(warps_per_block * 32), smem_bytes, s, p);
+    return launch_next(p.prefetch ? main_wide<true, true> : main_wide<false, true>, dim3(grid), dim3(warps_per_block * 32), smem_bytes, s, p);
   if (p.prefetch)
-    main_wide<true><<<grid, warps_per_block * 32, smem_bytes, s>>>(p);
+    main_wide<true, false><<<grid, warps_per_block * 32, smem_bytes, s>>>(p);
   else
-    main_wide<false><<<grid, warps_per_block * 32, smem_bytes, s>>>(p);
+    main_wide<false, false><<<grid, warps_per_block * 32, smem_bytes, s>>>(p);
   return cudaGetLastError();
 }
 

@@ -79,7 +79,7 @@ SHAPES = [  # n, N, m, kmin, kmax, emax, P
     (40, 2, 130, 1, 3, 2, 9),   # variables that do not occur
     (6, 1, 257, 2, 6, 3, 2),
     (33, 1, 5, 33, 33, 1, 6),
-    (70, 700, 2, 1, 2, 2, 7),   # many polynomials: runs that share a table
+    (70, 700, 6, 3, 6, 2, 7),   # many polynomials: runs that share a table
     (128, 2, 70, 20, 32, 4, 5),  # a large table: fewer points per tile
     (300, 1, 40, 2, 5, 12, 3),  # a table that outgrows shared memory in quad-double
 ]
