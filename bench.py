@@ -16,9 +16,8 @@ collective on the data path); the reported time is the maximum over ranks and
 double-double oracle on the host cores on bounded samples of the same
 workload instead.
 
-Besides the headline (double-double on the FP64 pipe) the line carries the
-same workload in complex double, in double-double with integer-pipe products
-and in quad-double, and under "secondary" the smaller workloads: n = 32 at
+Besides the headline (double-double) the line carries the
+same workload in complex double, with `PE_DD_INT` handles and in quad-double, and under "secondary" the smaller workloads: n = 32 at
 1024 points (with Newton steps, the paper's three-kernel design and path
 tracking), n = 64 at 4096 points, and the batch of 200 uneven systems in one
 launch.
@@ -26,7 +25,6 @@ launch.
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import os
 import statistics
@@ -49,26 +47,12 @@ WORKLOAD = ("n=128 variables, 128 polynomials, m=1024 monomials, k=32, exponents
 L2_FLUSH_BYTES = 256 << 20
 SMS = 152
 DFMA_PER_SM_CLK = 2  # nominal FP64 FMA lanes per SM per clock on GB300
-
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch
-# of the double-double main kernel on the first 512 points of the n = 128
-# workload, from one ncu capture, per point: a launch's traffic grows with its
-# points (points and power table in, f and J out, the J rows read and written
-# while they are summed), so it scales to the 16384-point launch by the points.
-# The figure belongs to the kernel sources it was taken on (their fingerprint,
-# kernel_sources_sha()); with other sources the line reports null.
-MAIN_TRAFFIC_PER_POINT = (19_233_778_176 + 35_684_915_200) / 512  # read + write bytes of the capture / points
-MAIN_TRAFFIC_SOURCES = "daec4a2983d22163"
-KERNEL_SOURCES = ("kernels.cu", "dd.cuh", "arith.cuh", "items.cuh", "internal.h")
-
-
-def kernel_sources_sha() -> str:
-    h = hashlib.sha256()
-    for name in KERNEL_SOURCES:
-        with open(os.path.join(ROOT, "paper_1201_0499_gb300", "csrc", name), "rb") as fh:
-            h.update(fh.read())
-    return h.hexdigest()[:16]
-
+# 64-bit integer multiply-adds (32 x 32 + 64 bits): lanes per SM and clock, as
+# measured with a loop of independent ones, and the number one complex product
+# takes in the evaluation from values (4 L (L + 1) / 2 for numbers of L digits)
+IMAD_PER_SM_CLK = 32
+IMAD_PER_PRODUCT = {"dd": 40, "ddint": 40, "f64": 24, "qd": 144}
+DD_TEXT = "products of four 30-bit integer digits per part, sums in integers of six 32-bit words"
 
 def env_dist():
     rank = int(os.environ.get("RANK", "0"))
@@ -239,7 +223,7 @@ def buf_fmt(prec):
 
 class Workload:
     """The batch one step evaluates, with an evaluator per precision
-    ("dd": double-double on the FP64 pipe, "ddint": integer-pipe products,
+    ("dd" and "ddint": PE_DD and PE_DD_INT handles, which differ in the general kernels,
     "f64": complex double, "qd": quad-double on the integer pipes, on the same
     data widened by two random lower parts), device buffers and, with
     `host`, pinned host buffers for the end-to-end leg."""
@@ -334,11 +318,17 @@ class Workload:
         return self.pkg.polyeval_autotune(self.handle(prec), x, self.points, f, J, stream)
 
     def cost_per_launch(self, prec):
-        """FP64 instructions and flops of one main-kernel launch."""
+        """FP64 instructions and flops of the fused FP64 kernel for one step."""
         if self.cfg == 4:
             return self.ev[prec].cost()  # a batch handle reports whole-evaluation totals
         ops, flops = self.ev[prec].cost()
         return ops * self.points, flops * self.points
+
+    def products(self):
+        """Complex products of one step: one per variable of a monomial and point."""
+        if self.cfg == 4:
+            return sum(float(s_.mono_ptr[-1]) * p_.shape[1] for s_, p_ in zip(self.system, self.pts))
+        return float(self.system.mono_ptr[-1]) * self.points
 
     def close(self):
         for ev in self.ev.values():
@@ -394,8 +384,8 @@ TRACK_N = 10  # variables of the path-tracking system (dense quadrics: 2^10 path
 def track_leg(pkg, torch):
     """Solve a generic system of TRACK_N dense quadrics (every monomial of
     degree <= 2) by following all 2^TRACK_N paths of the total-degree
-    homotopy: in double, in double-double (evaluations on the FP64 pipe and
-    on the integer pipes; linear solves in double with double-double
+    homotopy: in double, in double-double (PE_DD and PE_DD_INT handles;
+    linear solves in double with double-double
     residuals), and adaptively (double, then double-double refinement and
     re-tracking of failed paths)."""
     s = synth.dense_system(synth.SEED_BASE + 700, TRACK_N, [2] * TRACK_N)
@@ -492,8 +482,8 @@ def secondary(cfg, pkg, torch, timer, rank, world, dev, dist, reps, sm_max):
     for prec in PRECS:
         ms[prec] = leg_ms(timer, wl, prec, 1, reps, dist)
         out[prec] = {"evals_per_s": job_throughput(world, wl.points, ms[prec]), "ms_per_step": ms[prec]}
-    ops, _flops = wl.cost_per_launch("dd")
-    out["dd"]["fp64_issue_frac_of_step"] = ops / (ms["dd"] * 1e-3) / (SMS * DFMA_PER_SM_CLK * sm_max * 1e6)
+    out["dd"]["imad_frac_of_step"] = (wl.products() * IMAD_PER_PRODUCT["dd"] / (ms["dd"] * 1e-3)
+                                      / (SMS * IMAD_PER_SM_CLK * sm_max * 1e6))
     out["dd_fp64_time_ratio"] = ms["dd"] / ms["f64"]
     out["ddint_speedup_vs_fp64_dd"] = ms["dd"] / ms["ddint"]
     for prec in PRECS:
@@ -536,8 +526,8 @@ def main():
     ap.add_argument("--reference-points", type=int, default=REFERENCE_POINTS_PER_STEP,
                     help="points of the workload the oracle arm evaluates per step")
     ap.add_argument("--precision", default="dd", choices=["dd", "ddint"],
-                    help="dd: double-double on the FP64 pipe; ddint: products in 128-bit integer block "
-                         "floating point, sums in double-double (same inputs, outputs and accuracy bar)")
+                    help="dd: PE_DD handles; ddint: PE_DD_INT handles (same inputs, outputs and accuracy bar; "
+                         "they differ where the general kernels evaluate)")
     ap.add_argument("--graph", action="store_true",
                     help="replay the evaluation from a captured CUDA graph in the timed steps")
     ap.add_argument("--no-secondary", action="store_true", help="skip the smaller workloads")
@@ -672,10 +662,18 @@ def main():
     ms_per_step = max_over_ranks(total_ms / args.steps, dist)
     value = job_throughput(world, P, ms_per_step)
 
-    # roofline of the main (monomial) kernel: FP64 pipe bound
-    ops_launch, flops_launch = wl.cost_per_launch(prim)
+    # roofline of the monomial kernels (sum_kernel, and the general kernel's
+    # pass over the flags): bound by the 64-bit integer multiply-adds of the
+    # products, one product per variable of a monomial
     kern_avg_ms = kern_ms / max(launches, 1)
-    achieved_tflops = flops_launch / (kern_avg_ms * 1e-3) / 1e12
+    imads = wl.products() * IMAD_PER_PRODUCT[prim]
+    achieved_tops = 2 * imads / (kern_avg_ms * 1e-3) / 1e12
+    peak_tops = SMS * IMAD_PER_SM_CLK * 2 * sm_max * 1e6 / 1e12
+    # what the fused FP64 kernel (forward and backward products) would execute
+    # for the same evaluations, per second of this kernel: an equivalent, not
+    # a utilisation of the FP64 pipe, which is nearly idle here
+    _ops_launch, flops_launch = wl.cost_per_launch(prim)
+    fp64_equiv_tflops = flops_launch / (kern_avg_ms * 1e-3) / 1e12
     peak_nominal = SMS * DFMA_PER_SM_CLK * 2 * sm_max * 1e6 / 1e12
     # the paper's method at its own cost (6k - 5 complex products and k + 1
     # complex sums per monomial, dd product 88 flops, dd sum 40): what the same
@@ -683,11 +681,6 @@ def main():
     nominal_flops = nominal_paper_flops(wl.system, P) if cfg != 4 else None
     fma_rate, probe_mhz = pkg.polyeval_fp64_peak(stream)
     peak_probe = 2 * fma_rate / 1e12
-    issue_rate = ops_launch / (kern_avg_ms * 1e-3)
-    traffic = None
-    if (cfg == CONFIG_INDEX and prim == "dd" and MAIN_TRAFFIC_PER_POINT is not None
-            and MAIN_TRAFFIC_SOURCES == kernel_sources_sha()):
-        traffic = MAIN_TRAFFIC_PER_POINT * P
     paper_tflops = nominal_flops / (kern_avg_ms * 1e-3) / 1e12 if nominal_flops else None
 
     # complex double path and the other double-double paths on the same
@@ -734,8 +727,7 @@ def main():
         "dtype": "f64",
         "data": "synthetic",
         "config": {"workload": wl.text, "points_per_gpu": P, "gpu": torch.cuda.get_device_name(dev),
-                   "precision": ("complex double-double" if prim == "dd" else
-                                 "complex double-double in/out, products in 128-bit integer block floating point"),
+                   "precision": "complex double-double in/out, " + DD_TEXT,
                    "l2": "flushed between timed steps (256 MiB write outside the step events); the step's "
                          "outputs alone exceed the L2",
                    "cuda_graph": bool(args.graph),
@@ -746,37 +738,34 @@ def main():
                 "h2d_bytes_per_step": wl.h2d_bytes, "d2h_bytes_per_step": wl.d2h_bytes, "steps": e2e_steps,
                 "what": "polyeval_eval_host: pinned host points in, pinned host f and J out, synchronous"},
         "gpu_launches": kernels,
-        "roofline": {"bound": "alu", "achieved": achieved_tflops, "peak": peak_nominal, "unit": "TFLOP/s",
-                     "frac": achieved_tflops / peak_nominal, "traffic": traffic,
-                     "traffic_basis": ("ncu DRAM bytes per point of a 512-point launch of the same kernel on this "
-                                       "workload, times the points" if traffic is not None else
-                                       "no capture on the current kernel sources"),
-                     "kernel": "main_kernel<ArithDD>" if prim == "dd" else "main_wide",
-                     "kernel_ms": kern_avg_ms,
-                     "achieved_basis": "FP64 flops the kernel executes (polyeval_cost: FMA = 2, add and "
-                                       "multiply = 1), equal to the ncu instruction count",
-                     "peak_basis": f"nominal: {SMS} SMs x {DFMA_PER_SM_CLK} FP64 FMA/clk x 2 flops x {sm_max:.0f} MHz",
-                     "peak_probe": peak_probe, "frac_of_probe": achieved_tflops / peak_probe,
+        "roofline": {"bound": "alu", "achieved": achieved_tops, "peak": peak_tops, "unit": "TOP/s",
+                     "frac": achieved_tops / peak_tops, "traffic": None,
+                     "traffic_basis": "no DRAM capture of this kernel",
+                     "kernel": "sum_kernel", "kernel_ms": kern_avg_ms,
+                     "achieved_basis": f"64-bit integer multiply-adds of the products ({IMAD_PER_PRODUCT[prim]} each, "
+                                       "one product per variable of a monomial and point; counted as 2 operations), "
+                                       "not those of the rescaling and the sums",
+                     "peak_basis": f"{SMS} SMs x {IMAD_PER_SM_CLK} multiply-adds/clk (measured) x 2 x {sm_max:.0f} MHz",
+                     "fp64_peak_nominal_tflops": peak_nominal, "fp64_peak_probe_tflops": peak_probe,
                      "probe_sm_mhz": probe_mhz,
-                     "fp64_issue_frac": issue_rate / (SMS * DFMA_PER_SM_CLK * sm_max * 1e6),
+                     "fp64_method_equiv_tflops": fp64_equiv_tflops,
                      "paper_method_equiv_tflops": paper_tflops,
                      "paper_method_frac": paper_tflops / peak_nominal if paper_tflops else None},
-        "fp64_path": {"evals_per_s": job_throughput(world, P, ms64), "ms_per_step": ms64,
-                      # FP64 instructions of the step's main kernel over the whole step time
-                      "fp64_issue_frac": (wl.cost_per_launch("f64")[0] / (ms64 * 1e-3)
-                                          / (SMS * DFMA_PER_SM_CLK * sm_max * 1e6))},
+        "fp64_path": {"evals_per_s": job_throughput(world, P, ms64), "ms_per_step": ms64},
         "dd_fp64_time_ratio": ms_dd / ms64,
         ("int_pipe_path" if other == "ddint" else "fp64_dd_path"): {
             "evals_per_s": job_throughput(world, P, legs[other]), "ms_per_step": legs[other],
             "speedup_vs_fp64_dd": (ms_per_step / legs[other]) if other == "ddint" else (legs[other] / ms_per_step),
-            "precision": ("complex double-double in/out, products in 128-bit integer block floating point, "
-                          "sums in double-double" if other == "ddint" else "complex double-double on the FP64 pipe")},
+            "precision": "complex double-double in/out, " + DD_TEXT},
         "qd_int_path": {
             "evals_per_s": job_throughput(world, P, legs["qd"]), "ms_per_step": legs["qd"],
             "time_vs_fp64_dd": legs["qd"] / ms_dd,
-            "precision": "complex quad-double in/out (the same data with two random lower parts), products in "
-                         "256-bit integer block floating point, sums in 224-bit integer accumulators"},
-        "fp64_peak_frac": achieved_tflops / peak_nominal,
+            "precision": "complex quad-double in/out (the same data with two random lower parts), products of "
+                         "eight 29-bit integer digits, sums in integers of ten 32-bit words"},
+        # FP64 flops of the fused FP64 kernel for the same evaluations, over the
+        # FP64 peak: above 1, since the work is done on the integer pipes
+        "fp64_peak_frac": None,
+        "fp64_method_equiv_frac": fp64_equiv_tflops / peak_nominal,
         "clocks": clocks,
     }
     if cpu is not None:

@@ -14,6 +14,14 @@
  *     prefix products and one backward running product.
  *   - Section 3.3: coefficient products and the sums into f and J.
  *
+ * Where it is the faster one, polyeval_eval and polyeval_eval_many take the
+ * derivatives from the monomials' values instead: V = c x^a, f = sum V,
+ * x_i df/dx_i = sum a_i V, with products and sums of integers on the integer
+ * pipes (all precisions).  Points that this does not suit (a zero or
+ * non-finite coordinate, exponents near the range of a double, components of
+ * one coordinate more than 2^24 apart) are evaluated by the kernels of
+ * Sections 3.1-3.3 ("general kernels") in the same call.
+ *
  * Conventions for every entry point:
  *   - Return value: PE_OK (0) or a negative PE_E* code; nothing aborts and no
  *     C++ exception crosses this interface.  polyeval_strerror() names codes.
@@ -76,15 +84,14 @@ extern "C" {
 /* ---- precisions -------------------------------------------------------- */
 #define PE_DD 0  /* complex double-double (pe_cdd in and out)  */
 #define PE_F64 1 /* complex double        (pe_c64 in and out)  */
-/* Complex double-double in and out (pe_cdd), products computed in complex
- * block floating point with 128-bit integer mantissas on the integer pipes
+/* Complex double-double in and out (pe_cdd); in the general kernels products
+ * are computed in complex block floating point with 128-bit integer mantissas on the integer pipes
  * (error about 2^-120 per product relative to the operands' magnitudes),
- * sums in double-double.  Same method and layouts as PE_DD; more accurate
- * and, on GB300 where FP64 issues about 36x slower than integer multiply-add,
- * faster. */
+ * sums in double-double (about 4x faster there than PE_DD).  The evaluation
+ * from values is the same for PE_DD and PE_DD_INT.  Same layouts as PE_DD. */
 #define PE_DD_INT 2
 /* Complex quad-double in and out (pe_cqd), the precision of the QD library
- * the paper's CPU code uses (Section 1).  Products in complex block floating
+ * the paper's CPU code uses (Section 1).  In the general kernels products in complex block floating
  * point with 256-bit integer mantissas (error about 2^-246 per product
  * relative to the operands' magnitudes); every sum in a 224-bit integer
  * accumulator per output component, kept in place in the output arrays and
@@ -192,11 +199,12 @@ PE_API int polyeval_create(const pe_system *sys, int precision, uint32_t flags, 
  *   out_J   device, [n_polys][n_vars][P] of the same element type
  *   stream  cudaStream_t the work is queued on
  * Allocates nothing, synchronises nothing, and only queues kernels and one
- * 4-byte cudaMemsetAsync, so a call can be captured in a CUDA graph.  When
+ * small cudaMemsetAsync (the work counters and a flag per point), so a call
+ * can be captured in a CUDA graph.  When the general kernels evaluate and
  * the call has few (polynomial, tile of 16 points) work items, each
  * polynomial's monomials are split into up to 8 chunks whose partial sums go
  * to handle-owned scratch (at most 256 MiB, sized at create) and are added
- * by a final kernel (for PE_QD_INT the final kernel always runs: it rounds
+ * by a final kernel (for PE_QD_INT that kernel always runs there: it rounds
  * the integer sums in the outputs to quad-double, so the outputs hold
  * intermediate sums until it completes).  Calls on one handle must not overlap on the GPU (they
  * share the power table, the scratch and the work counter).  Errors: PE_EINVAL (null handle/pointer with P > 0),
@@ -205,8 +213,9 @@ PE_API int polyeval_create(const pe_system *sys, int precision, uint32_t flags, 
 PE_API int polyeval_eval(polyeval_t *h, const void *points, int64_t P, void *out_f, void *out_J, void *stream);
 
 /*
- * Choose the launch of polyeval_eval for P points by timing the candidates on
- * the caller's data: the number of chunks the monomials of each polynomial
+ * Choose the launch of polyeval_eval's general kernels for P points by timing
+ * the candidates on the caller's data (where the evaluation from values runs,
+ * the choice serves the points it leaves to them): the number of chunks the monomials of each polynomial
  * are split into (1, 2, 4, 8, as the handle's scratch allows), the launch
  * shape (1: one single-warp block per work item, all resident at once; 2: a
  * persistent grid taking items from the work counter) and, for PE_DD and
@@ -266,7 +275,8 @@ PE_API int polyeval_set_launch(polyeval_t *h, int64_t P, int chunks, int shape, 
  *   stream  as polyeval_eval
  * The solve is LU with partial pivoting per point (pivot of largest modulus)
  * in the handle's precision (double-double for PE_DD and PE_DD_INT, double
- * for PE_F64), 4 to 32 lanes of a warp per point.  PE_QD_INT handles
+ * for PE_F64), 4 to 32 lanes of a warp per point; double-double solves with
+ * 12 <= n <= 77 run on the integer pipes, a block per point.  PE_QD_INT handles
  * evaluate f and J in quad-double and solve for dx in double-double from
  * the leading two parts of each component (mixed precision, as iterative
  * refinement: each step gains about 104 bits less log2 cond(J) until x
@@ -332,8 +342,8 @@ PE_API int polyeval_eval_many(polyeval_t *h, const void *points, void *out_f, vo
  * Work counts of the handle, per evaluation point and summed over the
  * handle's systems (for a batch: over all points of all systems, i.e. one
  * whole polyeval_eval_many):
- *   fp64_ops    double-precision instructions (add, mul, fma) the method
- *               executes, counted from the compiled system (for PE_DD_INT:
+ *   fp64_ops    double-precision instructions (add, mul, fma) the general
+ *               kernels execute, counted from the compiled system (for PE_DD_INT:
  *               those of its double-double sums; 0 for PE_QD_INT, which
  *               has none)
  *   fp64_flops  the same with an fma counted as 2 flops
@@ -344,7 +354,7 @@ PE_API int polyeval_cost(const polyeval_t *h, double *fp64_ops, double *fp64_flo
 /*
  * Timing of the main (monomial) kernel, for measurement.  With enable != 0,
  * each following eval call records a pair of CUDA events on its stream
- * around the main kernel (at most 256 pairs are kept).  polyeval_timing_read
+ * around the main kernels (from values and general; at most 256 pairs are kept).  polyeval_timing_read
  * waits for the recorded events, returns the summed kernel time in
  * milliseconds, the number of timed launches and the number of kernels the
  * eval calls queued (power table, main kernel, combine passes), and starts a
