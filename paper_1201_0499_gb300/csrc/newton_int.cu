@@ -13,7 +13,9 @@
 // factors; then the trailing entries, the right-hand side as one more column,
 // while the first warp, which takes column k + 1, goes on to the next pivot (as
 // lu.cuh: largest modulus by the leading parts, smallest row on ties) and its
-// reciprocal.  The reciprocals are kept for the back substitution.  Points with entries that are not finite or beyond
+// reciprocal.  The other warps write the multipliers out, by position: an
+// exchange does not move those of earlier steps.  The reciprocals are kept for
+// the back substitution.  Points with entries that are not finite or beyond
 // 2^(+-kMaxExp) are solved by the double-double code of lu.cuh, whose
 // overflows and NaN they keep.
 #include <cuda_runtime.h>
@@ -308,12 +310,14 @@ __global__ void __launch_bounds__(256, 2) newton_int(const NewtonParams p) {
       }
     };
     int32_t *was = row, *now = row + n;  // row order before and after the exchange of this step
+    int done = n;                        // columns eliminated
     if (warp == 0) find_pivot(0, was);
     __syncthreads();
     for (int k = 0; k < n; k++) {
       singular = is_singular != 0;  // uniform
       if (singular) {
         now = was;
+        done = k;
         break;
       }
       const int piv = pivot, pr = was[piv] * cols;
@@ -326,7 +330,6 @@ __global__ void __launch_bounds__(256, 2) newton_int(const NewtonParams p) {
         Num<4> l = el_digits(A.load(at));
         if (!is_zero(l)) fx::mul<4>(l, inv);
         A.store_num(off_l + i, l);
-        A.store(at, el_of(l));
       }
       if (tid >= split)
         for (int j = k + 1 + tid - split; j < cols; j += T - split) A.store_num(off_u + j, el_factor(A.load(pr + j)));
@@ -358,6 +361,9 @@ __global__ void __launch_bounds__(256, 2) newton_int(const NewtonParams p) {
               i++;
             }
           }
+          // the multipliers stay where step k put them (later exchanges move
+          // the columns after k only), so they go out by position, now
+          for (int r = k + 1 + t1; r < n; r += T1) to_cdd(el_of(A.load_num(off_l + r))).store(gv.Jel(r, k));
         }
       }
       __syncthreads();
@@ -390,6 +396,7 @@ __global__ void __launch_bounds__(256, 2) newton_int(const NewtonParams p) {
     // factors and solution out (a singular point keeps what was eliminated)
     for (int k = tid; k < n * cols; k += T) {
       const int i = k / cols, j = k - i * cols;
+      if (j < min(i, done)) continue;  // a multiplier, written in step j
       const bool digits = !singular && j > i && j < n;
       const CDD v = to_cdd(digits ? el_of_factor(A.load_num(row[i] * cols + j)) : A.load(row[i] * cols + j));
       v.store(j < n ? gv.Jel(i, j) : gv.bel(i));

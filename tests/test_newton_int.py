@@ -99,3 +99,22 @@ def test_singular_points_step_nowhere():
     assert np.all(dx[:, 1] == 0.0) and np.isnan(norms[1, 1]) and np.array_equal(x1[:, 1], pts[:, 1])
     for q in (0, 2):
         assert backward_error(f, J, dx, q) <= 1e-28
+
+
+@pytest.mark.parametrize("n", [12, 17, 41])
+def test_factors_stay_where_each_step_puts_them(n):
+    """out_J entry by entry: an exchange at step k moves the columns from k on
+    and leaves the multipliers of earlier steps.  Tolerance: elimination in
+    complex double errs by n growth 2^-53 max|J| / |pivot| in a multiplier,
+    below 41 x 10 x 1.1e-16 x 1e3 = 5e-11; taken as 1e-9 of max|J|."""
+    s = linear_plus_square(740 + n, n)
+    f, J, dx, lu, norms, x1 = newton(s, synth.points(741 + n, n, 2))
+    for q in range(2):
+        a = J[:, :, q, 0] + 1j * J[:, :, q, 2]
+        scale = np.abs(a).max()
+        for k in range(n):
+            p = k + int(np.argmax(np.abs(a[k:, k])))
+            a[[k, p], k:] = a[[p, k], k:]
+            a[k + 1:, k] /= a[k, k]
+            a[k + 1:, k + 1:] -= np.outer(a[k + 1:, k], a[k, k + 1:])
+        assert np.abs(lu[:, :, q, 0] + 1j * lu[:, :, q, 2] - a).max() <= 1e-9 * scale
