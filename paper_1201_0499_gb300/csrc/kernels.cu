@@ -71,6 +71,9 @@ __device__ void process_item(const MainParams &kp, const Item &it, typename A::V
   auto xel = [&](int v) { return X + (static_cast<size_t>(v) * Pz + qc) * KD; };
   auto tel = [&](int e, int v) { return Tb + ((static_cast<size_t>(e - 2) * n + v) * Pz + qc) * KD; };
   auto jel = [&](int v) { return Jrow + (static_cast<size_t>(v) * Pz + qc) * KD; };
+  // In a launch over flagged points the table's kernel may still have been
+  // writing when this one started: no non-coherent loads then.
+  auto factor = [](const double *p) { return kSome ? A::load_coherent(p) : A::load_full(p); };
 
   if (valid)
     for (int v = 0; v < n; v++) A::store_comp(jel(v), c, A::zero());
@@ -98,19 +101,19 @@ __device__ void process_item(const MainParams &kp, const Item &it, typename A::V
     for (int j = 0; j < k; j++) {
       const uint32_t w = __ldg(vw + j);
       const int v = static_cast<int>(w & 0xffffu), a = static_cast<int>(w >> 16);
-      if (a >= 2) G = chain(G, A::load_full(a == 2 ? xel(v) : tel(a - 1, v)));
+      if (a >= 2) G = chain(G, factor(a == 2 ? xel(v) : tel(a - 1, v)));
     }
     // Stage 2, forward: slot j <- G x_{i_1} ... x_{i_j}, j = 0 .. k-2
     V Pc = G;
     for (int j = 0; j < k - 1; j++) {
       smem[j * 32 + lane] = Pc;
       const int v = static_cast<int>(__ldg(vw + j) & 0xffffu);
-      Pc = chain(Pc, A::load_full(xel(v)));
+      Pc = chain(Pc, factor(xel(v)));
     }
     // value c x^a = Pc x_{i_k}; derivative by x_{i_k} = a_k Pc
     const uint32_t wl = __ldg(vw + k - 1);
     const int vl = static_cast<int>(wl & 0xffffu), al = static_cast<int>(wl >> 16);
-    const Full xl = A::load_full(xel(vl));
+    const Full xl = factor(xel(vl));
     f = A::f_add(f, mul_x<A, false>(Pc, xl, sgn, kFull));
     accumulate<A>(jel(vl), c, valid, al == 1 ? Pc : A::mul_int(Pc, int_as_double(al)));
     // Stage 2, backward: Q = x_{i_{j+2}} ... x_{i_k}; derivative by x_{i_{j+1}} = a_{j+1} slot_j Q
@@ -121,7 +124,7 @@ __device__ void process_item(const MainParams &kp, const Item &it, typename A::V
       const int v = static_cast<int>(w & 0xffffu), a = static_cast<int>(w >> 16);
       const V D = mul_split<A>(smem[j * 32 + lane], Q, c, sgn, kFull);
       accumulate<A>(jel(v), c, valid, a == 1 ? D : A::mul_int(D, int_as_double(a)));
-      if (j > 0) Q = chain(Q, A::load_full(xel(v)));
+      if (j > 0) Q = chain(Q, factor(xel(v)));
     }
   }
   if (valid) {
@@ -170,6 +173,7 @@ __device__ void process_item_groups(const MainParams &kp, const Item &it, typena
   auto xel = [&](int v) { return X + (static_cast<size_t>(v) * Pz + qc) * KD; };
   auto tel = [&](int e, int v) { return Tb + ((static_cast<size_t>(e - 2) * n + v) * Pz + qc) * KD; };
   auto jel = [&](int v) { return Jrow + (static_cast<size_t>(v) * Pz + qc) * KD; };
+  auto factor = [](const double *p) { return kSome ? A::load_coherent(p) : A::load_full(p); };  // as process_item
 
   if (valid && g == 0)
     for (int v = 0; v < n; v++) A::store_comp(jel(v), c, A::zero());
@@ -201,17 +205,17 @@ __device__ void process_item_groups(const MainParams &kp, const Item &it, typena
         for (int j = 0; j < k; j++) {
           const uint32_t w = __ldg(vw + j);
           const int v = static_cast<int>(w & 0xffffu), a = static_cast<int>(w >> 16);
-          if (a >= 2) Gv = chain(Gv, A::load_full(a == 2 ? xel(v) : tel(a - 1, v)));
+          if (a >= 2) Gv = chain(Gv, factor(a == 2 ? xel(v) : tel(a - 1, v)));
         }
         V Pc = Gv;
         for (int j = 0; j < k - 1; j++) {
           smem[j * 32 + lane] = Pc;
           const int v = static_cast<int>(__ldg(vw + j) & 0xffffu);
-          Pc = chain(Pc, A::load_full(xel(v)));
+          Pc = chain(Pc, factor(xel(v)));
         }
         const uint32_t wl = __ldg(vw + k - 1);
         const int vl = static_cast<int>(wl & 0xffffu), al = static_cast<int>(wl >> 16);
-        const Full xl = A::load_full(xel(vl));
+        const Full xl = factor(xel(vl));
         f = A::f_add(f, mul_x<A, false>(Pc, xl, sgn, pm));
         // derivative terms into the slots: slot j <- term of x_{i_{j+1}}
         V Q = A::comp(xl, c);
@@ -220,7 +224,7 @@ __device__ void process_item_groups(const MainParams &kp, const Item &it, typena
           const int a = static_cast<int>(__ldg(vw + j) >> 16);
           const V D = mul_split<A>(smem[j * 32 + lane], Q, c, sgn, pm);
           smem[j * 32 + lane] = a == 1 ? D : A::mul_int(D, int_as_double(a));
-          if (j > 0) Q = chain(Q, A::load_full(xel(static_cast<int>(__ldg(vw + j) & 0xffffu))));
+          if (j > 0) Q = chain(Q, factor(xel(static_cast<int>(__ldg(vw + j) & 0xffffu))));
         }
         smem[(k - 1) * 32 + lane] = al == 1 ? Pc : A::mul_int(Pc, int_as_double(al));
       }

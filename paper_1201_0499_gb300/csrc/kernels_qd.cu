@@ -136,6 +136,9 @@ __device__ void process_item_qd(const MainParams &kp, const Item &it, uint32_t *
 
   auto tel = [&](int e, int v) { return Tb + ((static_cast<size_t>(e - 1) * n + v) * Pz + qc) * kQdWords; };
   auto jel = [&](int v) { return Jrow + (static_cast<size_t>(v) * Pz + qc) * kQdDoubles; };
+  // In a launch over flagged points the table's kernel may still have been
+  // writing when this one started: no non-coherent loads then.
+  auto factor = [](const uint32_t *p) { return kSome ? qd::load_wf_coherent(p) : qd::load_wf(p); };
 
   if (valid)
     for (int v = 0; v < n; v++) qd::store_acc(jel(v) + 4 * c, qd::acc_zero());
@@ -155,7 +158,7 @@ __device__ void process_item_qd(const MainParams &kp, const Item &it, uint32_t *
     for (int j = 0; j < k; j++) {
       const uint32_t w = __ldg(vw + j);
       const int v = static_cast<int>(w & 0xffffu), a = static_cast<int>(w >> 16);
-      if (a >= 2) G = qd::mul_x(G, qd::load_wf(tel(a - 1, v)), c);
+      if (a >= 2) G = qd::mul_x(G, factor(tel(a - 1, v)), c);
     }
     // Stage 2, forward: P_j = G x_{i_1} ... x_{i_j}; every kp.slot_stride-th
     // one is kept (slot j / stride), the others are recomputed below
@@ -164,11 +167,11 @@ __device__ void process_item_qd(const MainParams &kp, const Item &it, uint32_t *
     for (int j = 0; j < k - 1; j++) {
       if (j % stride == 0) store_slot(slots, j / stride, lane, Pc);
       const int v = static_cast<int>(__ldg(vw + j) & 0xffffu);
-      Pc = qd::mul_x(Pc, qd::load_wf(tel(1, v)), c);
+      Pc = qd::mul_x(Pc, factor(tel(1, v)), c);
     }
     const uint32_t wl = __ldg(vw + k - 1);
     const int vl = static_cast<int>(wl & 0xffffu), al = static_cast<int>(wl >> 16);
-    const WF xl = qd::load_wf(tel(1, vl));
+    const WF xl = factor(tel(1, vl));
     qd::acc_add(f, qd::mul_x(Pc, xl, c));
     accumulate(jel(vl), c, valid, al == 1 ? Pc : qd::mul_small(Pc, static_cast<uint32_t>(al)));
     // Stage 2, backward
@@ -178,10 +181,10 @@ __device__ void process_item_qd(const MainParams &kp, const Item &it, uint32_t *
       const int v = static_cast<int>(w & 0xffffu), a = static_cast<int>(w >> 16);
       WV Pj = load_slot(slots, j / stride, lane);
       for (int r = j - j % stride; r < j; r++)  // recompute P_j from the kept P_{j - j % stride}
-        Pj = qd::mul_x(Pj, qd::load_wf(tel(1, static_cast<int>(__ldg(vw + r) & 0xffffu))), c);
+        Pj = qd::mul_x(Pj, factor(tel(1, static_cast<int>(__ldg(vw + r) & 0xffffu))), c);
       const WV D = qd::mul_pair(Pj, Q, c);
       accumulate(jel(v), c, valid, a == 1 ? D : qd::mul_small(D, static_cast<uint32_t>(a)));
-      if (j > 0) Q = qd::mul_x(Q, qd::load_wf(tel(1, v)), c);
+      if (j > 0) Q = qd::mul_x(Q, factor(tel(1, v)), c);
     }
   }
   if (!valid) return;

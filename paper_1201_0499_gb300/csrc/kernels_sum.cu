@@ -581,7 +581,9 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2
       const int4 *src = reinterpret_cast<const int4 *>(blob);
       int4 *dst = reinterpret_cast<int4 *>(stab);
       const int words = static_cast<int>(tab_bytes / 16);
-      for (int i = tid; i < words; i += NT) dst[i] = __ldg(src + i);
+      // (a plain load: sum_powers may still have been writing the table when
+      // this kernel started, which non-coherent loads do not allow)
+      for (int i = tid; i < words; i += NT) dst[i] = src[i];
       held = tile_id;
     }
     const int4 *tab = reinterpret_cast<const int4 *>(kTabShared ? stab : blob);

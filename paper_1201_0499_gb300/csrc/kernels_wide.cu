@@ -127,7 +127,10 @@ __device__ void process_item_wide(const MainParams &kp, const Item &it, uint32_t
 
   auto tel = [&](int e, int v) { return Tb + ((static_cast<size_t>(e - 1) * n + v) * Pz + qc) * kWideWords; };
   auto jel = [&](int v) { return Jrow + (static_cast<size_t>(v) * Pz + qc) * 4; };
-  auto xw = [&](const uint32_t *vw, int j) { return wide::load_wf(tel(1, static_cast<int>(__ldg(vw + j) & 0xffffu))); };
+  // In a launch over flagged points the table's kernel may still have been
+  // writing when this one started: no non-coherent loads then.
+  auto factor = [](const uint32_t *p) { return kSome ? wide::load_wf_coherent(p) : wide::load_wf(p); };
+  auto xw = [&](const uint32_t *vw, int j) { return factor(tel(1, static_cast<int>(__ldg(vw + j) & 0xffffu))); };
 
   if (valid)
     for (int v = 0; v < n; v++) reinterpret_cast<double2 *>(jel(v))[c] = make_double2(0.0, 0.0);
@@ -159,21 +162,21 @@ __device__ void process_item_wide(const MainParams &kp, const Item &it, uint32_t
         if ((w >> 16) >= 2) break;
       }
       WF xa;
-      if (j < k) xa = wide::load_wf(tel(static_cast<int>(w >> 16) - 1, static_cast<int>(w & 0xffffu)));
+      if (j < k) xa = factor(tel(static_cast<int>(w >> 16) - 1, static_cast<int>(w & 0xffffu)));
       while (j < k) {
         const WF xc = xa;
         for (j++; j < k; j++) {
           w = __ldg(vw + j);
           if ((w >> 16) >= 2) break;
         }
-        if (j < k) xa = wide::load_wf(tel(static_cast<int>(w >> 16) - 1, static_cast<int>(w & 0xffffu)));
+        if (j < k) xa = factor(tel(static_cast<int>(w >> 16) - 1, static_cast<int>(w & 0xffffu)));
         G = chain(G, xc);
       }
     } else {
       for (int j = 0; j < k; j++) {
         const uint32_t w = __ldg(vw + j);
         const int v = static_cast<int>(w & 0xffffu), a = static_cast<int>(w >> 16);
-        if (a >= 2) G = chain(G, wide::load_wf(tel(a - 1, v)));
+        if (a >= 2) G = chain(G, factor(tel(a - 1, v)));
       }
     }
     // Stage 2, forward: P_j = G x_{i_1} ... x_{i_j}; every kp.slot_stride-th
@@ -198,7 +201,7 @@ __device__ void process_item_wide(const MainParams &kp, const Item &it, uint32_t
     if constexpr (Pf)
       xl = xf;  // x_{i_k}
     else
-      xl = wide::load_wf(tel(1, vl));
+      xl = factor(tel(1, vl));
     f = add(f, wide::to_dd(wide::mul_x<false>(Pc, xl, c)));  // to_dd takes any leading bit
     accumulate_dd(jel(vl), c, valid, wide::to_dd(al == 1 ? Pc : wide::mul_small(Pc, static_cast<uint32_t>(al))));
     // Stage 2, backward.  With Pf the J entry of the next term is read one
@@ -211,7 +214,7 @@ __device__ void process_item_wide(const MainParams &kp, const Item &it, uint32_t
     if constexpr (Pf) {
       if (k >= 2) {
         const int v0 = static_cast<int>(__ldg(vw + k - 2) & 0xffffu);
-        xb = wide::load_wf(tel(1, v0));
+        xb = factor(tel(1, v0));
         jb = reinterpret_cast<const double2 *>(jel(v0))[c];
       }
     }
@@ -225,7 +228,7 @@ __device__ void process_item_wide(const MainParams &kp, const Item &it, uint32_t
         jc = jb;
         if (j > 0) {
           const int vn = static_cast<int>(__ldg(vw + j - 1) & 0xffffu);
-          xb = wide::load_wf(tel(1, vn));
+          xb = factor(tel(1, vn));
           jb = reinterpret_cast<const double2 *>(jel(vn))[c];
         }
       }
@@ -244,7 +247,7 @@ __device__ void process_item_wide(const MainParams &kp, const Item &it, uint32_t
         if (j > 0) Q = chain(Q, xc);
       } else {
         accumulate_dd(jel(v), c, valid, term);
-        if (j > 0) Q = chain(Q, wide::load_wf(tel(1, v)));
+        if (j > 0) Q = chain(Q, factor(tel(1, v)));
       }
     }
   }
