@@ -193,7 +193,7 @@ struct SumParams {
 template <int L>
 constexpr int kSumCoefWords = L == 8 ? 20 : 12;
 
-// Rows of a tile's sums and marks: (active variable, component) tasks, rounded
+// Rows of a tile's sums and their leading bits: (active variable, component) tasks, rounded
 // up to eight, and the parts of f.
 __host__ __device__ constexpr int sum_rows(int act_max) { return ((2 * act_max + 7) & ~7) + 2 * kSumParts; }
 

@@ -22,8 +22,9 @@
 //      registers (two monomials where shared memory has room for the values);
 //   -  the block agrees on the largest exponent per point, and every value is
 //      stored as a W-word two's complement integer below it (the window);
-//      (a word per sum keeps the or of its terms' bits from kKeep up: none set
-//      means terms too small for the window, see own_windows)
+//      (the leading bit of a sum's terms is kept beside it and falls with the
+//      sum when a later chunk raises the window: below kKeep, the terms were
+//      too small for the window, see own_windows)
 //   B  one thread per (variable, component, point) adds the values of the
 //      monomials that hold its variable, times the exponent, from a list made
 //      at create; four list entries at a time, without branches.  (Additions
@@ -479,10 +480,10 @@ __device__ __forceinline__ void finish_entry(uint32_t (&zr)[Fmt<L>::W], uint32_t
 
 // The entries of J at point q (of the tile) whose every term lies so far
 // below the polynomial's largest monomial that the shared window cut them
-// short (no bit in `marks`): their monomials' values once more, each sum in a
+// short (not set in `kept`): their monomials' values once more, each sum in a
 // window of its own.  Variables sub, sub + subs, ...; o: the entry of variable 0.
 template <int L>
-__device__ __forceinline__ void own_windows(const SumParams &sp, int gp, const uint32_t *marks, const int4 *tab,
+__device__ __forceinline__ void own_windows(const SumParams &sp, int gp, const int32_t *kept, const int4 *tab,
                                          const int32_t *exps, const int4 *inv4, const int32_t *inve, int lg, int q, int hb,
                                          int sub, int subs, double *Jp, int P) {
   constexpr int W = Fmt<L>::W;
@@ -490,7 +491,7 @@ __device__ __forceinline__ void own_windows(const SumParams &sp, int gp, const u
   const int t0 = sp.poly_ptr[gp], blocks = (sp.poly_ptr[gp + 1] - t0 + kSumBlock - 1) / kSumBlock;
   for (int i = sub; i < sy.act_n; i += subs) {
     const int row = ((2 * i) << lg) + q;
-    if (marks[row] | marks[row + (1 << lg)]) continue;
+    if (kept[row]) continue;
     int E = fx::kZeroExp;
     uint32_t zr[W], zi[W];
 #pragma unroll
@@ -565,7 +566,7 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2
     const size_t tab_bytes = sum_tab_bytes(L, n, levels, lg);
     const size_t exp_off = static_cast<size_t>(levels) * n * kParts<L> * 16 << lg;
     // shared memory: values first (their place does not depend on the system),
-    // sums, marks, table
+    // sums, their leading bits, table
     const int vrows = 2 * NT * sp.values;
     int4 *vq = reinterpret_cast<int4 *>(smem);
     int32_t *vr = reinterpret_cast<int32_t *>(vq + Win<L>::Q * vrows);
@@ -574,7 +575,7 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2
     int4 *aq = reinterpret_cast<int4 *>(at);
     int32_t *ar = reinterpret_cast<int32_t *>(aq + Win<L>::Q * arows);
     if (!kOne) at += static_cast<size_t>(arows) * W * 4;
-    uint32_t *am = reinterpret_cast<uint32_t *>(at);
+    int32_t *am = reinterpret_cast<int32_t *>(at);
     unsigned char *stab = at + static_cast<size_t>(arows) * 4;
     const int64_t tile_id = (static_cast<int64_t>(s) << 32) | tile;
     if (kTabShared && held != tile_id) {
@@ -631,16 +632,20 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2
         }
         if (valid && u - fb < 2) store_sum<L>(fp + (u & 1) * KC, a, e0);
       };
-      // An entry of J: the sum times 1 / x_v.  The other component's sum is in
-      // lane ^ TP; each lane forms its own component of the product.
-      auto finish_J = [&](int u, uint32_t (&a)[W], uint32_t m) {
+      // An entry of J: the sum times 1 / x_v, where the window kept enough of
+      // its terms (`seen`: the or of their bits from kKeep up with one chunk,
+      // which leaves the window as it is; else their leading bit).  The other
+      // component's sum is in lane ^ TP; each lane forms its own component of
+      // the product.
+      auto finish_J = [&](int u, uint32_t (&a)[W], int32_t seen) {
         const int c = u & 1;
         const unsigned pair = (1u << lane) | (1u << (lane ^ TP));
         const int v = __ldg(sp.act + sy.act_off + (u >> 1));
         const Num<L> inv = load_factor<L>(inv4, inve, v, lg, q);
-        m |= __shfl_xor_sync(pair, m, TP);
-        am[(u << lg) + q] = m;
-        again = again || (m == 0u && valid);
+        const int32_t other_seen = __shfl_xor_sync(pair, seen, TP);
+        const bool kept = kOne ? (seen | other_seen) != 0 : max(seen, other_seen) >= Fmt<L>::kKeep;
+        am[(u << lg) + q] = kept;
+        again = again || (!kept && valid);
         int lead = lead_words<W>(a);
         lead = max(lead, __shfl_xor_sync(pair, lead, TP));
         int32_t own[L], other[L], r[L];
@@ -660,7 +665,7 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2
           }
         }
         fx::fold<L>(col, r);
-        if (valid && m != 0u)
+        if (valid && kept)
           store_product<L>(Jp + static_cast<size_t>(v) * P * 2 * KC + c * KC, r, ey + inv.e + B * L - 1);
       };
       int Eprev = 0;
@@ -671,7 +676,7 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2
           for (int i = 0; i < W; i++) z[i] = 0u;
           const int row = (u << lg) + q;
           store_window<L>(aq, ar, arows, row, z);
-          am[row] = 0u;
+          am[row] = -1;
         }
       }
       for (int tb = t0; kOne ? tb == t0 : tb < t1; tb += chunk) {
@@ -722,16 +727,17 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2
           if (u >= tasks && u < fb) continue;
           const int row = (u << lg) + q, c = u & 1;
           uint32_t a[W];
-          uint32_t m = 0u;
+          uint32_t m = 0u, low = 0u;  // the or of the terms' words above kw, of their words kw
+          int32_t top = -1;           // a bit that the terms of earlier chunks reach
           if constexpr (kOne) {
 #pragma unroll
             for (int i = 0; i < W; i++) a[i] = 0u;
           } else {
             load_window<L>(aq, ar, arows, row, a);
-            m = am[row];
+            top = am[row];
             if (grown > 0) {
               sar_words<W>(a, grown);
-              m >>= min(grown, 31);
+              top = max(top - grown, -1);
             }
           }
           if (u >= fb) {
@@ -779,7 +785,10 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2
                 mk |= z[x][kw] ^ sg;
               }
             }
-            m |= mk >> kb;
+            if constexpr (kOne)
+              m |= mk >> kb;
+            else
+              low |= mk;
           }
           uint32_t up[W];
           up[0] = 0u;
@@ -787,10 +796,12 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2
           for (int i = 0; i < W - 1; i++) up[i + 1] = odd[i];
           add_words<W>(a, up);
           if constexpr (kOne) {
-            finish_J(u, a, m);
+            finish_J(u, a, static_cast<int32_t>(m));
           } else {
             store_window<L>(aq, ar, arows, row, a);
-            am[row] = m;
+            // (exact but for bits above word kw + 1, which count as of that word)
+            if (m | low) top = max(top, (m ? 32 * kw + 63 : 32 * kw + 31) - __clz(static_cast<int>(m ? m : low)));
+            am[row] = top;
           }
         }
         eb ^= 1;
