@@ -41,8 +41,9 @@ namespace pe {
 namespace fx {
 
 // Per digit count: radix, words of the accumulation window (kernels_sum.cu),
-// and the least bit of the window that a derivative's largest term may have
-// as its leading one.
+// and the least bit of the window that the largest term of a derivative may
+// have as its leading one (a derivative of one term; sum_slack in internal.h
+// raises it for more).
 template <int L>
 struct Fmt;
 template <>

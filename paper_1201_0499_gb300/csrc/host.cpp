@@ -135,6 +135,7 @@ struct polyeval {
     size_t smem = 0;
   };
   SumLaunch sum_launch[3];
+  int sum_slack = 0;          // most of any derivative
   double sum_products = 0.0;  // products per point of the system (single)
   int sum_lg = 0;  // points per tile (log2) of batches and of calls with many points
   std::vector<pe::SumSys> sum_sys;
@@ -680,6 +681,8 @@ int setup_sum(polyeval *h, const Compiled &c) {
   // lists are then about equally long)
   std::vector<pe::SumPoly> sp(polys);
   std::vector<int32_t> act, count, slot;
+  std::vector<uint32_t> act_words;  // the same with the sums' slack
+  std::vector<int64_t> exp_sum, exp_min;
   std::vector<uint32_t> bits;
   int64_t pointers = 0;
   h->sum_sys.assign(S, pe::SumSys{});
@@ -692,7 +695,14 @@ int setup_sum(polyeval *h, const Compiled &c) {
     sp[gp].hit_off = pointers;
     bits.resize(bits.size() + static_cast<size_t>((d.n + 31) / 32), 0u);
     count.assign(d.n, 0);
-    for (int32_t j = c.mono_ptr[t0]; j < c.mono_ptr[t1]; j++) count[c.var[j] & 0xffffu]++;
+    exp_sum.assign(d.n, 0);
+    exp_min.assign(d.n, PE_MAX_EXP);
+    for (int32_t j = c.mono_ptr[t0]; j < c.mono_ptr[t1]; j++) {
+      const uint32_t v = c.var[j] & 0xffffu;
+      count[v]++;
+      exp_sum[v] += c.var[j] >> 16;
+      exp_min[v] = std::min<int64_t>(exp_min[v], c.var[j] >> 16);
+    }
     for (int v = 0; v < d.n; v++)
       if (count[v]) {
         act.push_back(v);
@@ -700,6 +710,11 @@ int setup_sum(polyeval *h, const Compiled &c) {
       }
     sp[gp].act_n = static_cast<int32_t>(act.size()) - sp[gp].act_off;
     std::stable_sort(act.begin() + sp[gp].act_off, act.end(), [&](int32_t a, int32_t b) { return count[a] > count[b]; });
+    for (size_t i = sp[gp].act_off; i < act.size(); i++) {
+      const int slack = pe::sum_slack(exp_sum[act[i]], exp_min[act[i]]);
+      act_words.push_back(static_cast<uint32_t>(act[i]) | static_cast<uint32_t>(slack) << 16);
+      h->sum_slack = std::max(h->sum_slack, slack);
+    }
     ss.act_max = std::max(ss.act_max, std::max(sp[gp].act_n, 1));
     pointers += static_cast<int64_t>((t1 - t0 + pe::kSumBlock - 1) / pe::kSumBlock) * (sp[gp].act_n + 1);
     if (pointers > kSumPointersMax || act.size() > INT32_MAX / 2 || bits.size() > INT32_MAX / 2) return PE_OK;
@@ -755,7 +770,7 @@ int setup_sum(polyeval *h, const Compiled &c) {
       // has more than one chunk and as many blocks stay resident
       for (int values = 1; values <= ((sl.threads >> lg) < m_max ? 2 : 1); values++) {
         size_t most = 0;
-        const bool one = (sl.threads >> lg) * values >= m_max;  // one chunk: no sums in shared memory
+        const bool one = (sl.threads >> lg) * values >= m_max && h->sum_slack <= pe::sum_one_slack(L);  // no sums in shared memory
         for (int s = 0; s < S; s++)
           most = std::max(most, pe::sum_smem_bytes(L, h->sys[s].n, h->sum_sys[s].act_max, h->sys[s].emax, lg, sl.threads,
                                                    values, one, shared != 0));
@@ -907,7 +922,7 @@ int setup_sum(polyeval *h, const Compiled &c) {
   // kernels
   DeviceBuf ord, co, fp;
   int rc;
-  if ((rc = fp.upload(fac_ptr)) || (rc = h->sum_fac.upload(fac)) || (rc = h->sum_polys.upload(sp)) || (rc = h->sum_act.upload(act)) || (rc = h->sum_bits.upload(bits)) ||
+  if ((rc = fp.upload(fac_ptr)) || (rc = h->sum_fac.upload(fac)) || (rc = h->sum_polys.upload(sp)) || (rc = h->sum_act.upload(act_words)) || (rc = h->sum_bits.upload(bits)) ||
       (rc = h->sum_hit_ptr.upload(hit_ptr)) || (rc = h->sum_hits.upload(hits)) || (rc = h->sum_sysd.upload(h->sum_sys)) ||
       (rc = h->sum_prefix.upload(prefix)) || (rc = h->sum_items.upload(words)) || (rc = ord.upload(order)) ||
       (rc = co.upload(c.coef)) ||
@@ -958,7 +973,7 @@ int run_sum(polyeval *h, const void *points, int64_t P, void *out_f, void *out_J
   sp.fac = static_cast<const uint32_t *>(h->sum_fac.p);
   sp.coef = static_cast<const int32_t *>(h->sum_coef.p);
   sp.polys = static_cast<const pe::SumPoly *>(h->sum_polys.p);
-  sp.act = static_cast<const int32_t *>(h->sum_act.p);
+  sp.act = static_cast<const uint32_t *>(h->sum_act.p);
   sp.act_bits = static_cast<const uint32_t *>(h->sum_bits.p);
   sp.hit_ptr = static_cast<const int32_t *>(h->sum_hit_ptr.p);
   sp.hits = static_cast<const uint2 *>(h->sum_hits.p);
@@ -1006,6 +1021,7 @@ int run_sum(polyeval *h, const void *points, int64_t P, void *out_f, void *out_J
   }
   const polyeval::SumLaunch &sl = h->sum_launch[lg];
   sp.values = sl.values;
+  sp.slack = h->sum_slack;
   sp.lg = lg;
   const size_t flagged = P >= 0 ? static_cast<size_t>(P) : static_cast<size_t>(h->sum_points);
   if (cudaMemsetAsync(h->sum_ctl.p, 0, kCtlFlags + flagged, s) != cudaSuccess) return PE_ECUDA;

@@ -163,7 +163,7 @@ struct SumParams {
   const uint32_t *fac;      // table entries (a - 1) n + v of each monomial
   const int32_t *coef;      // [M][kSumCoefWords] records: digits, exponent, first of fac, count, first factor
   const SumPoly *polys;     // [Ntot]
-  const int32_t *act;
+  const uint32_t *act;      // variable | slack << 16 (slack: see sum_slack)
   const uint32_t *act_bits;
   const int32_t *hit_ptr;
   const uint2 *hits;        // four 16-bit entries each: monomial of the block | exponent << 6 (0: no more)
@@ -181,6 +181,7 @@ struct SumParams {
   int32_t single_P;         // >= 0: single-system handle
   int32_t lg;               // log2 of the points per tile
   int32_t values;           // monomials per thread and chunk (1 or 2)
+  int32_t slack;            // most of any derivative (kernels of one chunk: at most sum_one_slack)
   SysDesc sys0;             // single: sys[0], sum_sys[0]
   SumSys sum_sys0;
   int32_t groups, group_polys;  // single: runs of polynomials per tile, polynomials per run
@@ -189,6 +190,16 @@ struct SumParams {
   int32_t *any;             // ... whether any point is flagged, zeroed before each call with ...
   unsigned char *flags;     // ... the flags of the points
 };
+
+// Every value is cut off below bit 0 of the window, so a derivative's sum is
+// less than sum a_t units off: `slack` = log2(sum a_t / min a_t), rounded up,
+// is how far above kKeep its largest term must lead for the sum to be as
+// accurate as a single term that leads there.
+inline int sum_slack(int64_t sum_a, int64_t min_a) {
+  int s = 0;
+  while (min_a << s < sum_a) s++;
+  return s;
+}
 
 template <int L>
 constexpr int kSumCoefWords = L == 8 ? 20 : 12;
@@ -209,6 +220,7 @@ __host__ __device__ constexpr size_t sum_blob_bytes(int L, int n, int levels, in
 size_t sum_smem_bytes(int L, int n, int act_max, int levels, int lg, int threads, int values, bool one,
                       bool tab_shared);
 int sum_head_bits_min(int L);
+int sum_one_slack(int L);  // most slack for which the words above kKeep's tell enough in a kernel of one chunk
 cudaError_t prepare_sum(int L, bool batch, size_t smem);
 cudaError_t sum_occupancy(int L, bool batch, bool one, bool tab_shared, int threads, size_t smem, int *blocks);
 cudaError_t launch_sum_powers(int L, const SumParams &p, cudaStream_t s);

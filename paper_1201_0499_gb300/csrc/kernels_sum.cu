@@ -515,7 +515,7 @@ __device__ __forceinline__ void own_windows(const SumParams &sp, int gp, const i
         for (unsigned a = h / kSumBlock; a > 0; a--) add_words<W>(zi, z);
       }
     }
-    const int v = sp.act[sy.act_off + i];
+    const int v = static_cast<int>(sp.act[sy.act_off + i] & 0xffffu);
     finish_entry<L>(zr, zi, E - (32 * W - 1 - hb), load_factor<L>(inv4, inve, v, lg, q),
                     Jp + static_cast<size_t>(v) * P * 2 * kComp<L>);
   }
@@ -633,17 +633,20 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2
         if (valid && u - fb < 2) store_sum<L>(fp + (u & 1) * KC, a, e0);
       };
       // An entry of J: the sum times 1 / x_v, where the window kept enough of
-      // its terms (`seen`: the or of their bits from kKeep up with one chunk,
-      // which leaves the window as it is; else their leading bit).  The other
+      // its terms (`seen`: the or of their bits from kKeep + sp.slack up with
+      // one chunk, which leaves the window as it is; else their leading bit).
+      // (The slack of every entry by itself, in a register through the loop
+      // below, cost n = 32 in double-double 2 % with one chunk.)  The other
       // component's sum is in lane ^ TP; each lane forms its own component of
       // the product.
       auto finish_J = [&](int u, uint32_t (&a)[W], int32_t seen) {
         const int c = u & 1;
         const unsigned pair = (1u << lane) | (1u << (lane ^ TP));
-        const int v = __ldg(sp.act + sy.act_off + (u >> 1));
+        const uint32_t entry = __ldg(sp.act + sy.act_off + (u >> 1));
+        const int v = static_cast<int>(entry & 0xffffu);
         const Num<L> inv = load_factor<L>(inv4, inve, v, lg, q);
         const int32_t other_seen = __shfl_xor_sync(pair, seen, TP);
-        const bool kept = kOne ? (seen | other_seen) != 0 : max(seen, other_seen) >= Fmt<L>::kKeep;
+        const bool kept = kOne ? (seen | other_seen) != 0 : max(seen, other_seen) >= Fmt<L>::kKeep + static_cast<int>(entry >> 16);
         am[(u << lg) + q] = kept;
         again = again || (!kept && valid);
         int lead = lead_words<W>(a);
@@ -786,7 +789,7 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2
               }
             }
             if constexpr (kOne)
-              m |= mk >> kb;
+              m |= __funnelshift_rc(mk, 0u, kb + sp.slack);
             else
               low |= mk;
           }
@@ -858,6 +861,10 @@ size_t sum_smem_bytes(int L, int n, int act_max, int levels, int lg, int threads
   return static_cast<size_t>(2) * threads * values * W * 4 +
          (static_cast<size_t>(sum_rows(act_max)) << lg) * (one ? 4 : W * 4 + 4) +
          (tab_shared ? sum_tab_bytes(L, n, levels, lg) : 0);
+}
+
+int sum_one_slack(int L) {
+  return 32 - (L == 3 ? Fmt<3>::kKeep : L == 4 ? Fmt<4>::kKeep : Fmt<8>::kKeep) % 32;
 }
 
 int sum_head_bits_min(int L) { return L == 3 ? Fmt<3>::kHeadMin : L == 4 ? Fmt<4>::kHeadMin : Fmt<8>::kHeadMin; }

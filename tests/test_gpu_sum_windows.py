@@ -47,3 +47,27 @@ def test_sums_outgrown_by_a_later_chunk(prec, growth, small, P):
     f, J = evaluate(s_in, p_in, prec)
     ef, ej = errors(s_ref, p_ref, f, J, prec, [0, P - 1])
     assert ef <= tol(prec) and ej <= tol(prec), (ef, ej)
+
+
+# Relative to its terms a derivative may lose: 2^-111 double-double, 2^-71
+# double, 2^-223 quad-double by the window; its products 2^-109, 2^-77, 2^-219
+# (x^256: 255 units of 2^-117, 2^-85, 2^-227); its rounding 2^-106, 2^-53, 2^-211.
+CLOSE = {"dd": 2.0**-104, "ddint": 2.0**-104, "f64": 2.0**-52, "qd": 2.0**-210}
+
+
+@pytest.mark.parametrize("prec", PRECS)
+@pytest.mark.parametrize("below", [30, 50, 55, 58, 59, 60, 61, 62, 63, 64, 65, 66, 67, 70, 90])
+@pytest.mark.parametrize("m", [100, 300, 2000])
+def test_many_tiny_terms_beside_a_small_one(prec, below, m):
+    """d f / d x_0 has one term 2^-below and m of 2^-130, which only the floors
+    of the window show, 256 units each; x_1 alone is of size 1.  m = 100: one
+    chunk; 300: one chunk but for a slack of 17 bits; 2000: several."""
+    n, P = 2, 2
+    rng = np.random.Generator(np.random.PCG64(970))
+    polys = [[([1], [1]), ([0], [1])] + [([0], [256])] * m]
+    s = synth.from_monomials(n, polys, scaled(rng, [0, below] + [130] * m))
+    pts = synth.points(971, n, P)
+    s_in, p_in, s_ref, p_ref = inputs(s, pts, prec, 972)
+    f, J = evaluate(s_in, p_in, prec)
+    ef, ej = errors(s_ref, p_ref, f, J, prec, range(P))
+    assert ef <= CLOSE[prec] and ej <= CLOSE[prec], (ef, ej)
