@@ -423,12 +423,16 @@ __global__ void __launch_bounds__(256, 2) newton_int(const NewtonParams p) {
 }  // namespace
 
 // The integer elimination takes a block per point; its shared memory bounds n.
-bool newton_int_fits(int n) { return n >= kIntLuMin && int_lu_bytes(n) <= 220 * 1024; }
+constexpr size_t kIntLuBytesMax = 220 * 1024;
+bool newton_int_fits(int n) { return n >= kIntLuMin && int_lu_bytes(n) <= kIntLuBytesMax; }
 
 cudaError_t launch_newton_int(const NewtonParams &p, cudaStream_t s) {
   const size_t bytes = int_lu_bytes(p.n);
   if (bytes > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(newton_int, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+    // the same limit on every call: it belongs to the kernel, not to this call,
+    // and another thread may be about to launch a larger system
+    const cudaError_t e =
+        cudaFuncSetAttribute(newton_int, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kIntLuBytesMax));
     if (e != cudaSuccess) return e;
   }
   // threads as the trailing updates need; the last warp does the reciprocals
