@@ -112,6 +112,15 @@ extern "C" {
  * else PE_EINVAL.  The term array takes (n^2 + n) m complex double-doubles
  * per point of max_points. */
 #define PE_PAPER_KERNELS 2u
+/* Evaluate every call with the general kernels alone.  PE_DD and PE_F64 then
+ * hold each component of an output to the accuracy that its own terms allow
+ * (see "Accuracy" above), and polyeval_autotune and polyeval_set_launch choose
+ * what polyeval_eval and polyeval_eval_many run. */
+#define PE_GENERAL_KERNELS 4u
+/* Evaluate from the monomials' values wherever those kernels can take the
+ * system, also where the library expects the general ones to be faster.
+ * PE_GENERAL_KERNELS goes before it. */
+#define PE_FROM_VALUES 8u
 
 /* ---- limits ------------------------------------------------------------ */
 #define PE_MAX_VARS 65535 /* n_vars                                        */
@@ -178,7 +187,8 @@ PE_API int polyeval_validate(const pe_system *sys, uint32_t flags);
  * Compile one system for evaluation (Section 2 format -> device metadata).
  *   sys         host system, copied; the caller may free it on return
  *   precision   PE_DD, PE_F64, PE_DD_INT or PE_QD_INT
- *   flags       PE_ALLOW_ZERO_COEF or 0
+ *   flags       0 or an or of PE_ALLOW_ZERO_COEF, PE_PAPER_KERNELS,
+ *               PE_GENERAL_KERNELS, PE_FROM_VALUES
  *   max_points  largest P any later polyeval_eval call will pass (>= 1);
  *               sizes the table of powers (Section 3.1) kept on the device
  *   out         receives the handle; *out is NULL on failure
@@ -214,9 +224,9 @@ PE_API int polyeval_eval(polyeval_t *h, const void *points, int64_t P, void *out
 
 /*
  * Choose the launch of polyeval_eval's general kernels for P points by timing
- * the candidates on the caller's data (where the evaluation from values runs,
- * the choice serves the points it leaves to them): the number of chunks the monomials of each polynomial
- * are split into (1, 2, 4, 8, as the handle's scratch allows), the launch
+ * the candidates, with those kernels alone, on the caller's data (where the
+ * evaluation from values runs, the choice serves the points it leaves to
+ * them): the number of chunks the monomials of each polynomial are split into (1, 2, 4, 8, as the handle's scratch allows), the launch
  * shape (1: one single-warp block per work item, all resident at once; 2: a
  * persistent grid taking items from the work counter) and, for PE_DD and
  * PE_F64 calls with fewer than 64 points, the threads per monomial: groups
@@ -245,8 +255,9 @@ PE_API int polyeval_autotune(polyeval_t *h, const void *points, int64_t P, void 
                              int *chunks, int *shape, int *groups);
 
 /*
- * Set the launch polyeval_eval uses for calls with exactly P points (what
- * polyeval_autotune would store): chunks 1..8 monomial chunks per polynomial
+ * Set the launch of polyeval_eval's general kernels for calls with exactly P
+ * points (what polyeval_autotune would store; where the evaluation from values
+ * runs, it governs the pass over the points left to them): chunks 1..8 monomial chunks per polynomial
  * (capped by the handle's scratch at run time), shape 1 (one single-warp
  * block per work item) or 2 (persistent grid), and groups 1, 2, 4, 8 or 16
  * monomial groups per warp (PE_DD and PE_F64; ignored by the integer-pipe
@@ -255,7 +266,9 @@ PE_API int polyeval_autotune(polyeval_t *h, const void *points, int64_t P, void 
  * Batch handles: P = 0; chunks and shape as above for polyeval_eval_many,
  * groups the most monomial groups of a partial last tile (0 or 16: as many as
  * fill the warp, the built-in choice); the call waits for all work on the
- * device when it rewrites the item table.  Errors: PE_EINVAL; PE_ECUDA.
+ * device when it rewrites the item table.  Batch handles that evaluate from
+ * values take one chunk and a persistent grid for the points left over,
+ * whatever chunks and shape say.  Errors: PE_EINVAL; PE_ECUDA.
  */
 PE_API int polyeval_set_launch(polyeval_t *h, int64_t P, int chunks, int shape, int groups);
 

@@ -32,6 +32,8 @@ PE_QD_INT = 3
 
 PE_ALLOW_ZERO_COEF = 1
 PE_PAPER_KERNELS = 2
+PE_GENERAL_KERNELS = 4
+PE_FROM_VALUES = 8
 
 PE_MAX_VARS = 65535
 PE_MAX_EXP = 256
@@ -229,8 +231,10 @@ def polyeval_eval(h: int, points, P: int, out_f, out_J, stream=None) -> None:
 
 
 def polyeval_autotune(h: int, points, P: int, out_f, out_J, stream=None):
-    """Time the launch candidates for P points and keep the fastest in the
-    handle; returns (chunks, shape, groups)."""
+    """Time the launch candidates of the general kernels for P points and keep
+    the fastest in the handle; returns (chunks, shape, groups).  On a
+    handle that evaluates from the monomials' values the choice serves the
+    points left to them; PE_GENERAL_KERNELS makes one that does not."""
     c, m, g = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
     _check(load_library().polyeval_autotune(h, _addr(points), int(P), _addr(out_f), _addr(out_J), _stream(stream),
                                             ctypes.byref(c), ctypes.byref(m), ctypes.byref(g)), "polyeval_autotune")
@@ -238,7 +242,7 @@ def polyeval_autotune(h: int, points, P: int, out_f, out_J, stream=None):
 
 
 def polyeval_set_launch(h: int, P: int, chunks: int = 0, shape: int = 0, groups: int = 0) -> None:
-    """Fix the launch for calls with P points (0 = built-in choice)."""
+    """Fix the launch of the general kernels for calls with P points (0 = built-in choice)."""
     _check(load_library().polyeval_set_launch(h, int(P), int(chunks), int(shape), int(groups)), "polyeval_set_launch")
 
 
@@ -383,7 +387,7 @@ class PolyEval:
         return out_f, out_J
 
     def autotune(self, points, out_f=None, out_J=None, stream=None):
-        """Tune the launch for this point count; returns (chunks, shape, groups)."""
+        """Tune the general kernels' launch for this point count; returns (chunks, shape, groups)."""
         import torch
 
         c = _elem(self.precision)
@@ -495,7 +499,7 @@ class PolyEvalMany:
         return self.views(f_buf, J_buf)
 
     def autotune(self, pts_buf, f_buf, J_buf, stream=None):
-        """Tune the batch launch on the packed buffers; returns (chunks, shape, groups)."""
+        """Tune the general kernels' batch launch on the packed buffers; returns (chunks, shape, groups)."""
         return polyeval_autotune(self.handle, pts_buf, 0, f_buf, J_buf, stream)
 
     def set_launch(self, chunks: int = 0, shape: int = 0, groups: int = 0):

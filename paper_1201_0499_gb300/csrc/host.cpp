@@ -666,7 +666,8 @@ bool sum_pays(const polyeval *h, const Compiled &c, const std::vector<pe::SumPol
 // Lists, digits and buffers for a compiled system set, after everything the
 // general kernels need.  PE_OK with h->sum_L = 0 when the set does not suit
 // the kernels or the device has no room: those then evaluate every call.
-int setup_sum(polyeval *h, const Compiled &c) {
+// `always`: whatever the cost rule says.
+int setup_sum(polyeval *h, const Compiled &c, bool always) {
   int dev = 0, optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
@@ -719,7 +720,7 @@ int setup_sum(polyeval *h, const Compiled &c) {
     pointers += static_cast<int64_t>((t1 - t0 + pe::kSumBlock - 1) / pe::kSumBlock) * (sp[gp].act_n + 1);
     if (pointers > kSumPointersMax || act.size() > INT32_MAX / 2 || bits.size() > INT32_MAX / 2) return PE_OK;
   }
-  if (!sum_pays(h, c, sp)) return PE_OK;
+  if (!always && !sum_pays(h, c, sp)) return PE_OK;
   // per system: magnitude range, headroom
   int m_max = 1, act_most = 1;
   for (int s = 0; s < S; s++) {
@@ -947,9 +948,10 @@ int setup_sum(polyeval *h, const Compiled &c) {
 }
 
 // Without host memory for the lists the handle does without them.
-int try_setup_sum(polyeval *h, const Compiled &c) {
+int try_setup_sum(polyeval *h, const Compiled &c, uint32_t flags) {
+  if (flags & PE_GENERAL_KERNELS) return PE_OK;
   try {
-    return setup_sum(h, c);
+    return setup_sum(h, c, (flags & PE_FROM_VALUES) != 0);
   } catch (const std::bad_alloc &) {
     h->sum_L = 0;
     return PE_OK;
@@ -1133,7 +1135,7 @@ int polyeval_create(const pe_system *sys, int precision, uint32_t flags, int64_t
         return rc;
       }
     }
-    if ((rc = try_setup_sum(h, c)) != PE_OK) {
+    if ((rc = try_setup_sum(h, c, flags)) != PE_OK) {
       delete h;
       return rc;
     }
@@ -1233,7 +1235,7 @@ int polyeval_create_many(const pe_system *systems, int32_t count, int precision,
         return rc;
       }
     }
-    if ((rc = try_setup_sum(h, c)) != PE_OK) {
+    if ((rc = try_setup_sum(h, c, flags)) != PE_OK) {
       delete h;
       return rc;
     }
