@@ -140,7 +140,8 @@ struct polyeval {
   int sum_lg = 0;  // points per tile (log2) of batches and of calls with many points
   std::vector<pe::SumSys> sum_sys;
   int64_t sum_power_total = 0, sum_items_n = 0;  // batch
-  DeviceBuf sum_fac, sum_coef, sum_polys, sum_act, sum_bits, sum_hit_ptr, sum_hits, sum_sysd, sum_prefix, sum_items;
+  DeviceBuf sum_fac, sum_coef, sum_polys, sum_act, sum_bits, sum_hit_ptr, sum_hits, sum_sysd, sum_prefix, sum_items,
+      sum_const_var, sum_const_val;
   DeviceBuf sum_table, sum_ctl;  // sum_ctl: two work counters, whether any point is flagged, the points' flags
   int64_t sum_points = 0;        // flags
   // timing of the main kernel
@@ -684,6 +685,8 @@ int setup_sum(polyeval *h, const Compiled &c, bool always) {
   std::vector<int32_t> act, count, slot;
   std::vector<uint32_t> act_words;  // the same with the sums' slack
   std::vector<int64_t> exp_sum, exp_min;
+  std::vector<int32_t> const_var;   // entries of J that are one coefficient
+  std::vector<double> const_val;
   std::vector<uint32_t> bits;
   int64_t pointers = 0;
   h->sum_sys.assign(S, pe::SumSys{});
@@ -704,6 +707,18 @@ int setup_sum(polyeval *h, const Compiled &c, bool always) {
       exp_sum[v] += c.var[j] >> 16;
       exp_min[v] = std::min<int64_t>(exp_min[v], c.var[j] >> 16);
     }
+    sp[gp].const_off = static_cast<int32_t>(const_var.size());
+    if (!h->qd)  // (quad-double: the general kernels hold components no better than this path)
+      for (int32_t t = t0; t < t1; t++) {
+        if (c.mono_ptr[t + 1] - c.mono_ptr[t] != 1) continue;
+        const uint32_t v = c.var[c.mono_ptr[t]] & 0xffffu;
+        if (count[v] != 1 || c.var[c.mono_ptr[t]] >> 16 != 1) continue;
+        count[v] = 0;
+        const_var.push_back(static_cast<int32_t>(v));
+        const_val.insert(const_val.end(), c.coef.begin() + static_cast<size_t>(t) * cd, c.coef.begin() + static_cast<size_t>(t + 1) * cd);
+        bits[sp[gp].bits_off + (v >> 5)] |= 1u << (v & 31);
+      }
+    sp[gp].const_n = static_cast<int32_t>(const_var.size()) - sp[gp].const_off;
     for (int v = 0; v < d.n; v++)
       if (count[v]) {
         act.push_back(v);
@@ -844,7 +859,7 @@ int setup_sum(polyeval *h, const Compiled &c, bool always) {
   for (size_t gp = 0; gp < polys; gp++) {
     const int n = h->sys[c.poly_sys[gp]].n, na = sp[gp].act_n;
     const int32_t t0 = c.poly_ptr[gp], t1 = c.poly_ptr[gp + 1];
-    slot.resize(n);
+    slot.assign(n, -1);
     for (int i = 0; i < na; i++) slot[act[sp[gp].act_off + i]] = i;
     auto k_of = [&](int32_t t) { return c.mono_ptr[t + 1] - c.mono_ptr[t]; };
     std::iota(order.begin() + t0, order.begin() + t1, t0);
@@ -856,7 +871,7 @@ int setup_sum(polyeval *h, const Compiled &c, bool always) {
         for (int32_t j = c.mono_ptr[order[t]]; j < c.mono_ptr[order[t] + 1]; j++) {
           const uint32_t v = c.var[j] & 0xffffu, a = c.var[j] >> 16;
           fac[nf++] = (a - 1) * static_cast<uint32_t>(n) + v;
-          at[slot[v]]++;
+          if (slot[v] >= 0) at[slot[v]]++;
         }
         fac_ptr[t + 1] = nf;
       }
@@ -872,7 +887,8 @@ int setup_sum(polyeval *h, const Compiled &c, bool always) {
       hits.resize(nh, 0);
       for (int32_t t = b; t < e; t++)
         for (int32_t j = c.mono_ptr[order[t]]; j < c.mono_ptr[order[t] + 1]; j++)
-          hits[at[slot[c.var[j] & 0xffffu]]++] = static_cast<uint16_t>((t - b) | (c.var[j] >> 16) << 6);
+          if (const int32_t i = slot[c.var[j] & 0xffffu]; i >= 0)
+            hits[at[i]++] = static_cast<uint16_t>((t - b) | (c.var[j] >> 16) << 6);
       for (int i = 0; i < na; i++)  // filled up to a multiple of four: the last monomial, zero times
         for (size_t x = at[i]; x < 4 * static_cast<size_t>(hit_ptr[hp + i + 1]); x++)
           hits[x] = static_cast<uint16_t>(hits[x - 1] & (pe::kSumBlock - 1));
@@ -925,12 +941,13 @@ int setup_sum(polyeval *h, const Compiled &c, bool always) {
   int rc;
   if ((rc = fp.upload(fac_ptr)) || (rc = h->sum_fac.upload(fac)) || (rc = h->sum_polys.upload(sp)) || (rc = h->sum_act.upload(act_words)) || (rc = h->sum_bits.upload(bits)) ||
       (rc = h->sum_hit_ptr.upload(hit_ptr)) || (rc = h->sum_hits.upload(hits)) || (rc = h->sum_sysd.upload(h->sum_sys)) ||
-      (rc = h->sum_prefix.upload(prefix)) || (rc = h->sum_items.upload(words)) || (rc = ord.upload(order)) ||
+      (rc = h->sum_prefix.upload(prefix)) || (rc = h->sum_const_var.upload(const_var)) ||
+      (rc = h->sum_const_val.upload(const_val)) || (rc = h->sum_items.upload(words)) || (rc = ord.upload(order)) ||
       (rc = co.upload(c.coef)) ||
       (rc = h->sum_coef.alloc(static_cast<size_t>(M) * 4 * (L == 8 ? 20 : 12))) ||
       (rc = h->sum_table.alloc(tb)) || (rc = h->sum_ctl.alloc(kCtlFlags + static_cast<size_t>(fl)))) {
     for (DeviceBuf *b : {&h->sum_fac, &h->sum_polys, &h->sum_act, &h->sum_bits, &h->sum_hit_ptr, &h->sum_hits, &h->sum_sysd,
-                         &h->sum_prefix, &h->sum_items, &h->sum_coef, &h->sum_table, &h->sum_ctl})
+                         &h->sum_prefix, &h->sum_items, &h->sum_const_var, &h->sum_const_val, &h->sum_coef, &h->sum_table, &h->sum_ctl})
       b->alloc(0);
     return rc == PE_ENOMEM ? PE_OK : rc;
   }
@@ -977,6 +994,8 @@ int run_sum(polyeval *h, const void *points, int64_t P, void *out_f, void *out_J
   sp.polys = static_cast<const pe::SumPoly *>(h->sum_polys.p);
   sp.act = static_cast<const uint32_t *>(h->sum_act.p);
   sp.act_bits = static_cast<const uint32_t *>(h->sum_bits.p);
+  sp.const_var = static_cast<const int32_t *>(h->sum_const_var.p);
+  sp.const_val = static_cast<const double *>(h->sum_const_val.p);
   sp.hit_ptr = static_cast<const int32_t *>(h->sum_hit_ptr.p);
   sp.hits = static_cast<const uint2 *>(h->sum_hits.p);
   sp.sys = static_cast<const SysDesc *>(h->sysd.p);

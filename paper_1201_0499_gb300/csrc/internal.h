@@ -149,13 +149,15 @@ struct SumSys {
 };
 
 // One polynomial: its variables ("active"), and its lists, per block of
-// kSumBlock monomials one per active variable.
+// kSumBlock monomials one per active variable.  A variable that occurs in one
+// monomial only, c x, is not active: its derivative is c, with both components
+// as given (c x / x would hold the smaller to the larger one's precision).
 struct SumPoly {
   int64_t hit_off;   // first list pointer: per block act_n + 1 offsets into hits
   int32_t act_off;   // active variables, in act
   int32_t act_n;
-  int32_t bits_off;  // the same as a bit mask of n bits
-  int32_t pad;
+  int32_t bits_off;  // a bit mask of n bits: the active and the constant entries
+  int32_t const_off, const_n;  // constant entries of J, in const_var and const_val
 };
 
 struct SumParams {
@@ -165,6 +167,8 @@ struct SumParams {
   const SumPoly *polys;     // [Ntot]
   const uint32_t *act;      // variable | slack << 16 (slack: see sum_slack)
   const uint32_t *act_bits;
+  const int32_t *const_var;  // entries of J that are one coefficient: the variable ...
+  const double *const_val;   // ... and the value
   const int32_t *hit_ptr;
   const uint2 *hits;        // four 16-bit entries each: monomial of the block | exponent << 6 (0: no more)
   const SysDesc *sys;

@@ -605,13 +605,20 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2
       double *Jp = sp.out_J + (static_cast<size_t>(sd.J_off) + static_cast<size_t>(pl) * n * P + qg) * 2 * KC;
       double *fp = sp.out_f + (static_cast<size_t>(sd.f_off) + static_cast<size_t>(pl) * P + qg) * 2 * KC;
       // entries of variables that do not occur in the polynomial
-      if (sy.act_n < n && valid) {
+      if (sy.act_n + sy.const_n < n && valid) {
         for (int v = sub; v < n; v += subs) {
           if (__ldg(sp.act_bits + sy.bits_off + (v >> 5)) >> (v & 31) & 1u) continue;
           double *o = Jp + static_cast<size_t>(v) * P * 2 * KC;
           store_zero<L>(o);
           store_zero<L>(o + KC);
         }
+      }
+      // entries that are one coefficient
+      for (int i = sub; i < sy.const_n && valid; i += subs) {
+        const double *c = sp.const_val + static_cast<size_t>(sy.const_off + i) * 2 * KC;
+        double *o = Jp + static_cast<size_t>(sp.const_var[sy.const_off + i]) * P * 2 * KC;
+#pragma unroll
+        for (int k = 0; k < 2 * KC; k++) o[k] = c[k];
       }
       if (t0 == t1) {  // no monomials
         if (valid && sub < 2) store_zero<L>(fp + sub * KC);

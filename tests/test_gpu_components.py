@@ -1,0 +1,110 @@
+"""Each component of f and J by itself, where its terms are far below the other
+component's: a derivative that is one coefficient, points near the real axis.
+
+Measure: |error of a component| over the sum of its terms' parts, (|re|, |im|)
+pairs multiplied without cancellation ((a, b)(c, d) = (ac + bd, ad + bc)).
+Bound: that of the general kernels, which compute components apart: a product
+errs by 2^-102 (double-double) of its parts, a chain of 8 and a sum stay below
+2^-98; in double 2^-52 each, 2^-48."""
+import numpy as np
+import pytest
+
+import synth
+from fractions import Fraction
+from oracle import exact as E
+
+from test_gpu_methods import evaluate
+from test_gpu_sum import inputs, system
+
+pytestmark = pytest.mark.gpu
+
+BOUND = {"dd": 2.0**-98, "f64": 2.0**-48}
+
+
+def pair(v):
+    w = len(v) // 2
+    return abs(sum(v[:w])), abs(sum(v[w:]))
+
+
+def times(a, b):
+    return a[0] * b[0] + a[1] * b[1], a[0] * b[1] + a[1] * b[0]
+
+
+def part_scales(s, pts, q, p):
+    """The measure's denominators: f [2], J [n, 2] of polynomial p at point q."""
+    x = [pair(pts[v, q]) for v in range(s.n_vars)]
+    f, J = np.zeros(2), np.zeros((s.n_vars, 2))
+    for t in range(int(s.poly_ptr[p]), int(s.poly_ptr[p + 1])):
+        vs = s.pos[s.mono_ptr[t]:s.mono_ptr[t + 1]]
+        es = s.exp[s.mono_ptr[t]:s.mono_ptr[t + 1]]
+        less, full = [], []
+        for v, e in zip(vs, es):
+            y = (1.0, 0.0)
+            for _ in range(e - 1):
+                y = times(y, x[v])
+            less.append(y)
+            full.append(times(y, x[v]))
+        value = pair(s.coef[t])
+        for y in full:
+            value = times(value, y)
+        f += value
+        for j in range(len(vs)):
+            d = pair(s.coef[t])
+            for i in range(len(vs)):
+                d = times(d, less[i] if i == j else full[i])
+            J[vs[j]] += es[j] * np.array(d)
+    return f, J
+
+
+def component_error(got, exact, scale):
+    w = len(got) // 2
+    worst = 0.0
+    for c in range(2):
+        value = sum((Fraction(float(v)) for v in got[c * w:(c + 1) * w]), Fraction(0))
+        d = float(abs(value - Fraction(exact[c]) * Fraction(2) ** exact[2]))
+        worst = max(worst, d / scale[c] if scale[c] else (0.0 if d == 0.0 else np.inf))
+    return worst
+
+
+def worst_components(s, pts, f, J, points, polys):
+    worst = 0.0
+    for q in points:
+        fx, Jx = E.evaluate_point(s, pts, q, polys)
+        for p in polys:
+            sf, sJ = part_scales(s, pts, q, p)
+            worst = max(worst, component_error(f[p, q], fx[p], sf))
+            for i, v in Jx[p].items():
+                worst = max(worst, component_error(J[p, i, q], v, sJ[i]))
+    return worst
+
+
+@pytest.mark.parametrize("prec", ["dd", "ddint", "f64"])
+@pytest.mark.parametrize("apart", [12, 22, 34])
+def test_derivatives_that_are_one_coefficient(prec, apart):
+    """x_6 .. x_9 occur once per polynomial, as c x with components 2^-apart of
+    each other: their derivatives are c, bit for bit, at any point."""
+    import paper_1201_0499_gb300 as pkg
+
+    n, N, P = 10, 3, 9
+    base = system(1200, 6, N, 70, 2, 5, 3)
+    rng = np.random.Generator(np.random.PCG64(1201))
+    polys, coef, m = [], [], 0
+    for p in range(N):
+        mons = []
+        for t in range(int(base.poly_ptr[p]), int(base.poly_ptr[p + 1])):
+            mons.append((base.pos[base.mono_ptr[t]:base.mono_ptr[t + 1]].tolist(),
+                         base.exp[base.mono_ptr[t]:base.mono_ptr[t + 1]].tolist()))
+        coef += [c for c in base.coef[int(base.poly_ptr[p]):int(base.poly_ptr[p + 1])]]
+        own = synth.random_cdd(rng, 4)
+        own[:2, 2:] = np.ldexp(own[:2, 2:], -apart)
+        own[2:, :2] = np.ldexp(own[2:, :2], -apart)
+        polys.append(mons + [([6 + i], [1]) for i in range(4)])
+        coef += [c for c in own]
+    s = synth.from_monomials(n, polys, np.array(coef))
+    pts = synth.points(1202, n, P)
+    s_in, p_in, s_ref, p_ref = inputs(s, pts, prec, 1203)
+    f, J = evaluate(s_in, p_in, prec, pkg.PE_FROM_VALUES)
+    for p in range(N):
+        for i in range(4):
+            c = s_ref.coef[int(s.poly_ptr[p + 1]) - 4 + i]
+            assert np.all(J[p, 6 + i] == (c[[0, 2]] if prec == "f64" else c)), (p, i)
