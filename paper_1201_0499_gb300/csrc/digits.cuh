@@ -35,6 +35,7 @@
 
 #include <cstdint>
 
+#include "internal.h"
 #include "wide8.cuh"
 
 namespace pe {
@@ -258,6 +259,8 @@ __device__ __forceinline__ float scale_modulus(Num<L> &y, int t) {
 struct Seen {
   bool bad;      // not finite, zero, or its components too far apart
   float log2m;   // base-2 logarithm of the modulus
+  bool near_axis = false;  // components more than kSumNearAxis bits apart, or one zero
+  bool real = false;       // no imaginary component
 };
 
 // Components further apart than this many bits are left to the general
@@ -282,7 +285,10 @@ __device__ __forceinline__ Num<L> from_parts(const double *v, int t, Seen &seen)
       // exponents of the leading bits
       const int tr = r.e + r.lead, ti = i.e + i.lead;
       const int top = r.lead < 0 ? ti : i.lead < 0 ? tr : max(tr, ti);
-      seen.bad = r.lead >= 0 && i.lead >= 0 && (tr - ti > kMaxSkew || ti - tr > kMaxSkew);
+      const bool both = r.lead >= 0 && i.lead >= 0;
+      seen.bad = both && (tr - ti > kMaxSkew || ti - tr > kMaxSkew);
+      seen.near_axis = !both || tr - ti > kSumNearAxis || ti - tr > kSumNearAxis;
+      seen.real = i.lead < 0;
       // leading bit of the larger component to bit B - 2 of the top digit
       y.e = top - (B * L - 2);
       if (r.lead >= 0) r.shift(y.e - r.e);

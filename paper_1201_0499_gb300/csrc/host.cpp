@@ -135,6 +135,7 @@ struct polyeval {
     size_t smem = 0;
   };
   SumLaunch sum_launch[3];
+  bool sum_axial = false;     // any system with near-axis points to leave
   int sum_slack = 0;          // most of any derivative
   double sum_products = 0.0;  // products per point of the system (single)
   int sum_lg = 0;  // points per tile (log2) of batches and of calls with many points
@@ -142,7 +143,7 @@ struct polyeval {
   int64_t sum_power_total = 0, sum_items_n = 0;  // batch
   DeviceBuf sum_fac, sum_coef, sum_polys, sum_act, sum_bits, sum_hit_ptr, sum_hits, sum_sysd, sum_prefix, sum_items,
       sum_const_var, sum_const_val;
-  DeviceBuf sum_table, sum_ctl;  // sum_ctl: two work counters, whether any point is flagged, the points' flags
+  DeviceBuf sum_table, sum_ctl;  // sum_ctl: see kCtlCounts
   int64_t sum_points = 0;        // flags
   // timing of the main kernel
   bool timing = false;
@@ -624,8 +625,13 @@ int run_main(polyeval *h, const pe::MainParams &mp, cudaStream_t s, int mode = 0
 // ---------------------------------------------------------------------------
 
 // sum_ctl: work counter of the sum kernel, whether any point is flagged, the
-// general kernels' counter, one spare word, the flags.
-constexpr size_t kCtlFlags = 16;
+// general kernels' counter, one spare word, the points' counts of near-axis
+// coordinates (handles with an axial system), the points' flags.
+constexpr size_t kCtlCounts = 16;
+
+size_t ctl_flags(const polyeval *h, int64_t points) {
+  return kCtlCounts + (h->sum_axial ? 4 * static_cast<size_t>(points) : 0);
+}
 
 // Whether the evaluation from values is the faster one for these systems:
 // nanoseconds per polynomial and point of both, fitted to measurements from 1
@@ -662,6 +668,35 @@ bool sum_pays(const polyeval *h, const Compiled &c, const std::vector<pe::SumPol
     }
   }
   return 1.1 * values < general;
+}
+
+// Whether terms of a system may lie near an axis where all coordinates of a
+// point do (SumSys::axial; double-double): the parts of the coefficients of a
+// polynomial, or of one of its derivatives, summed up, more than 2^kSumNearAxis
+// apart.  kAxialReal: all coefficients are real.
+int32_t axial_system(const Compiled &c, const SysDesc &d) {
+  bool axial = false, real = true;
+  std::vector<double> re(d.n), im(d.n);
+  auto apart = [](double a, double b) { return std::max(a, b) > 0.0 && std::min(a, b) * (1 << pe::kSumNearAxis) < std::max(a, b); };
+  for (int32_t gp = d.poly0; gp < d.poly0 + d.N; gp++) {
+    std::fill(re.begin(), re.end(), 0.0);
+    std::fill(im.begin(), im.end(), 0.0);
+    double fr = 0.0, fi = 0.0;
+    for (int32_t t = c.poly_ptr[gp]; t < c.poly_ptr[gp + 1]; t++) {
+      const double *cf = &c.coef[static_cast<size_t>(t) * 4];
+      const double a = std::fabs(cf[0]), b = std::fabs(cf[2]);
+      real = real && b == 0.0;
+      fr += a;
+      fi += b;
+      for (int32_t j = c.mono_ptr[t]; j < c.mono_ptr[t + 1]; j++) {
+        re[c.var[j] & 0xffffu] += a * (c.var[j] >> 16);
+        im[c.var[j] & 0xffffu] += b * (c.var[j] >> 16);
+      }
+    }
+    axial = axial || apart(fr, fi);
+    for (int v = 0; v < d.n && !axial; v++) axial = apart(re[v], im[v]);
+  }
+  return !axial ? 0 : real ? pe::kAxialReal : pe::kAxial;
 }
 
 // Lists, digits and buffers for a compiled system set, after everything the
@@ -755,13 +790,17 @@ int setup_sum(polyeval *h, const Compiled &c, bool always) {
         int er = 0, ei = 0;
         std::frexp(re, &er);
         std::frexp(im, &ei);
-        // components so far apart that one common exponent would cost the
-        // smaller one its own relative precision
+        // One common exponent leaves the smaller component 118 (double 88,
+        // quad-double 230) bits less their distance, and J is rounded 8 bits
+        // higher: all it was given in double; in double-double that shows near
+        // the axes only (see axial).
         if (re != 0.0 && im != 0.0 && std::abs(er - ei) > kSumCoefSkew) return PE_OK;
         if (re != 0.0 || im != 0.0)
           gamma = std::max(gamma, std::fabs(static_cast<double>(re > im ? er : ei)) + 1.0);
       }
     }
+    ss.axial = L == 4 ? axial_system(c, d) : 0;
+    h->sum_axial = h->sum_axial || ss.axial != 0;
     // every monomial value within 2^(+-900) of 1: no overflow, and the low
     // parts of the results well above the smallest normal double
     if (gamma > 800.0) return PE_OK;
@@ -945,7 +984,7 @@ int setup_sum(polyeval *h, const Compiled &c, bool always) {
       (rc = h->sum_const_val.upload(const_val)) || (rc = h->sum_items.upload(words)) || (rc = ord.upload(order)) ||
       (rc = co.upload(c.coef)) ||
       (rc = h->sum_coef.alloc(static_cast<size_t>(M) * 4 * (L == 8 ? 20 : 12))) ||
-      (rc = h->sum_table.alloc(tb)) || (rc = h->sum_ctl.alloc(kCtlFlags + static_cast<size_t>(fl)))) {
+      (rc = h->sum_table.alloc(tb)) || (rc = h->sum_ctl.alloc(ctl_flags(h, fl) + static_cast<size_t>(fl)))) {
     for (DeviceBuf *b : {&h->sum_fac, &h->sum_polys, &h->sum_act, &h->sum_bits, &h->sum_hit_ptr, &h->sum_hits, &h->sum_sysd,
                          &h->sum_prefix, &h->sum_items, &h->sum_const_var, &h->sum_const_val, &h->sum_coef, &h->sum_table, &h->sum_ctl})
       b->alloc(0);
@@ -1013,7 +1052,6 @@ int run_sum(polyeval *h, const void *points, int64_t P, void *out_f, void *out_J
   unsigned char *ctl = static_cast<unsigned char *>(h->sum_ctl.p);
   sp.counter = reinterpret_cast<unsigned *>(ctl);
   sp.any = reinterpret_cast<int32_t *>(ctl + 4);
-  sp.flags = ctl + kCtlFlags;
   int lg = h->sum_lg;
   if (P >= 0) {
     const SysDesc &d = h->sys[0];
@@ -1044,8 +1082,10 @@ int run_sum(polyeval *h, const void *points, int64_t P, void *out_f, void *out_J
   sp.values = sl.values;
   sp.slack = h->sum_slack;
   sp.lg = lg;
-  const size_t flagged = P >= 0 ? static_cast<size_t>(P) : static_cast<size_t>(h->sum_points);
-  if (cudaMemsetAsync(h->sum_ctl.p, 0, kCtlFlags + flagged, s) != cudaSuccess) return PE_ECUDA;
+  const int64_t points_n = P >= 0 ? P : h->sum_points;
+  sp.near = reinterpret_cast<unsigned *>(ctl + kCtlCounts);
+  sp.flags = ctl + ctl_flags(h, points_n);
+  if (cudaMemsetAsync(h->sum_ctl.p, 0, ctl_flags(h, points_n) + static_cast<size_t>(points_n), s) != cudaSuccess) return PE_ECUDA;
   if (pe::launch_sum_powers(h->sum_L, sp, s) != cudaSuccess) return PE_ECUDA;
   if (e0 && cudaEventRecord(e0, s) != cudaSuccess) return PE_ECUDA;
   const int grid = static_cast<int>(std::min<int64_t>(sp.n_items, sl.blocks));
@@ -1056,7 +1096,7 @@ int run_sum(polyeval *h, const void *points, int64_t P, void *out_f, void *out_J
 
 const int32_t *sum_any(const polyeval *h) { return reinterpret_cast<const int32_t *>(static_cast<const unsigned char *>(h->sum_ctl.p) + 4); }
 unsigned *general_counter(const polyeval *h) { return reinterpret_cast<unsigned *>(static_cast<unsigned char *>(h->sum_ctl.p) + 8); }
-const unsigned char *sum_flags(const polyeval *h) { return static_cast<const unsigned char *>(h->sum_ctl.p) + kCtlFlags; }
+const unsigned char *sum_flags(const polyeval *h, int64_t points) { return static_cast<const unsigned char *>(h->sum_ctl.p) + ctl_flags(h, points); }
 
 }  // namespace
 
@@ -1362,7 +1402,7 @@ int eval_single(polyeval *h, const void *points, int64_t P, void *out_f, void *o
     pe::PowerParams pp{};
     if (by_values) {
       pp.any = sum_any(h);
-      pp.flags = sum_flags(h);
+      pp.flags = sum_flags(h, P);
     }
     pp.sys = static_cast<const SysDesc *>(h->sysd.p);
     pp.points = static_cast<const double *>(points);
@@ -1424,7 +1464,7 @@ int eval_single(polyeval *h, const void *points, int64_t P, void *out_f, void *o
   pe::Only only{nullptr, nullptr, static_cast<int32_t>(P)};
   if (by_values) {
     mp.any = only.any = sum_any(h);
-    mp.flags = only.flags = sum_flags(h);
+    mp.flags = only.flags = sum_flags(h, P);
     mp.regroup = regroup;
     mp.counter = general_counter(h);
   }
@@ -1464,7 +1504,7 @@ int eval_many(polyeval *h, const void *points, void *out_f, void *out_J, cudaStr
     pe::PowerParams pp{};
     if (by_values) {
       pp.any = sum_any(h);
-      pp.flags = sum_flags(h);
+      pp.flags = sum_flags(h, h->sum_points);
     }
     pp.sys = static_cast<const SysDesc *>(h->sysd.p);
     pp.prefix = static_cast<const int64_t *>(h->prefix.p);
@@ -1499,7 +1539,7 @@ int eval_many(polyeval *h, const void *points, void *out_f, void *out_J, cudaStr
   mp.finish = by_values && C == 1;
   if (by_values) {
     mp.any = sum_any(h);
-    mp.flags = sum_flags(h);
+    mp.flags = sum_flags(h, h->sum_points);
     mp.regroup = !block_format(h);
     mp.counter = general_counter(h);
   }

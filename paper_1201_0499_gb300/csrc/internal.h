@@ -137,6 +137,7 @@ struct PowerParams {
 constexpr int kSumThreadsMax = 256;
 constexpr int kSumPointsMax = 4;   // points per tile: 1, 2 or 4
 constexpr int kSumParts = 4;       // sums that f is split into
+constexpr int kSumNearAxis = 4;    // bits between the components of a number near an axis
 constexpr int kSumBlock = 64;      // monomials per block of the addition lists (their entries hold 6 bits of it)
 
 // One compiled system.
@@ -146,7 +147,9 @@ struct SumSys {
   float most_log2;    // points with a coordinate modulus outside 2^(+-most_log2) are flagged
   int32_t act_max;    // most variables of a polynomial
   int32_t head_bits;  // headroom of the window: log2 of a bound of sum_t a_t
+  int32_t axial;      // leave near-axis points to the general kernels (kAxial, kAxialReal: but real ones)
 };
+constexpr int32_t kAxial = 1, kAxialReal = 2;
 
 // One polynomial: its variables ("active"), and its lists, per block of
 // kSumBlock monomials one per active variable.  A variable that occurs in one
@@ -192,7 +195,8 @@ struct SumParams {
   int32_t n_polys_total;
   unsigned *counter;        // work counter and ...
   int32_t *any;             // ... whether any point is flagged, zeroed before each call with ...
-  unsigned char *flags;     // ... the flags of the points
+  unsigned char *flags;     // ... the flags of the points ...
+  unsigned *near;           // ... and counts of their near-axis coordinates (all, 2^16 those not real)
 };
 
 // Every value is cut off below bit 0 of the window, so a derivative's sum is

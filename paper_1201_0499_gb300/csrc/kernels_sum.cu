@@ -15,6 +15,22 @@
 // and the general kernels (kernels.cu, kernels_wide.cu, kernels_qd.cu)
 // evaluate them.
 //
+// Near-axis points (double-double).  A number's components share its exponent
+// here, so the smaller one errs like the larger.  That shows where a term's
+// smaller component comes from smaller components alone, (a + ib)(c + id) with
+// b << a, d << c: not with one factor off the axes, whose components then
+// reach both.  The general kernels compute components apart; so a point whose
+// every coordinate lies near an axis (components more than 2^kSumNearAxis apart)
+// is left to them, where the coefficients of a polynomial or of a derivative
+// lie near one too (`axial`, by the sums of their parts).  Real points of real
+// systems stay: their imaginary parts are exact zeros.  Double and quad-double
+// need no such rule: 88 bits hold 53 down to 2^-24, and the general
+// quad-double kernels share exponents in the same way.  (Worst error of a
+// component over its terms' parts, real coefficients, components of the points
+// 2^-8, 2^-16, 2^-22 apart: general 2^-103.5, 2^-103.3, 2^-103.6, from values
+// 2^-97, 2^-89, 2^-82.5; on the unit circle 2^-104.4 and 2^-105.9.  Points on
+// the circle: (2 2^-kSumNearAxis)^n of them lie near an axis in n coordinates.)
+//
 // Layout.  One block works on one tile of 1, 2, 4 or 8 points of a system and
 // a run of polynomials.  The tile's power table (digits.cuh) is copied to
 // shared memory once.  For each polynomial, chunks of monomials:
@@ -318,6 +334,16 @@ __global__ void __launch_bounds__(128) sum_powers(const SumParams sp) {
     fx::Seen seen;
     Num<L> y = read_number<L>(sp.points + (sd.pt_off + static_cast<int64_t>(v) * P + qc) * 2 * kComp<L>, Fmt<L>::B - 1, seen);
     const bool bad = seen.bad || fabsf(seen.log2m) > ss.most_log2;
+    if constexpr (L == 4) {
+      if (seen.near_axis && ss.axial && !inverse && qg < P) {
+        const unsigned one = seen.real ? 1u : 0x10001u;
+        const unsigned c = atomicAdd(sp.near + ss.flag_off + qg, one) + one;
+        if ((c & 0xffffu) == static_cast<unsigned>(n) && (ss.axial == kAxial || c >> 16)) {  // the last one sees it
+          sp.flags[ss.flag_off + qg] = 1;
+          *sp.any = 1;
+        }
+      }
+    }
     if (bad) {
       if (!inverse) {
         sp.flags[ss.flag_off + qc] = 1;

@@ -78,8 +78,7 @@ def worst_components(s, pts, f, J, points, polys):
     return worst
 
 
-@pytest.mark.parametrize("prec", ["dd", "ddint", "f64"])
-@pytest.mark.parametrize("apart", [12, 22, 34])
+@pytest.mark.parametrize("prec,apart", [("dd", 12), ("dd", 22), ("dd", 34), ("ddint", 12), ("ddint", 34), ("f64", 12)])
 def test_derivatives_that_are_one_coefficient(prec, apart):
     """x_6 .. x_9 occur once per polynomial, as c x with components 2^-apart of
     each other: their derivatives are c, bit for bit, at any point."""
@@ -108,3 +107,83 @@ def test_derivatives_that_are_one_coefficient(prec, apart):
         for i in range(4):
             c = s_ref.coef[int(s.poly_ptr[p + 1]) - 4 + i]
             assert np.all(J[p, 6 + i] == (c[[0, 2]] if prec == "f64" else c)), (p, i)
+
+
+def run(s, pts, prec, flags):
+    import torch
+
+    import paper_1201_0499_gb300 as pkg
+    from _util import pe_precision
+
+    ev = pkg.PolyEval(s, pe_precision(prec), max_points=pts.shape[1], flags=flags)
+    f, J = ev.eval(torch.from_numpy(np.ascontiguousarray(pts)).cuda())
+    torch.cuda.synchronize()
+    assert ev.status() == pkg.PE_OK
+    ev.close()
+    return f.cpu().numpy(), J.cpu().numpy()
+
+
+def near_axis_case(kind, apart, seed, n=7, N=4, m=60, P=11):
+    """A system and points with imaginary parts 2^-apart of the real ones, in
+    the coefficients, the points, or both; points 4 and 9 on the unit circle."""
+    s = system(seed, n, N, m, 0, 5, 3)
+    pts = synth.points(seed + 1, n, P)
+    circle = pts.copy()
+    if "near" in kind[0]:
+        s.coef[:, 2:] = np.ldexp(s.coef[:, 2:], -apart)
+    elif kind[0] == "real":
+        s.coef[:, 2:] = 0.0
+    elif kind[0] == "imaginary":
+        s.coef[:, :2] = 0.0
+    if kind[1] == "near":
+        pts[..., 2:] = np.ldexp(pts[..., 2:], -apart)
+    else:
+        pts[..., 2:] = 0.0
+    pts[:, [4, 9]] = circle[:, [4, 9]]
+    return s, pts
+
+
+@pytest.mark.parametrize("prec", ["dd", "f64"])
+@pytest.mark.parametrize("apart", [8, 16, 22])
+@pytest.mark.parametrize("wanted", ["values", "own"])  # own: the library's choice
+@pytest.mark.parametrize("kind", [("real", "near"), ("near", "near"), ("near", "real"), ("imaginary", "near"), ("any", "near")])
+def test_near_the_axes(prec, apart, kind, wanted):
+    import paper_1201_0499_gb300 as pkg
+
+    s, pts = near_axis_case(kind, apart, 1210 + apart)
+    s_in, p_in, s_ref, p_ref = inputs(s, pts, prec, 1211)
+    f, J = run(s_in, p_in, prec, pkg.PE_FROM_VALUES if wanted == "values" else 0)
+    assert worst_components(s_ref, p_ref, f, J, range(pts.shape[1]), [0, 3]) <= BOUND[prec]
+
+
+def test_near_the_axes_in_a_batch():
+    """One system of real coefficients among others; its near-real points."""
+    import torch
+
+    import paper_1201_0499_gb300 as pkg
+
+    cases = [near_axis_case(k, 16, 1230 + i, n=5 + i, P=10 + i) for i, k in
+             enumerate([("any", "near"), ("real", "near"), ("near", "real")])]
+    ev = pkg.PolyEvalMany([s for s, _ in cases], [p.shape[1] for _, p in cases], pkg.PE_DD, pkg.PE_FROM_VALUES)
+    fs, Js = ev.eval([torch.from_numpy(p).cuda() for _, p in cases])
+    torch.cuda.synchronize()
+    for (s, p), f, J in zip(cases, fs, Js):
+        assert worst_components(s, p, f.cpu().numpy(), J.cpu().numpy(), range(p.shape[1]), [1]) <= BOUND["dd"]
+    ev.close()
+
+
+@pytest.mark.parametrize("prec", ["dd", "ddint", "f64", "qd"])
+def test_real_points_of_real_systems(prec):
+    """Imaginary parts are exact zeros, the real parts as accurate as ever."""
+    import paper_1201_0499_gb300 as pkg
+
+    s, pts = near_axis_case(("real", "real"), 0, 1240)
+    pts[..., 2:] = 0.0
+    s_in, p_in, s_ref, p_ref = inputs(s, pts, prec, 1241)
+    if prec == "qd":  # no lower parts to the zeros
+        s_in.coef[:, 4:] = 0.0
+        p_in[..., 4:] = 0.0
+    f, J = evaluate(s_in, p_in, prec, pkg.PE_FROM_VALUES)
+    w = f.shape[-1] // 2
+    assert np.all(f[..., w:] == 0.0) and np.all(J[..., w:] == 0.0)
+    assert worst_components(s_ref, p_ref, f, J, [0, 10], [0]) <= (2.0**-195 if prec == "qd" else BOUND.get(prec, 2.0**-90))
