@@ -38,7 +38,7 @@ constexpr int kQdSlotsFull = 12;
 constexpr size_t kSumTableAsk = size_t{1} << 30;
 constexpr int64_t kSumPointersMax = int64_t{64} << 20;
 constexpr int kSumTiles = 3;       // log2 of the points per tile: 0, 1, 2
-constexpr int kSumCoefSkew = 40;  // and bits the components of a coefficient may be apart
+constexpr int kSumCoefSkew = 40, kSumCoefSkew64 = 26;  // bits the components of a coefficient may be apart (26: double)
 
 struct DeviceBuf {
   void *p = nullptr;
@@ -794,7 +794,7 @@ int setup_sum(polyeval *h, const Compiled &c, bool always) {
         // quad-double 230) bits less their distance, and J is rounded 8 bits
         // higher: all it was given in double; in double-double that shows near
         // the axes only (see axial).
-        if (re != 0.0 && im != 0.0 && std::abs(er - ei) > kSumCoefSkew) return PE_OK;
+        if (re != 0.0 && im != 0.0 && std::abs(er - ei) > (L == 3 ? kSumCoefSkew64 : kSumCoefSkew)) return PE_OK;
         if (re != 0.0 || im != 0.0)
           gamma = std::max(gamma, std::fabs(static_cast<double>(re > im ? er : ei)) + 1.0);
       }

@@ -156,6 +156,20 @@ def test_near_the_axes(prec, apart, kind, wanted):
     assert worst_components(s_ref, p_ref, f, J, range(pts.shape[1]), [0, 3]) <= BOUND[prec]
 
 
+@pytest.mark.parametrize("apart", [24, 31, 38])
+def test_coefficients_far_apart_in_double(apart):
+    """At real points and on the unit circle."""
+    import paper_1201_0499_gb300 as pkg
+
+    s, pts = near_axis_case(("real", "real"), 0, 1250)
+    rng = np.random.Generator(np.random.PCG64(1252))
+    s.coef[:, 0] = rng.uniform(0.5, 1.0, len(s.coef))
+    s.coef[:, 2] = np.ldexp(rng.uniform(0.5, 1.0, len(s.coef)), -apart)
+    s_in, p_in, s_ref, p_ref = inputs(s, pts, "f64", 1251)
+    f, J = run(s_in, p_in, "f64", pkg.PE_FROM_VALUES)
+    assert worst_components(s_ref, p_ref, f, J, range(pts.shape[1]), [0, 3]) <= BOUND["f64"]
+
+
 def test_near_the_axes_in_a_batch():
     """One system of real coefficients among others; its near-real points."""
     import torch
