@@ -17,7 +17,10 @@
 // exchange does not move those of earlier steps.  The reciprocals are kept for
 // the back substitution.  Points with entries that are not finite or beyond
 // 2^(+-kMaxExp) are solved by the double-double code of lu.cuh, whose
-// overflows and NaN they keep.
+// overflows and NaN they keep; so are systems all of whose entries lie near an
+// axis (components more than 2^kElApart apart) unless all are real, whose
+// smaller parts come from smaller parts alone and would take the error of the
+// larger ones (118 bits for both, 106 each there).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -35,6 +38,7 @@ namespace {
 using fx::Num;
 
 constexpr int kMaxExp = 200;
+constexpr int kElApart = 10;
 constexpr int kZeroEl = -(1 << 20);  // exponent of an exactly zero entry
 
 struct El {
@@ -80,16 +84,24 @@ __device__ __forceinline__ void component_words(double h, double l, uint32_t (&w
   e = wide::is_zero(c.m) ? kZeroEl : c.e;
 }
 
-// An entry from the evaluator's (normalised) double-doubles.  `usual` is
-// cleared for values the integer elimination is not meant for.  No FP64
+// What the entries of a system are: usual, or values that the integer
+// elimination is not meant for; some not real; some away from the axes.
+struct Kinds {
+  bool usual = true, complex = false, off_axis = false;
+};
+
+// An entry from the evaluator's (normalised) double-doubles.  No FP64
 // arithmetic: 1000 entries of 5 blocks would queue for its pipe.
-__device__ __forceinline__ El el_from(const CDD &v, bool &usual) {
+__device__ __forceinline__ El el_from(const CDD &v, Kinds &kinds) {
   auto exponent = [](double x) { return static_cast<int>(static_cast<unsigned long long>(__double_as_longlong(x)) >> 52) & 0x7ff; };
   auto zero = [](double x) { return (__double_as_longlong(x) << 1) == 0; };
-  const int top = max(exponent(v.re.h), exponent(v.im.h));
-  if (!(zero(v.re.h) && zero(v.im.h)) && (top > 1023 + kMaxExp || top < 1023 - kMaxExp)) usual = false;
+  const int xr = exponent(v.re.h), xi = exponent(v.im.h), top = max(xr, xi);
+  const bool zr = zero(v.re.h), zi = zero(v.im.h);
+  if (!(zr && zi) && (top > 1023 + kMaxExp || top < 1023 - kMaxExp)) kinds.usual = false;
+  kinds.complex = kinds.complex || !zi;
+  kinds.off_axis = kinds.off_axis || (!zr && !zi && xr - xi <= kElApart && xi - xr <= kElApart);
   El x;
-  if (!usual) {
+  if (!kinds.usual) {
     for (int k = 0; k < 4; k++) x.r[k] = x.i[k] = 0u;
     x.e = kZeroEl;
     return x;
@@ -249,12 +261,12 @@ __global__ void __launch_bounds__(256, 2) newton_int(const NewtonParams p) {
     return v;
   };
 
-  bool usual = true;
+  Kinds kinds;
   double fnorm = 0.0;
   for (int i = tid; i < n; i += T) {
     const CDD v = CDD::load(gv.bel(i));
     fnorm = nan_max(fnorm, v.abs_hi());
-    A.store(i * cols + n, el_from(v.neg(), usual));
+    A.store(i * cols + n, el_from(v.neg(), kinds));
   }
   for (int k0 = tid; k0 < n * n; k0 += 4 * T) {  // four loads in flight
     CDD v[4];
@@ -263,13 +275,15 @@ __global__ void __launch_bounds__(256, 2) newton_int(const NewtonParams p) {
       if (k0 + x * T < n * n) v[x] = CDD::load(gv.Jel((k0 + x * T) / n, (k0 + x * T) % n));
 #pragma unroll
     for (int x = 0; x < 4; x++)
-      if (k0 + x * T < n * n) A.store((k0 + x * T) / n * cols + (k0 + x * T) % n, el_from(v[x], usual));
+      if (k0 + x * T < n * n) A.store((k0 + x * T) / n * cols + (k0 + x * T) % n, el_from(v[x], kinds));
   }
   for (int i = tid; i < n; i += T) row[i] = i;
   if (tid == 0) is_singular = 0;
   fnorm = block_max(fnorm, red[0]);
   bool singular = false;
-  if (!__syncthreads_and(usual)) {
+  const bool usual = __syncthreads_and(kinds.usual);
+  const bool near_axis = !__syncthreads_or(kinds.off_axis) && __syncthreads_or(kinds.complex);
+  if (!usual || near_axis) {
     // the double-double elimination in place, by the first warp
     if (warp == 0) {
       for (int i = lane; i < n; i += 32) CDD::load(gv.bel(i)).neg().store(gv.bel(i));
