@@ -226,16 +226,20 @@ __global__ void __launch_bounds__(kWarpsPerBlockMax * 32, kSome ? 1 : 7) main_qd
 // One thread per output component (32 bytes): the sum of the chunks'
 // accumulators, rounded to a quad-double in place.  `components` covers f
 // (the first f_components) and then J.
+template <bool kSome>
 __global__ void finalize_qd(double *out_f, double *out_J, const double *scratch_f, const double *scratch_J,
                             int64_t f_components, int64_t J_components, int chunks, Only only) {
-  wait_for_previous();
-  if (only.any && *only.any == 0) return;
+  if constexpr (kSome) {
+    wait_for_previous();
+    if (*only.any == 0) return;
+  }
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   const int64_t total = f_components + J_components;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < total; i += stride) {
     const bool isf = i < f_components;
     const int64_t j = isf ? i : i - f_components;
-    if (only.any && !only.flags[j / 2 % only.P]) continue;
+    if constexpr (kSome)
+      if (!only.flags[j / 2 % only.P]) continue;
     double *p = (isf ? out_f : out_J) + j * 4;
     const double *sc = isf ? scratch_f : scratch_J;
     const int64_t cs = (isf ? f_components : J_components) * 4;  // doubles between chunk copies
@@ -287,9 +291,9 @@ cudaError_t launch_finalize_qd(double *out_f, double *out_J, const double *scrat
   int64_t blocks = (total + 255) / 256;
   if (blocks > kSms * 16) blocks = kSms * 16;
   if (only.any)
-    return launch_next(finalize_qd, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, s, out_f, out_J, scratch_f, scratch_J,
+    return launch_next(finalize_qd<true>, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, s, out_f, out_J, scratch_f, scratch_J,
                        f_components, J_components, chunks, only);
-  finalize_qd<<<static_cast<unsigned>(blocks), 256, 0, s>>>(out_f, out_J, scratch_f, scratch_J, f_components,
+  finalize_qd<false><<<static_cast<unsigned>(blocks), 256, 0, s>>>(out_f, out_J, scratch_f, scratch_J, f_components,
                                                             J_components, chunks, only);
   return cudaGetLastError();
 }
