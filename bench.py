@@ -317,6 +317,20 @@ class Workload:
             return self.ev[prec].autotune(x, f, J, stream)
         return self.pkg.polyeval_autotune(self.handle(prec), x, self.points, f, J, stream)
 
+    def from_values(self, prec):
+        """Whether the handle evaluates from the monomials' values, by the
+        kernels that one evaluation of a single monomial chunk queues: the
+        general kernels take a table, a main and, in quad-double, a rounding
+        kernel; from values come two more, and no rounding one."""
+        points = 0 if self.cfg == 4 else self.points
+        self.pkg.polyeval_set_launch(self.handle(prec), points, 1)
+        self.pkg.polyeval_timing(self.handle(prec), True)
+        self.eval(prec)
+        kernels = self.pkg.polyeval_timing_read(self.handle(prec))[2]
+        self.pkg.polyeval_timing(self.handle(prec), False)
+        self.pkg.polyeval_set_launch(self.handle(prec), points)
+        return kernels > (3 if prec == "qd" else 2)
+
     def cost_per_launch(self, prec):
         """FP64 instructions and flops of the fused FP64 kernel for one step."""
         if self.cfg == 4:
@@ -460,32 +474,54 @@ def paper_leg(pkg, torch, timer, wl, ms_dd, reps, dist, world):
     ev_paper.eval(xd, fd, Jd)
     ms = max_over_ranks(timer.run(lambda: ev_paper.eval(xd, fd, Jd), reps) / reps, dist)
     ev_paper.close()
-    return {"ms_per_step": ms, "evals_per_s": job_throughput(world, P, ms), "fused_fp64_dd_speedup": ms / ms_dd,
+    return {"ms_per_step": ms, "evals_per_s": job_throughput(world, P, ms), "dd_speedup": ms / ms_dd,
             "what": "the paper's K1 common factors / K2 Speelpenning + coefficients into zero-padded Mons / "
                     "K3 one thread per output, complex double-double (PE_PAPER_KERNELS)"}
 
 
+def general_leg(pkg, timer, wl, reps, dist, world):
+    """The same batch with the general kernels (PE_GENERAL_KERNELS), autotuned."""
+    out = {"what": "common factors and Speelpenning products: PE_DD and PE_F64 on the FP64 pipe, PE_DD_INT and "
+                   "PE_QD_INT in integer block floating point"}
+    codes = {"dd": pkg.PE_DD, "ddint": pkg.PE_DD_INT, "f64": pkg.PE_F64, "qd": pkg.PE_QD_INT}
+    for prec in PRECS:
+        x, f, J = wl.bufs[buf_fmt(prec)]
+        system = (wl.system.as_fp64() if prec == "f64" else
+                  wl.system.to_qd(QD_SEED + 1) if prec == "qd" else wl.system)
+        ev = pkg.PolyEval(system, codes[prec], max_points=wl.points, flags=pkg.PE_GENERAL_KERNELS)
+        ev.autotune(x, f, J, timer.stream)
+        ms = max_over_ranks(timer.run(lambda: ev.eval(x, f, J), reps) / reps, dist)
+        out[prec] = {"evals_per_s": job_throughput(world, wl.points, ms), "ms_per_step": ms}
+        ev.close()
+    return out
+
+
 def secondary(cfg, pkg, torch, timer, rank, world, dev, dist, reps, sm_max):
-    """One of the smaller workloads: every precision after autotuning, and on
-    the n = 32 workload the Newton step, the paper's three kernels and the
-    path tracker."""
+    """One of the smaller workloads: every precision (general kernels after
+    autotuning), and on the n = 32 workload the general kernels by themselves,
+    the Newton step, the paper's three kernels and the path tracker."""
     wl = Workload(cfg, rank, dev)
     out = {"workload": wl.text, "points_per_gpu": wl.points}
-    tuned = {}
+    tuned = {}  # the autotuner chooses launches of the general kernels
+    out["from_values"] = [prec for prec in PRECS if wl.from_values(prec)]
     for prec in PRECS:
+        if prec in out["from_values"]:
+            continue
         c, m, g = wl.autotune(prec, timer.stream)
         tuned[prec] = {"chunks": c, "shape": "one wave" if m == 1 else "persistent",
                        ("partial_tile_groups_cap" if cfg == 4 else "monomial_groups_per_warp"): g}
     torch.cuda.synchronize()
-    out["autotuned_launch"] = tuned
+    out["autotuned_launch"] = tuned or None
     ms = {}
     for prec in PRECS:
         ms[prec] = leg_ms(timer, wl, prec, 1, reps, dist)
         out[prec] = {"evals_per_s": job_throughput(world, wl.points, ms[prec]), "ms_per_step": ms[prec]}
-    out["dd"]["imad_frac_of_step"] = (wl.products() * IMAD_PER_PRODUCT["dd"] / (ms["dd"] * 1e-3)
-                                      / (SMS * IMAD_PER_SM_CLK * sm_max * 1e6))
+    if "dd" in out["from_values"]:
+        out["dd"]["imad_frac_of_step"] = (wl.products() * IMAD_PER_PRODUCT["dd"] / (ms["dd"] * 1e-3)
+                                          / (SMS * IMAD_PER_SM_CLK * sm_max * 1e6))
     out["dd_fp64_time_ratio"] = ms["dd"] / ms["f64"]
-    out["ddint_speedup_vs_fp64_dd"] = ms["dd"] / ms["ddint"]
+    if cfg == 2:
+        out["general_kernels"] = general_leg(pkg, timer, wl, reps, dist, world)
     for prec in PRECS:
         assert pkg.polyeval_status(wl.handle(prec)) == pkg.PE_OK
     # the double-double evaluation captured once in a CUDA graph and replayed
@@ -592,20 +628,25 @@ def main():
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
 
     tuned = {}
+    by_values = wl.from_values(prim)
+    if by_values:
+        launch_note = "evaluation from the monomials' values: launch by the library's rule"
     if cfg != CONFIG_INDEX and not args.no_autotune:
         # pick the launch per precision on this batch, before any timed step
+        # (of the general kernels: the autotuner's choice is theirs)
         for prec in PRECS:
+            if wl.from_values(prec):
+                continue
             c, m, g = wl.autotune(prec, stream)
             tuned[prec] = {"chunks": c, "shape": "one wave" if m == 1 else "persistent", "groups": g}
         torch.cuda.synchronize()
-        launch_note = "autotuned per precision (polyeval_autotune)"
-    elif cfg != CONFIG_INDEX:
-        launch_note = "built-in (autotuning skipped)"
-    else:
-        # 128 x 1024 (polynomial, tile) items fill many waves and one chunk of
-        # outputs (8.7 GB) exceeds the chunk scratch: the tuner's only
-        # candidate is the built-in persistent launch, so it is not run
-        launch_note = "built-in: one monomial chunk, persistent grid of 4-warp blocks (the only candidate here)"
+        if not by_values:
+            launch_note = "autotuned (polyeval_autotune)"
+    elif not by_values:
+        # at the headline workload 128 x 1024 (polynomial, tile) items fill
+        # many waves and one chunk of outputs (8.7 GB) exceeds the chunk
+        # scratch: the tuner's only candidate is the built-in persistent launch
+        launch_note = "general kernels, built-in launch"
 
     graphs = {}
 
@@ -664,10 +705,11 @@ def main():
 
     # roofline of the monomial kernels (sum_kernel, and the general kernel's
     # pass over the flags): bound by the 64-bit integer multiply-adds of the
-    # products, one product per variable of a monomial
+    # products, one product per variable of a monomial; none where the general
+    # kernels evaluate
     kern_avg_ms = kern_ms / max(launches, 1)
-    imads = wl.products() * IMAD_PER_PRODUCT[prim]
-    achieved_tops = 2 * imads / (kern_avg_ms * 1e-3) / 1e12
+    imads = wl.products() * IMAD_PER_PRODUCT[prim] if by_values else None
+    achieved_tops = 2 * imads / (kern_avg_ms * 1e-3) / 1e12 if by_values else None
     peak_tops = SMS * IMAD_PER_SM_CLK * 2 * sm_max * 1e6 / 1e12
     # what the fused FP64 kernel (forward and backward products) would execute
     # for the same evaluations, per second of this kernel: an equivalent, not
@@ -739,9 +781,9 @@ def main():
                 "what": "polyeval_eval_host: pinned host points in, pinned host f and J out, synchronous"},
         "gpu_launches": kernels,
         "roofline": {"bound": "alu", "achieved": achieved_tops, "peak": peak_tops, "unit": "TOP/s",
-                     "frac": achieved_tops / peak_tops, "traffic": None,
+                     "frac": achieved_tops / peak_tops if by_values else None, "traffic": None,
                      "traffic_basis": "no DRAM capture of this kernel",
-                     "kernel": "sum_kernel", "kernel_ms": kern_avg_ms,
+                     "kernel": "sum_kernel" if by_values else "general", "kernel_ms": kern_avg_ms,
                      "achieved_basis": f"64-bit integer multiply-adds of the products ({IMAD_PER_PRODUCT[prim]} each, "
                                        "one product per variable of a monomial and point; counted as 2 operations), "
                                        "not those of the rescaling and the sums",
@@ -753,13 +795,13 @@ def main():
                      "paper_method_frac": paper_tflops / peak_nominal if paper_tflops else None},
         "fp64_path": {"evals_per_s": job_throughput(world, P, ms64), "ms_per_step": ms64},
         "dd_fp64_time_ratio": ms_dd / ms64,
-        ("int_pipe_path" if other == "ddint" else "fp64_dd_path"): {
+        # the other double-double handles: the same kernel where both evaluate from values
+        ("PE_DD_INT" if other == "ddint" else "PE_DD") + "_handles": {
             "evals_per_s": job_throughput(world, P, legs[other]), "ms_per_step": legs[other],
-            "speedup_vs_fp64_dd": (ms_per_step / legs[other]) if other == "ddint" else (legs[other] / ms_per_step),
             "precision": "complex double-double in/out, " + DD_TEXT},
         "qd_int_path": {
             "evals_per_s": job_throughput(world, P, legs["qd"]), "ms_per_step": legs["qd"],
-            "time_vs_fp64_dd": legs["qd"] / ms_dd,
+            "time_vs_dd": legs["qd"] / ms_dd,
             "precision": "complex quad-double in/out (the same data with two random lower parts), products of "
                          "eight 29-bit integer digits, sums in integers of ten 32-bit words"},
         # FP64 flops of the fused FP64 kernel for the same evaluations, over the

@@ -19,8 +19,14 @@
  * x_i df/dx_i = sum a_i V, with products and sums of integers on the integer
  * pipes (all precisions).  Points that this does not suit (a zero or
  * non-finite coordinate, exponents near the range of a double, components of
- * one coordinate more than 2^24 apart) are evaluated by the kernels of
- * Sections 3.1-3.3 ("general kernels") in the same call.
+ * one coordinate more than 2^24 apart; in double-double every coordinate near
+ * an axis, components more than 2^4 apart, of systems whose coefficients may
+ * lie near one) are evaluated by the kernels of Sections 3.1-3.3 ("general
+ * kernels") in the same call.  A handle keeps to the general kernels alone
+ * when they are expected to be faster, when one of its coefficients has
+ * components more than 2^40 (PE_F64: 2^26) apart or lies near the range of a
+ * double, or when there is no memory for the tables; for a batch that goes for
+ * all its systems.  PE_GENERAL_KERNELS and PE_FROM_VALUES override the first.
  *
  * Conventions for every entry point:
  *   - Return value: PE_OK (0) or a negative PE_E* code; nothing aborts and no
@@ -55,7 +61,14 @@
  * over absolute values: sum |c| |x^a| for f, sum |c| a_i |x^(a - e_i)| for
  * J): <= 1e-28 for PE_DD and PE_DD_INT, <= 1e-60 for PE_QD_INT and <= 1e-13
  * for PE_F64 on the workloads this library is tested on; see the tests for
- * the exact cases.
+ * the exact cases.  The measure takes the modulus of a complex number: where a
+ * component of an output is far smaller than the other, its own relative
+ * accuracy depends on the kernels.  The general PE_DD and PE_F64 kernels
+ * compute components apart.  The evaluation from values holds a component to
+ * 2^-107 (PE_F64 2^-80, PE_QD_INT 2^-219) of its terms' moduli, and leaves
+ * near-axis points to the general kernels as told above; a point of which some
+ * coordinates lie near an axis and others do not stays, and terms in the
+ * former alone then have their smaller component to that precision.
  */
 #ifndef POLYEVAL_H
 #define POLYEVAL_H
@@ -289,7 +302,9 @@ PE_API int polyeval_set_launch(polyeval_t *h, int64_t P, int chunks, int shape, 
  * The solve is LU with partial pivoting per point (pivot of largest modulus)
  * in the handle's precision (double-double for PE_DD and PE_DD_INT, double
  * for PE_F64), 4 to 32 lanes of a warp per point; double-double solves with
- * 12 <= n <= 77 run on the integer pipes, a block per point.  PE_QD_INT handles
+ * 12 <= n <= 77 run on the integer pipes, a block per point, but for points
+ * with non-finite or huge entries and for nearly real systems (every entry of
+ * J and f near an axis, not all real).  PE_QD_INT handles
  * evaluate f and J in quad-double and solve for dx in double-double from
  * the leading two parts of each component (mixed precision, as iterative
  * refinement: each step gains about 104 bits less log2 cond(J) until x

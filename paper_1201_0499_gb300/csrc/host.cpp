@@ -38,6 +38,7 @@ constexpr int kQdSlotsFull = 12;
 constexpr size_t kSumTableAsk = size_t{1} << 30;
 constexpr int64_t kSumPointersMax = int64_t{64} << 20;
 constexpr int kSumTiles = 3;       // log2 of the points per tile: 0, 1, 2
+static_assert((1 << (kSumTiles - 1)) <= pe::kSumPointsMax, "sum_kernel keeps an exponent per point of a tile");
 constexpr int kSumCoefSkew = 40, kSumCoefSkew64 = 26;  // bits the components of a coefficient may be apart (26: double)
 
 struct DeviceBuf {
@@ -801,8 +802,9 @@ int setup_sum(polyeval *h, const Compiled &c, bool always) {
     }
     ss.axial = L == 4 ? axial_system(c, d) : 0;
     h->sum_axial = h->sum_axial || ss.axial != 0;
-    // every monomial value within 2^(+-900) of 1: no overflow, and the low
-    // parts of the results well above the smallest normal double
+    // every monomial value within 2^(+-900) of 1: no overflow, and the second
+    // parts of the results well above the smallest normal double (the fourth
+    // parts of quad-doubles may fall below it, as they do everywhere)
     if (gamma > 800.0) return PE_OK;
     ss.most_log2 = static_cast<float>((900.0 - gamma) / deg);
     int bl = 1;

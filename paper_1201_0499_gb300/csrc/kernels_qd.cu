@@ -225,7 +225,9 @@ __global__ void __launch_bounds__(kWarpsPerBlockMax * 32, kSome ? 1 : 7) main_qd
 
 // One thread per output component (32 bytes): the sum of the chunks'
 // accumulators, rounded to a quad-double in place.  `components` covers f
-// (the first f_components) and then J.
+// (the first f_components) and then J.  kSome: the flagged points only (the
+// question in the loop of the other cost it 30 of 560 us at n = 50, 8
+// monomials of 2 variables, 4096 points).
 template <bool kSome>
 __global__ void finalize_qd(double *out_f, double *out_J, const double *scratch_f, const double *scratch_J,
                             int64_t f_components, int64_t J_components, int chunks, Only only) {

@@ -31,7 +31,7 @@
 // 2^-97, 2^-89, 2^-82.5; on the unit circle 2^-104.4 and 2^-105.9.  Points on
 // the circle: (2 2^-kSumNearAxis)^n of them lie near an axis in n coordinates.)
 //
-// Layout.  One block works on one tile of 1, 2, 4 or 8 points of a system and
+// Layout.  One block works on one tile of 1, 2 or 4 points of a system and
 // a run of polynomials.  The tile's power table (digits.cuh) is copied to
 // shared memory once.  For each polynomial, chunks of monomials:
 //   A  one thread per (monomial, point) multiplies its k factors in

@@ -169,8 +169,9 @@ __device__ bool lu_solve(const V &v, const Lanes<S> g) {
     g.sync();
   }
   // back substitution, y overwrites b, by columns: x_i = y_i / U_ii (every
-  // lane, which costs the FP64 pipe no more than one), then the lanes over
-  // the rows r < i take x_i out of y_r
+  // lane, which costs the FP64 pipe no more than one; the reciprocal kept by
+  // lane i, or formed again where n > S), then the lanes over the rows r < i
+  // take x_i out of y_r
   for (int i = n - 1; i >= 0; i--) {
     const C xi = C::mul(C::load(v.bel(i)), keep ? kept.shfl(g.mask, i, S) : C::recip(C::load(v.Jel(i, i))));
     g.sync();

@@ -449,7 +449,7 @@ cudaError_t launch_newton_int(const NewtonParams &p, cudaStream_t s) {
         cudaFuncSetAttribute(newton_int, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kIntLuBytesMax));
     if (e != cudaSuccess) return e;
   }
-  // threads as the trailing updates need; the last warp does the reciprocals
+  // threads as the trailing updates need (the first warp also finds the pivots and their reciprocals)
   const int threads = p.n <= 16 ? 64 : p.n <= 40 ? 128 : 256;
   newton_int<<<static_cast<unsigned>(p.P), threads, bytes, s>>>(p);
   return cudaGetLastError();

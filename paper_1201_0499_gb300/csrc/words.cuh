@@ -1,6 +1,6 @@
 // Two's complement integers of W 32-bit words (word 0 least significant): the
 // shifts and conversions of the kernels that sum or eliminate with them
-// (kernels_sum.cu, newton.cu).
+// (kernels_sum.cu, newton_int.cu).
 #pragma once
 
 #include <cstdint>
