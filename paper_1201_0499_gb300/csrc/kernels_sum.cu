@@ -764,17 +764,12 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2
           const int row = (u << lg) + q, c = u & 1;
           uint32_t a[W];
           uint32_t m = 0u, low = 0u;  // the or of the terms' words above kw, of their words kw
-          int32_t top = -1;           // a bit that the terms of earlier chunks reach
           if constexpr (kOne) {
 #pragma unroll
             for (int i = 0; i < W; i++) a[i] = 0u;
           } else {
             load_window<L>(aq, ar, arows, row, a);
-            top = am[row];
-            if (grown > 0) {
-              sar_words<W>(a, grown);
-              top = max(top - grown, -1);
-            }
+            if (grown > 0) sar_words<W>(a, grown);
           }
           if (u >= fb) {
             constexpr int len = kSumBlock / kSumParts;
@@ -836,6 +831,7 @@ __global__ void __launch_bounds__(kSumThreadsMax, L == 8 && !kOne && !kBatch ? 2
           } else {
             store_window<L>(aq, ar, arows, row, a);
             // (exact but for bits above word kw + 1, which count as of that word)
+            int32_t top = max(am[row] - grown, -1);
             if (m | low) top = max(top, (m ? 32 * kw + 63 : 32 * kw + 31) - __clz(static_cast<int>(m ? m : low)));
             am[row] = top;
           }
