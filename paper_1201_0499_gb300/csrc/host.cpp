@@ -751,7 +751,7 @@ int setup_sum(polyeval *h, const Compiled &c, bool always) {
         if (count[v] != 1 || c.var[c.mono_ptr[t]] >> 16 != 1) continue;
         count[v] = 0;
         const_var.push_back(static_cast<int32_t>(v));
-        const_val.insert(const_val.end(), c.coef.begin() + static_cast<size_t>(t) * cd, c.coef.begin() + static_cast<size_t>(t + 1) * cd);
+        for (int i = 0; i < cd; i++) const_val.push_back(c.coef[static_cast<size_t>(t) * cd + i] + 0.0);  // no -0: a sum from 0
         bits[sp[gp].bits_off + (v >> 5)] |= 1u << (v & 31);
       }
     sp[gp].const_n = static_cast<int32_t>(const_var.size()) - sp[gp].const_off;

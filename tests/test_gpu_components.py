@@ -109,6 +109,19 @@ def test_derivatives_that_are_one_coefficient(prec, apart):
             assert np.all(J[p, 6 + i] == (c[[0, 2]] if prec == "f64" else c)), (p, i)
 
 
+@pytest.mark.parametrize("prec", ["dd", "f64"])
+def test_constant_derivatives_have_no_negative_zeros(prec):
+    """A sum that starts from 0: the zero parts of a coefficient come out as +0."""
+    import paper_1201_0499_gb300 as pkg
+
+    s = synth.from_monomials(2, [[([0], [1]), ([1], [2])]], np.array([[-0.0, -0.0, 2.0, -0.0], [1.0, 0.0, 1.0, 0.0]]))
+    pts = synth.points(1260, 2, 5)
+    s_in, p_in, _, _ = inputs(s, pts, prec, 1261)
+    for flags in (pkg.PE_FROM_VALUES, pkg.PE_GENERAL_KERNELS):
+        J = evaluate(s_in, p_in, prec, flags)[1]
+        assert np.all(J[0, 0, :, J.shape[-1] // 2] == 2.0) and not np.any(np.signbit(J[0, 0]))
+
+
 def run(s, pts, prec, flags):
     import torch
 
