@@ -66,9 +66,12 @@
  * accuracy depends on the kernels.  The general PE_DD and PE_F64 kernels
  * compute components apart.  The evaluation from values holds a component to
  * 2^-107 (PE_F64 2^-80, PE_QD_INT 2^-219) of its terms' moduli, and leaves
- * near-axis points to the general kernels as told above; a point of which some
- * coordinates lie near an axis and others do not stays, and terms in the
- * former alone then have their smaller component to that precision.
+ * near-axis points to the general kernels as told above.  That rule goes by
+ * whole points and by sums over the coefficients' parts: where only some
+ * coordinates lie near an axis, where a polynomial is dominated by terms whose
+ * coefficient and coordinates all do, or where real points mix real and
+ * imaginary terms of very different size, the smaller component has that
+ * precision and no more.  PE_GENERAL_KERNELS is for callers who need it.
  */
 #ifndef POLYEVAL_H
 #define POLYEVAL_H
